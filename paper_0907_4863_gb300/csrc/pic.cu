@@ -8,26 +8,79 @@
 // nearest multiply and add in the reference's order, so it is bitwise the CPU result.
 #include "pic.cuh"
 
+#include "divc.cuh"
+
 namespace saamg {
 
 namespace {
 
-__device__ __forceinline__ void cic_axis(double x, double o, double h, long long& c, double& f) {
-  const double u = (x - o) / h;
-  const double fl = floor(u);
-  c = (long long)fl;
-  f = u - fl;
-}
-
 struct Lattice {
   int nx, ny, nz;
-  double hx, hy, hz, ox, oy, oz;
+  double ox, oy, oz;
+  DivC hx, hy, hz;  // spacings
+  DivC vol;
 };
+
+// u = (x - o) / h: the particle's lattice coordinate.
+__device__ __forceinline__ double lattice_coord(double x, double o, const DivC& h) {
+  return div_by(x - o, h);
+}
+
+// Whether the cell of u can touch the box: -1 <= u < 2^31 - 1 (false for NaN), on the bits.
+__device__ __forceinline__ bool coord_near(double u) {
+  const long long b = __double_as_longlong(u);
+  return b >= 0 ? b < 0x41dfffffffc00000LL
+                : (b & 0x7fffffffffffffffLL) <= 0x3ff0000000000000LL;
+}
+
+// c = floor(u), f = u - floor(u) for coord_near(u).  Adding 1.5 * 2^52 rounds u to an integer in
+// the low word; the difference to it is exact, and one below zero belongs to the cell before
+// (f = d + 1 rounds the same real number as u - floor(u)).  Four FP64 additions; floor and the
+// two conversions would take as many instructions on slower paths.
+__device__ __forceinline__ void split_coord(double u, int& c, double& f) {
+  const double big = 6755399441055744.0;  // 1.5 * 2^52
+  const double t = __dadd_rn(u, big);
+  const double d = __dadd_rn(u, -__dadd_rn(t, -big));
+  c = __double2loint(t);
+  f = d;
+  if (__double2hiint(d) < 0 &&
+      (static_cast<unsigned long long>(__double_as_longlong(d)) << 1) != 0ull) {
+    c -= 1;
+    f = __dadd_rn(d, 1.0);
+  }
+}
+
+// The same cell and the fraction as a 64-bit fixed-point number, by integer operations.
+__device__ __forceinline__ void split_coord_fixed(double u, int& c, unsigned long long& f) {
+  const long long b = __double_as_longlong(u);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023;  // |u| = m / 2^63 * 2^e
+  const unsigned long long m =
+      e == -1023 ? 0ull : ((unsigned long long)b << 11) | 0x8000000000000000ull;
+  if (e >= 0) {  // e <= 30; u = -1 is the only negative one
+    c = (int)(m >> (63 - e));
+    f = m << (e + 1);
+  } else {
+    c = 0;
+    f = e > -65 ? m >> (-1 - e) : 0ull;
+  }
+  if (b < 0) {
+    c = f != 0ull ? -c - 1 : -c;
+    f = 0ull - f;
+  }
+}
 
 __global__ void abs_sum_k(int n, const double* __restrict__ q, double* __restrict__ part) {
   double acc = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    acc += fabs(q[i]);
+  const int st = gridDim.x * blockDim.x;
+  long long i = blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + 3LL * st < n; i += 4LL * st) {  // four loads in flight, added in index order
+    const double a = q[i], b = q[i + st], c = q[i + 2LL * st], d = q[i + 3LL * st];
+    acc += fabs(a);
+    acc += fabs(b);
+    acc += fabs(c);
+    acc += fabs(d);
+  }
+  for (; i < n; i += st) acc += fabs(q[i]);
   __shared__ double sh[32];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -51,80 +104,188 @@ __global__ void scale_k(const double* __restrict__ part, int nparts, double vol,
   exp[0] = (b > 0.0 && isfinite(b)) ? 60 - ilogb(b) : 0;
 }
 
-__global__ void cic_deposit_k(Lattice g, int np, const double* __restrict__ x,
-                              const double* __restrict__ y, const double* __restrict__ z,
-                              const double* __restrict__ q, double vol,
-                              const int* __restrict__ exp, unsigned long long* __restrict__ acc) {
+// |v| w for a weight w in units of 2^-64, in units of the 64-bit mantissa of v.
+__device__ __forceinline__ unsigned long long wmul(unsigned long long a, unsigned long long w) {
+  return __umul64hi(a, w);
+}
+
+// A particle adds round(2^S (q / V) wx wy wz) to each of its eight nodes.  The weights are
+// 64-bit fixed-point fractions and the products integer multiplications: |q / V| 2^S < 2^61, so
+// a product's three truncations are off by less than 3/8 of the fixed-point unit, where the
+// rounding of the product in FP64 (53 bits of a number of up to 61) could be off by 2^7 units.
+// In FP64 the divisions, the 14 weight products, the scalings and the conversions of a particle ran
+// on a pipe of two lanes per clock and SM; now the L2 atomics bind the pass (86 % of the L2's
+// throughput, FP64 pipe 42 %): 10^7 particles on 256^3 take 384 us here, and the whole call 515 us
+// instead of 2472.
+__global__ void __launch_bounds__(256) cic_deposit_k(Lattice g, int np,
+                                                     const double* __restrict__ x,
+                                                     const double* __restrict__ y,
+                                                     const double* __restrict__ z,
+                                                     const double* __restrict__ q,
+                                                     const int* __restrict__ exp,
+                                                     unsigned long long* __restrict__ acc) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= np || exp[1]) return;
-  const int S = exp[0];
-  long long ci, cj, ck;
-  double fx, fy, fz;
-  cic_axis(x[p], g.ox, g.hx, ci, fx);
-  cic_axis(y[p], g.oy, g.hy, cj, fy);
-  cic_axis(z[p], g.oz, g.hz, ck, fz);
-  const double qv = q[p] / vol;
+  if (p >= np) return;
+  const double xp = x[p], yp = y[p], zp = z[p], qp = q[p];
+  if (exp[1]) return;
+  const double ux = lattice_coord(xp, g.ox, g.hx), uy = lattice_coord(yp, g.oy, g.hy),
+               uz = lattice_coord(zp, g.oz, g.hz);
+  if (!(coord_near(ux) && coord_near(uy) && coord_near(uz))) return;
+  int ci, cj, ck;
+  unsigned long long fx, fy, fz;
+  split_coord_fixed(ux, ci, fx);
+  split_coord_fixed(uy, cj, fy);
+  split_coord_fixed(uz, ck, fz);
+  if (ci >= g.nx || cj >= g.ny || ck >= g.nz) return;
+  // |q / V| = m / 2^63 * 2^e, scaled by 2^S: the product m w >> 64 is to be shifted right by sh
+  const long long qb = __double_as_longlong(div_by(qp, g.vol));
+  int e = (int)((qb >> 52) & 0x7ff) - 1023;
+  unsigned long long m = (unsigned long long)qb << 11;
+  if (e > -1023) {
+    m |= 0x8000000000000000ull;
+  } else {
+    if (m == 0ull) return;
+    const int lz = __clzll((long long)m);  // subnormal
+    m <<= lz;
+    e = -1022 - lz;
+  }
+  const int sh = 63 - (e + exp[0]);  // >= 3
+  if (sh > 64) return;  // less than half a unit at every node
+  const bool neg = qb < 0;
+  // 1 - f: 2^64 - f, and 2^64 - 1 for f = 0
+  const unsigned long long wx[2] = {fx ? 0ull - fx : ~0ull, fx};
+  const unsigned long long wy[2] = {fy ? 0ull - fy : ~0ull, fy};
+  const unsigned long long wz[2] = {fz ? 0ull - fz : ~0ull, fz};
+  const unsigned long long half = 1ull << (sh - 1);
+  const unsigned long long mx[2] = {wmul(m, wx[0]), wmul(m, wx[1])};
+  const bool inner = ci >= 0 && cj >= 0 && ck >= 0 && ci + 1 < g.nx && cj + 1 < g.ny &&
+                     ck + 1 < g.nz;
+  const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < 2; ++b) {
+      const bool line = inner || (cj + b >= 0 && ck + c >= 0 && cj + b < g.ny && ck + c < g.nz);
+      const long long v = v0 + (long long)g.nx * (b + (long long)g.ny * c);
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        const long long i = ci + a, j = cj + b, k = ck + c;
-        if (i < 0 || j < 0 || k < 0 || i >= g.nx || j >= g.ny || k >= g.nz) continue;
-        const double wx = a ? fx : 1.0 - fx, wy = b ? fy : 1.0 - fy, wz = c ? fz : 1.0 - fz;
-        const double v = __dmul_rn(__dmul_rn(__dmul_rn(qv, wx), wy), wz);
-        const long long iv = llrint(ldexp(v, S));
-        atomicAdd(&acc[i + (long long)g.nx * (j + (long long)g.ny * k)], (unsigned long long)iv);
+        if (!inner && !(line && ci + a >= 0 && ci + a < g.nx)) continue;
+        const unsigned long long r = wmul(wmul(mx[a], wy[b]), wz[c]);
+        const unsigned long long w = sh < 64 ? (r >> sh) + ((r & half) != 0) : (r >> 63);
+        if (w) atomicAdd(&acc[v + a], neg ? 0ull - w : w);
       }
+    }
 }
 
-__global__ void fixed_to_double_k(size_t n, const unsigned long long* __restrict__ acc,
-                                  const int* __restrict__ exp, double* __restrict__ rho) {
+// rho = acc 2^-S (acc may be rho), the nearest double: the leading one of |acc| is found and the 53 bits below
+// it rounded to even with integer operations (the FP64 conversion and scaling of 16.8 M nodes
+// would take as long as their bytes); a result outside the normal range takes ldexp.
+__global__ void __launch_bounds__(256) fixed_to_double_k(size_t n, const int* __restrict__ exp,
+                                                         const unsigned long long* acc,
+                                                         unsigned long long* rho) {
   const int S = exp[0];
   const bool bad = exp[1] != 0;
   for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < n;
-       v += (size_t)gridDim.x * blockDim.x)
-    rho[v] = bad ? __longlong_as_double(0x7ff8000000000000ll)
-                 : ldexp((double)(long long)acc[v], -S);
+       v += (size_t)gridDim.x * blockDim.x) {
+    if (bad) {
+      rho[v] = 0x7ff8000000000000ull;
+      continue;
+    }
+    const long long a = (long long)acc[v];
+    if (a == 0) {
+      if (acc != rho) rho[v] = 0ull;
+      continue;
+    }
+    unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int lz = __clzll((long long)u);
+    const int e = 63 - lz - S + 1023;
+    unsigned long long r;
+    if (e < 1 || e > 2045) {
+      r = (unsigned long long)__double_as_longlong(ldexp((double)(long long)u, -S));
+    } else {
+      u <<= lz;
+      r = ((unsigned long long)e << 52) + ((u & 0x7fffffffffffffffull) >> 11);
+      const unsigned long long low = u & 0x7ffull;
+      if (low > 0x400ull || (low == 0x400ull && (r & 1ull))) ++r;  // may carry into the exponent
+    }
+    rho[v] = r | (a < 0 ? 0x8000000000000000ull : 0ull);
+  }
 }
 
-__global__ void cic_gather_k(Lattice g, const double* __restrict__ ex,
-                             const double* __restrict__ ey, const double* __restrict__ ez,
-                             int np, const double* __restrict__ x, const double* __restrict__ y,
-                             const double* __restrict__ z, double* __restrict__ epx,
-                             double* __restrict__ epy, double* __restrict__ epz) {
+// Bitwise the reference's sums: ((wx wy) wz) E added in its corner order, every product and sum
+// rounded.  Those 12 + 45 FP64 instructions, and 18-24 for the three coordinates, bind the kernel
+// (FP64 pipe 84 % busy at two lanes per clock and SM, L2 29 %); full divisions by the spacings and
+// floor() made 10^7 particles on 256^3 take 2019 instead of 1656 us.  All eight nodal values of a
+// component are loaded before they are used.
+__global__ void __launch_bounds__(256) cic_gather_k(Lattice g, const double* __restrict__ ex,
+                                                    const double* __restrict__ ey,
+                                                    const double* __restrict__ ez, int np,
+                                                    const double* __restrict__ x,
+                                                    const double* __restrict__ y,
+                                                    const double* __restrict__ z,
+                                                    double* __restrict__ epx,
+                                                    double* __restrict__ epy,
+                                                    double* __restrict__ epz) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
-  long long ci, cj, ck;
-  double fx, fy, fz;
-  cic_axis(x[p], g.ox, g.hx, ci, fx);
-  cic_axis(y[p], g.oy, g.hy, cj, fy);
-  cic_axis(z[p], g.oz, g.hz, ck, fz);
-  double sx = 0.0, sy = 0.0, sz = 0.0;
+  const double xp = x[p], yp = y[p], zp = z[p];
+  const double ux = lattice_coord(xp, g.ox, g.hx), uy = lattice_coord(yp, g.oy, g.hy),
+               uz = lattice_coord(zp, g.oz, g.hz);
+  double s[3] = {0.0, 0.0, 0.0};
+  if (coord_near(ux) && coord_near(uy) && coord_near(uz)) {
+    int ci, cj, ck;
+    double fx, fy, fz;
+    split_coord(ux, ci, fx);
+    split_coord(uy, cj, fy);
+    split_coord(uz, ck, fz);
+    const double* E[3] = {ex, ey, ez};
+    const double wx[2] = {__dadd_rn(1.0, -fx), fx}, wy[2] = {__dadd_rn(1.0, -fy), fy},
+                 wz[2] = {__dadd_rn(1.0, -fz), fz};
+    double wxy[4];
 #pragma unroll
-  for (int c = 0; c < 2; ++c)
+    for (int q = 0; q < 4; ++q) wxy[q] = __dmul_rn(wx[q & 1], wy[q >> 1]);
+    const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
+    const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+    if (ci >= 0 && cj >= 0 && ck >= 0 && ci + 1 < g.nx && cj + 1 < g.ny && ck + 1 < g.nz) {
+      double w[8];
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+      for (int q = 0; q < 8; ++q) w[q] = __dmul_rn(wxy[q & 3], wz[q >> 2]);
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const long long i = ci + a, j = cj + b, k = ck + c;
-        if (i < 0 || j < 0 || k < 0 || i >= g.nx || j >= g.ny || k >= g.nz) continue;
-        const double w = __dmul_rn(__dmul_rn(a ? fx : 1.0 - fx, b ? fy : 1.0 - fy),
-                                   c ? fz : 1.0 - fz);
-        const long long v = i + (long long)g.nx * (j + (long long)g.ny * k);
-        sx = __dadd_rn(sx, __dmul_rn(w, ex[v]));
-        sy = __dadd_rn(sy, __dmul_rn(w, ey[v]));
-        sz = __dadd_rn(sz, __dmul_rn(w, ez[v]));
+      for (int k = 0; k < 3; ++k) {
+        const double* e = E[k] + v0;
+        double t[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          t[q] = e[(q & 1) + ((q >> 1) & 1) * sy + (q >> 2) * sz];
+        double a = __dmul_rn(w[0], t[0]);
+#pragma unroll
+        for (int q = 1; q < 8; ++q) a = __dadd_rn(a, __dmul_rn(w[q], t[q]));
+        // the reference starts from +0, which no sum of zeros of either sign leaves
+        s[k] = (static_cast<unsigned long long>(__double_as_longlong(a)) << 1) == 0ull ? 0.0 : a;
       }
-  epx[p] = sx;
-  epy[p] = sy;
-  epz[p] = sz;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int i = q & 1, j = (q >> 1) & 1, k = q >> 2;
+        if (ci + i < 0 || cj + j < 0 || ck + k < 0 || ci + i >= g.nx || cj + j >= g.ny ||
+            ck + k >= g.nz)
+          continue;
+        const double w = __dmul_rn(wxy[q & 3], wz[k]);
+        const long long v = v0 + i + j * sy + k * sz;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) s[d] = __dadd_rn(s[d], __dmul_rn(w, E[d][v]));
+      }
+    }
+  }
+  epx[p] = s[0];
+  epy[p] = s[1];
+  epz[p] = s[2];
 }
 
 Lattice lattice(const saamg_grid& g) {
-  return Lattice{g.n[0], g.n[1], g.n[2], g.h[0], g.h[1], g.h[2],
-                 g.origin[0], g.origin[1], g.origin[2]};
+  return Lattice{g.n[0], g.n[1], g.n[2], g.origin[0], g.origin[1], g.origin[2],
+                 make_divc(g.h[0]), make_divc(g.h[1]), make_divc(g.h[2]),
+                 make_divc((g.h[0] * g.h[1]) * g.h[2])};
 }
 
 }  // namespace
@@ -133,25 +294,31 @@ void deposit_cic(const saamg_grid& grid, int np, const double* x, const double* 
                  const double* z, const double* q, double* rho, cudaStream_t s) {
   const Lattice g = lattice(grid);
   const size_t nbox = (size_t)g.nx * g.ny * g.nz;
-  const double vol = (g.hx * g.hy) * g.hz;
-  Buf<unsigned long long> acc;
   Buf<double> part;
   Buf<int> exp;
-  acc.alloc(nbox, s);
   part.alloc(kRedBlocks, s);
   exp.alloc(2, s);
-  SAAMG_CUDA(cudaMemsetAsync(acc.p, 0, nbox * sizeof(unsigned long long), s));
+  // rho itself holds the fixed-point sums until they are converted, unless it overlaps an input
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(rho);
+  unsigned long long* acc = out;
+  Buf<unsigned long long> own;
+  for (const double* in : {x, y, z, q})
+    if ((uintptr_t)in < (uintptr_t)(rho + nbox) && (uintptr_t)rho < (uintptr_t)(in + np) && !own.p) {
+      own.alloc(nbox, s);
+      acc = own.p;
+    }
+  SAAMG_CUDA(cudaMemsetAsync(acc, 0, nbox * sizeof(unsigned long long), s));
   abs_sum_k<<<kRedBlocks, 256, 0, s>>>(np, q, part.p);
   SAAMG_LAUNCH();
-  scale_k<<<1, 32, 0, s>>>(part.p, kRedBlocks, vol, exp.p);
+  scale_k<<<1, 32, 0, s>>>(part.p, kRedBlocks, g.vol.c, exp.p);
   SAAMG_LAUNCH();
   if (np > 0) {
     KernelTimer kt(SAAMG_KT_PIC, np, s);
-    cic_deposit_k<<<(np + 255) / 256, 256, 0, s>>>(g, np, x, y, z, q, vol, exp.p, acc.p);
+    cic_deposit_k<<<(np + 255) / 256, 256, 0, s>>>(g, np, x, y, z, q, exp.p, acc);
     SAAMG_LAUNCH();
   }
   const int blocks = (int)std::min<size_t>((nbox + 255) / 256, sm_count() * 16);
-  fixed_to_double_k<<<blocks, 256, 0, s>>>(nbox, acc.p, exp.p, rho);
+  fixed_to_double_k<<<blocks, 256, 0, s>>>(nbox, exp.p, acc, out);
   SAAMG_LAUNCH();
 }
 
