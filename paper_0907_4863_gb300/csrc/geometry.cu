@@ -6,6 +6,7 @@
 // below and never with fused multiply-adds.
 #include <climits>
 
+#include "divc.cuh"
 #include "operator.cuh"
 
 namespace saamg {
@@ -834,115 +835,187 @@ StencilDev<float> OperatorData::view<float>() const {
 
 namespace {
 
-// Derivative of the quadratic through the node value p0 and its neighbours along one axis,
-// at distances h (unknown neighbour) or s h (wall point, value 0); written with the same
-// operations, in the same order, as the CPU reference (this unit is compiled without FMA
-// contraction, so the results agree bit for bit).
-__device__ double axis_derivative(double h, bool in_m, bool in_p, double pm, double p0,
-                                  double pp, double t, double s) {
-  if (in_m && in_p) return (pp - pm) / (2.0 * h);
-  if (in_m) return (-(s * s) * pm + (s * s - 1.0) * p0) / (h * s * (1.0 + s));
-  if (in_p) return ((t * t) * pp - (t * t - 1.0) * p0) / (h * t * (1.0 + t));
-  return p0 * (s - t) / (h * s * t);
-}
+// The divisors that every node of a launch shares.
+struct GradDiv {
+  DivC h[3], two_h[3], dist;
+};
 
 __device__ __forceinline__ bool line_has(const LineInfo& l, int i) { return i >= l.lo && i <= l.hi; }
 
-// E = -grad phi at unknown (i, line L) of chunk offset row `q` in the box.  Neighbours inside
-// Omega_h use their phi; an outside neighbour is replaced by the wall point at the boundary
-// fraction with phi = 0; on a Robin end plane the z-derivative is the Robin condition's.
-__device__ __forceinline__ void gradient_node(const GeomParams& g,
-                                              const LineInfo* __restrict__ lines, int L,
-                                              const LineInfo& me, int i,
-                                              const double* __restrict__ phi,
-                                              double* __restrict__ ex, double* __restrict__ ey,
-                                              double* __restrict__ ez) {
-  const int j = L % g.ny, k = L / g.ny;
-  const size_t sy = (size_t)g.nx, sz = (size_t)g.nx * g.ny;
-  const size_t q = (size_t)i + sy * (size_t)j + sz * (size_t)k;
-  const double p0 = phi[q];
-  const double dist = 0.5 * ((double)(g.nz - 1) * g.h[2]);
-  const size_t stride[3] = {1, sy, sz};
-  double* E[3] = {ex, ey, ez};
-  for (int ax = 0; ax < 3; ++ax) {
-    double d;
-    if (ax == 2 && g.zbc == SAAMG_Z_ROBIN && (k == 0 || k == g.nz - 1)) {
-      d = (k == 0 ? 1.0 : -1.0) * p0 / dist;
-    } else {
-      // membership from the line records (the classification node_inside produced)
-      bool in_m, in_p;
-      if (ax == 0) {
-        in_m = i - 1 >= me.lo;
-        in_p = i + 1 <= me.hi;
-      } else {
-        const int lstride = ax == 1 ? 1 : g.ny;
-        const bool has_m = ax == 1 ? j > 0 : k > 0;
-        const bool has_p = ax == 1 ? j < g.ny - 1 : k < g.nz - 1;
-        in_m = has_m && line_has(lines[L - lstride], i);
-        in_p = has_p && line_has(lines[L + lstride], i);
-      }
-      const double pm = in_m ? phi[q - stride[ax]] : 0.0;
-      const double pp = in_p ? phi[q + stride[ax]] : 0.0;
-      const double t = in_m ? 1.0 : boundary_fraction(g, i, j, k, 2 * ax);
-      const double s = in_p ? 1.0 : boundary_fraction(g, i, j, k, 2 * ax + 1);
-      d = axis_derivative(g.h[ax], in_m, in_p, pm, p0, pp, t, s);
-    }
-    E[ax][q] = -d;
+// Derivative at p0 of the quadratic through a node and its neighbours along axis ax, of which at
+// least one is outside: that neighbour is the wall point (value 0) at the boundary fraction.  The
+// operations, and their order, are the CPU reference's (this unit is compiled without FMA
+// contraction, so the results agree bit for bit):
+//   plus side outside:  (-(s s) pm + (s s - 1) p0) / ((h s) (1 + s))
+//   minus side outside: ((t t) pp - (t t - 1) p0) / ((h t) (1 + t)), the first with -1 before it
+//   both:               p0 (s - t) / ((h s) t)
+// pn: the value on the side that is inside.
+__device__ __forceinline__ double wall_derivative(const GeomParams& g, const GradDiv& dv, int ax,
+                                                  bool in_m, bool in_p, int i, int j, int k,
+                                                  double pn, double p0) {
+  if (!in_m && !in_p) {
+    const double t = boundary_fraction(g, i, j, k, 2 * ax);
+    const double s = boundary_fraction(g, i, j, k, 2 * ax + 1);
+    return p0 * (s - t) / (g.h[ax] * s * t);
   }
+  double f;
+  if (ax < 2) {  // boundary_fraction of the outside side, one division for either side
+    const double x = node_coord(g.o[0], i, g.h[0]), y = node_coord(g.o[1], j, g.h[1]);
+    const double sg = taper_sigma(g, node_coord(g.o[2], k, g.h[2]));
+    const double pos = ax == 0 ? x : y, pc = ax == 0 ? g.cx : g.cy;
+    const double pa = ax == 0 ? g.a : g.b, oa = ax == 0 ? g.b : g.a;
+    const double v = (ax == 0 ? y - g.cy : x - g.cx) / (oa * sg);
+    const double w = (pa * sg) * sqrt(1.0 - v * v);
+    f = clamp_frac(div_by(in_m ? (pc + w) - pos : pos - (pc - w), dv.h[ax]));
+  } else {
+    f = boundary_fraction(g, i, j, k, in_m ? 5 : 4);
+  }
+  const double ff = f * f;
+  const double num = -ff * pn + (ff - 1.0) * p0;
+  return (in_m ? num : -num) / (g.h[ax] * f * (1.0 + f));
 }
 
-// Warp per chunk, lane per unknown: the nodes whose six neighbours are all unknowns (and not
-// on a Robin plane) take central differences here; the others -- a few per cent, where the
-// boundary fractions, their divisions and square roots would hold a whole warp on the FP64
-// pipe for one lane -- are listed for gradient_boundary_k, one per lane of a full warp.
-__global__ void field_gradient_k(GeomParams g, const LineInfo* __restrict__ lines,
-                                 const int2* __restrict__ chunks, int nchunks,
-                                 const double* __restrict__ phi, double* __restrict__ ex,
-                                 double* __restrict__ ey, double* __restrict__ ez,
-                                 int2* __restrict__ list, int* __restrict__ nlist) {
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+constexpr int kGradLines = 16;  // lattice lines per block, two per warp
+
+// E = -grad phi at the unknowns, 0 elsewhere, in one pass that writes every box node once.
+// Neighbours inside Omega_h use their phi, an outside one is replaced by the wall point, and on a
+// Robin end plane the z-derivative is the Robin condition's.
+// The inside run of a line meets those of its four neighbour lines in one interval [ilo, ihi],
+// so a line splits into zeros, central differences and the few nodes beside the wall.  A warp
+// takes its lines in x order and leaves the nodes beside the wall to the end of the block, which
+// gathers those of its 16 lines (four a line on a 256^3 pipe), one per thread: their central axes
+// are done at once, and each axis that meets the wall -- a boundary fraction with two divisions
+// and a square root, and the division of the derivative -- is an item of a shared list, so that
+// full warps run them.
+// Bound by FP64 issue (two lanes per clock and SM): a difference and a division per axis and
+// node, three instructions a division, one where the spacing is a power of two.  256^3: 210 us
+// instead of 676 (three memsets, general divisions, and a second kernel over a list of the nodes
+// beside the wall, appended to with one global atomic per warp); of that, 90 us are the FP64 work of
+// the central differences and 79 us the bytes.
+__global__ void __launch_bounds__(256) field_gradient_k(GeomParams g, GradDiv dv, int nlines,
+                                                        const LineInfo* __restrict__ lines,
+                                                        const double* __restrict__ phi,
+                                                        double* __restrict__ ex,
+                                                        double* __restrict__ ey,
+                                                        double* __restrict__ ez) {
+  __shared__ int s_off[kGradLines + 1];  // nodes beside the wall, then their prefix sums
+  __shared__ int s_lo[kGradLines], s_ilo[kGradLines], s_ihi[kGradLines];
+  __shared__ int2 s_item[3 * 256];  // (line of the block | axis << 8 | in_m << 10 | in_p << 11, i)
+  __shared__ int s_items;
   const int lane = threadIdx.x & 31;
-  if (c >= nchunks) return;  // warp-uniform
-  const int2 ch = chunks[c];
-  const int L = ch.x;
-  const LineInfo me = lines[L];
-  const int i = me.lo + ch.y + lane;
-  const bool active = i <= me.hi;
-  bool inner = false;
-  if (active) {
+  const size_t sy = (size_t)g.nx, sz = (size_t)g.nx * g.ny;
+  const int L0 = blockIdx.x * kGradLines;
+  if (threadIdx.x == 0) s_items = 0;
+  for (int w = threadIdx.x >> 5; w < kGradLines; w += blockDim.x >> 5) {
+    const int L = L0 + w;
+    if (L >= nlines) {
+      if (lane == 0) s_off[w + 1] = 0;
+      continue;
+    }
     const int j = L % g.ny, k = L / g.ny;
     const bool robin = g.zbc == SAAMG_Z_ROBIN && (k == 0 || k == g.nz - 1);
-    inner = !robin && i - 1 >= me.lo && i + 1 <= me.hi && j > 0 && j < g.ny - 1 && k > 0 &&
-            k < g.nz - 1 && line_has(lines[L - 1], i) && line_has(lines[L + 1], i) &&
-            line_has(lines[L - g.ny], i) && line_has(lines[L + g.ny], i);
-    if (inner) {
-      const size_t sy = (size_t)g.nx, sz = (size_t)g.nx * g.ny;
-      const size_t q = (size_t)i + sy * (size_t)j + sz * (size_t)k;
-      // the central differences of axis_derivative, same operations
-      ex[q] = -((phi[q + 1] - phi[q - 1]) / (2.0 * g.h[0]));
-      ey[q] = -((phi[q + sy] - phi[q - sy]) / (2.0 * g.h[1]));
-      ez[q] = -((phi[q + sz] - phi[q - sz]) / (2.0 * g.h[2]));
+    const LineInfo me = lines[L];
+    int ilo = me.lo + 1, ihi = me.hi - 1;
+    auto meet = [&](bool has, int Ln) {
+      if (!has) {
+        ihi = ilo - 1;
+        return;
+      }
+      const LineInfo l = lines[Ln];
+      ilo = max(ilo, l.lo);
+      ihi = min(ihi, l.hi);
+    };
+    if (me.hi >= me.lo) {
+      meet(j > 0, L - 1);
+      meet(j < g.ny - 1, L + 1);
+      if (!robin) {
+        meet(k > 0, L - g.ny);
+        meet(k < g.nz - 1, L + g.ny);
+      }
+    }
+    if (ihi < ilo) {
+      ilo = me.lo;
+      ihi = me.lo - 1;
+    }
+    if (lane == 0) {
+      s_off[w + 1] = (me.hi - me.lo + 1) - (ihi - ilo + 1);
+      s_lo[w] = me.lo;
+      s_ilo[w] = ilo;
+      s_ihi[w] = ihi;
+    }
+    const size_t q0 = sy * (size_t)L;
+    const int zhi = me.hi >= me.lo ? me.hi + 1 : 0;  // zeros: [0, lo) and [zhi, nx)
+    for (int i = lane; i < me.lo; i += 32) ex[q0 + i] = ey[q0 + i] = ez[q0 + i] = 0.0;
+    for (int i = zhi + lane; i < g.nx; i += 32) ex[q0 + i] = ey[q0 + i] = ez[q0 + i] = 0.0;
+#pragma unroll 2
+    for (int i = ilo + lane; i <= ihi; i += 32) {
+      const size_t q = q0 + i;
+      const double xm = phi[q - 1], xp = phi[q + 1], ym = phi[q - sy], yp = phi[q + sy];
+      if (!robin) {
+        const double zm = phi[q - sz], zp = phi[q + sz];
+        ez[q] = -div_by(zp - zm, dv.two_h[2]);
+      } else {
+        const double p0 = phi[q];
+        ez[q] = -div_by(k == 0 ? p0 : -p0, dv.dist);
+      }
+      ex[q] = -div_by(xp - xm, dv.two_h[0]);
+      ey[q] = -div_by(yp - ym, dv.two_h[1]);
     }
   }
-  const unsigned need = __ballot_sync(0xffffffffu, active && !inner);
-  if (!need) return;
-  int base = 0;
-  if (lane == 0) base = atomicAdd(nlist, __popc(need));
-  base = __shfl_sync(0xffffffffu, base, 0);
-  if (active && !inner) list[base + __popc(need & ((1u << lane) - 1u))] = make_int2(c, lane);
-}
-
-__global__ void gradient_boundary_k(GeomParams g, const LineInfo* __restrict__ lines,
-                                    const int2* __restrict__ chunks,
-                                    const int2* __restrict__ list, const int* __restrict__ nlist,
-                                    const double* __restrict__ phi, double* __restrict__ ex,
-                                    double* __restrict__ ey, double* __restrict__ ez) {
-  const int cnt = *nlist;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += gridDim.x * blockDim.x) {
-    const int2 it = list[e];
-    const int2 ch = chunks[it.x];
-    const LineInfo me = lines[ch.x];
-    gradient_node(g, lines, ch.x, me, me.lo + ch.y + it.y, phi, ex, ey, ez);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_off[0] = 0;
+    for (int w = 0; w < kGradLines; ++w) s_off[w + 1] += s_off[w];
+  }
+  __syncthreads();
+  double* const E[3] = {ex, ey, ez};
+  const size_t stride[3] = {1, sy, sz};
+  for (int e0 = 0; e0 < s_off[kGradLines]; e0 += blockDim.x) {
+    const int e = e0 + threadIdx.x;
+    if (e < s_off[kGradLines]) {
+      int w = 0;
+      while (e >= s_off[w + 1]) ++w;
+      const int r = e - s_off[w], left = s_ilo[w] - s_lo[w];
+      const int i = r < left ? s_lo[w] + r : s_ihi[w] + 1 + (r - left);
+      const int L = L0 + w, j = L % g.ny, k = L / g.ny;
+      const LineInfo me = lines[L];
+      const size_t q = sy * (size_t)L + i;
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax) {
+        if (ax == 2 && g.zbc == SAAMG_Z_ROBIN && (k == 0 || k == g.nz - 1)) {
+          const double p0 = phi[q];
+          ez[q] = -div_by(k == 0 ? p0 : -p0, dv.dist);
+          continue;
+        }
+        bool in_m, in_p;  // from the line records (the classification node_inside produced)
+        if (ax == 0) {
+          in_m = i - 1 >= me.lo;
+          in_p = i + 1 <= me.hi;
+        } else {
+          const int ls = ax == 1 ? 1 : g.ny;
+          in_m = (ax == 1 ? j > 0 : k > 0) && line_has(lines[L - ls], i);
+          in_p = (ax == 1 ? j < g.ny - 1 : k < g.nz - 1) && line_has(lines[L + ls], i);
+        }
+        if (in_m && in_p)
+          E[ax][q] = -div_by(phi[q + stride[ax]] - phi[q - stride[ax]], dv.two_h[ax]);
+        else
+          s_item[atomicAdd(&s_items, 1)] =
+              make_int2(w | (ax << 8) | ((int)in_m << 10) | ((int)in_p << 11), i);
+      }
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < s_items; t += blockDim.x) {
+      const int2 it = s_item[t];
+      const int L = L0 + (it.x & 0xff), ax = (it.x >> 8) & 3, i = it.y;
+      const bool in_m = (it.x >> 10) & 1, in_p = (it.x >> 11) & 1;
+      const size_t st = ax == 0 ? 1 : (ax == 1 ? sy : sz), q = sy * (size_t)L + i;
+      const double pn = in_m ? phi[q - st] : (in_p ? phi[q + st] : 0.0);
+      double* out = ax == 0 ? ex : (ax == 1 ? ey : ez);
+      out[q] = -wall_derivative(g, dv, ax, in_m, in_p, i, L % g.ny, L / g.ny, pn, phi[q]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_items = 0;
+    __syncthreads();
   }
 }
 
@@ -950,22 +1023,15 @@ __global__ void gradient_boundary_k(GeomParams g, const LineInfo* __restrict__ l
 
 void field_gradient(const OperatorData& op, const double* phi, double* ex, double* ey,
                     double* ez, cudaStream_t s) {
-  const size_t nbox = (size_t)op.g.nx * op.g.ny * op.g.nz;
-  SAAMG_CUDA(cudaMemsetAsync(ex, 0, nbox * sizeof(double), s));
-  SAAMG_CUDA(cudaMemsetAsync(ey, 0, nbox * sizeof(double), s));
-  SAAMG_CUDA(cudaMemsetAsync(ez, 0, nbox * sizeof(double), s));
-  if (op.n == 0) return;
-  Buf<int2> list;
-  Buf<int> count;
-  list.alloc(op.n, s);
-  count.alloc(1, s);
-  fill_int(count.p, 0, 1, s);
-  field_gradient_k<<<warp_blocks(op.nchunks), 256, 0, s>>>(op.g, op.lines.p, op.chunks.p,
-                                                            op.nchunks, phi, ex, ey, ez, list.p,
-                                                            count.p);
-  SAAMG_LAUNCH();
-  gradient_boundary_k<<<sm_count() * 8, 256, 0, s>>>(op.g, op.lines.p, op.chunks.p, list.p, count.p,
-                                              phi, ex, ey, ez);
+  if (op.nlines == 0) return;
+  GradDiv dv;
+  for (int a = 0; a < 3; ++a) {
+    dv.h[a] = make_divc(op.g.h[a]);
+    dv.two_h[a] = make_divc(2.0 * op.g.h[a]);
+  }
+  dv.dist = make_divc(0.5 * ((double)(op.g.nz - 1) * op.g.h[2]));
+  field_gradient_k<<<(op.nlines + kGradLines - 1) / kGradLines, 256, 0, s>>>(
+      op.g, dv, op.nlines, op.lines.p, phi, ex, ey, ez);
   SAAMG_LAUNCH();
 }
 
