@@ -8,6 +8,10 @@
 #include "coarse.cuh"
 #include "rows.cuh"
 
+#include <cooperative_groups.h>
+
+#include <utility>
+
 namespace saamg {
 
 namespace {
@@ -19,400 +23,324 @@ __global__ void densify_k(int n, const int* __restrict__ rowptr, const int* __re
   for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) a[(size_t)col[p] * n + i] = val[p];
 }
 
-// --- explicit inverse by Gauss-Jordan elimination ------------------------------------
-// Partial pivoting as in the LU: at step k the pivot is the row i >= k of largest |a_ik|
-// (lowest row on ties); rows k and p are exchanged and column k is eliminated from every
-// other row, which leaves (P A)^-1 in place; the columns are unscrambled at the end.
-// One launch per step: each block owns a range of columns, so all writes of a step stay in
-// the writer's own columns.  Column k is read from a copy (made in the previous step by the
-// owner of that column, together with its pivot row), so no block reads a column that
-// another block is writing.
+// --- explicit inverse by blocked Gauss-Jordan elimination ------------------------------
+// Step k picks the pivot among the rows not yet pivoted (largest |a_ik|, lowest row on ties; rows
+// are never exchanged), scales that row p by 1 / a_pk to r, and takes a_ik r off every other row;
+// column k becomes 1 / a_pk in row p and -a_ik / a_pk elsewhere.  After n steps with pivot rows
+// p_k the inverse is inv(k, p_j) = a(p_k, j).
+// B steps make a panel.  gj_panel_k factors the panel's B columns on one cluster of 16 blocks, each
+// with a range of rows in its shared memory, and leaves the multipliers c_s(i) = a_ik of its steps
+// (B x n); gj_update_k applies the B steps to the whole matrix: per column the B values r_s by a
+// forward substitution over the pivot rows, then x_i - sum_s c_s(i) r_s on every row, an FP64
+// contraction of depth B that runs on all SMs from registers.  The update reads one copy of the
+// matrix and writes the other, so a tile never reads a pivot row that another tile has overwritten.
+// The panel of the next steps needs only its own columns of the updated matrix: gj_panel_k applies
+// the pending panel to them itself and runs beside the update.  It is launched first and lets the
+// update start once its blocks are resident (programmatic dependent launch); their shared-memory
+// requests keep the two off the same SM, where the update's warps would queue before every FP64
+// instruction of the panel's serial chain (n = 1250: 70 instead of 52 us a panel).
+constexpr int kGjB = 16;           // steps of a panel
+constexpr int kGjCluster = 16;     // blocks of the panel kernel (an opt-in size)
+constexpr int kGjThreads = 256;    // panel kernel: two of the panel's columns per warp
+constexpr int kGjMaxRows = 16384 / kGjCluster;  // rows per panel block at the largest n
+constexpr int kGjUpdThreads = 512;
+constexpr int kGjUpdCols = 32;     // most columns of an update tile, two per warp
+// dynamic shared memory: a panel block's rows at the largest n, and enough on either side that a
+// panel block and an update block do not fit one SM (228 KB)
+constexpr size_t kGjRowBytes = kGjB * sizeof(double) + sizeof(int);
+constexpr size_t kGjPanelSmem = 192u << 10, kGjUpdSmem = 36u << 10;
+static_assert(kGjMaxRows * kGjRowBytes <= kGjPanelSmem, "the panel's rows fit a block");
+static_assert(kGjThreads / 32 * 2 == kGjB && kGjUpdThreads / 32 * 2 == kGjUpdCols && kGjB == 16,
+              "a half-warp per column in the forward substitutions");
 
-// Block argmax of |col[i]| over i in [lo, n), lowest index on ties.
-__device__ void block_argmax(const double* __restrict__ col, int lo, int n, double* sv, int* si,
-                             double& best_out, int& idx_out) {
-  double best = -1.0;
-  int bi = n;
-  for (int i = lo + threadIdx.x; i < n; i += blockDim.x) {
-    const double v = fabs(col[i]);
-    if (v > best) {
-      best = v;
-      bi = i;
-    }
-  }
-  sv[threadIdx.x] = best;
-  si[threadIdx.x] = bi;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      const double v = sv[threadIdx.x + w];
-      const int i = si[threadIdx.x + w];
-      if (v > sv[threadIdx.x] || (v == sv[threadIdx.x] && i < si[threadIdx.x])) {
-        sv[threadIdx.x] = v;
-        si[threadIdx.x] = i;
-      }
-    }
-    __syncthreads();
-  }
-  best_out = sv[0];
-  idx_out = si[0];
+// What a panel leaves for its update beside the multipliers: the pivot rows, their pivots'
+// reciprocals and l[t][s] = c_s(p_t) / pivot_s for s < t.
+struct GjPanel {
+  double ip[kGjB];
+  double l[kGjB][kGjB];
+  int row[kGjB];
+};
+
+// Pivot keys order like |v| as integers, so the search runs on the integer units instead of the
+// FP64 pipe: 0 for no row, 1 for a NaN (it loses against every number), 2 + the bits of |v|.
+__device__ __forceinline__ unsigned long long pivot_key(double v) {
+  const unsigned long long b =
+      (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return b > 0x7ff0000000000000ull ? 1ull : b + 2ull;
 }
 
-constexpr int kGjThreads = 256;
-constexpr int kGjMaxCols = 64;  // columns per block
-
-// step 0: pivot of column 0 and its copy
-__global__ void __launch_bounds__(kGjThreads) gj_first_k(int n, const double* __restrict__ a,
-                                                         double* __restrict__ colk,
-                                                         int* __restrict__ pivrow,
-                                                         int* __restrict__ err) {
-  __shared__ double sv[kGjThreads];
-  __shared__ int si[kGjThreads];
-  double best;
-  int p;
-  block_argmax(a, 0, n, sv, si, best, p);
-  if (threadIdx.x == 0) {
-    // a zero or NaN column: flagged, and the pivot index stays a valid row
-    if (!(best > 0.0)) {
-      atomicOr(err, 1);
-      p = 0;
-    }
-    pivrow[0] = p;
-  }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) colk[i] = a[i];
+// (key, index) maximum over a warp, lowest index on ties, by three integer warp reductions (a
+// butterfly of 64-bit shuffles takes five times as long); every lane holds the result
+__device__ __forceinline__ void gj_warp_argmax(unsigned long long& key, int& idx) {
+  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  idx = (int)__reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)idx : 0x7fffffffu);
+  key = ((unsigned long long)mh << 32) | ml;
 }
 
-__global__ void __launch_bounds__(kGjThreads) gj_step_k(int n, int k, int cpb,
-                                                        double* __restrict__ a,
-                                                        const double* __restrict__ colk,
-                                                        double* __restrict__ colk_next,
-                                                        int* __restrict__ pivrow,
-                                                        int* __restrict__ err) {
-  __shared__ double rk[kGjMaxCols], rp[kGjMaxCols];
-  __shared__ double sv[kGjThreads / 32];
+// r_t of one column in lane t of a half-warp, from the column's value x in pivot row t; the steps
+// s <= s0 and s >= bw do not apply.  A step is one shuffle and one FP64 instruction (a warp's
+// FP64 instruction holds its quarter of the SM for 64 clocks: a thread per column would take 136).
+__device__ __forceinline__ double gj_forward(double x, int t, const GjPanel& pn, int s0, int bw) {
+  if (t <= s0 || t >= bw) x = 0.0;
+#pragma unroll
+  for (int s = 0; s < kGjB - 1; ++s) {
+    const double xs = __shfl_sync(0xffffffffu, x, s, kGjB);
+    if (t > s && t < bw && t > s0) x = fma(-pn.l[t][s], xs, x);
+  }
+  return t > s0 && t < bw ? x * pn.ip[t] : 0.0;
+}
+
+// Factors the panel of columns k0 .. k0 + bw - 1 after applying the pending panel (pend = 0: none)
+// to them.  A step's chain -- the next column's update and pivot search, the exchange of the
+// blocks' candidates through distributed shared memory, one division -- is what bounds the kernel:
+// the candidate's own row is brought up to date by one instruction per panel column, and the rest
+// of the panel is updated while the cluster barrier is on its way.
+__global__ void __launch_bounds__(kGjThreads)
+    gj_panel_k(int n, int k0, int rpb, const double* __restrict__ a, int pend,
+               const GjPanel* __restrict__ ppn, const double* __restrict__ pc,
+               GjPanel* __restrict__ opn, double* __restrict__ oc, const int* __restrict__ pstep,
+               int* __restrict__ step, int* __restrict__ prow, int* __restrict__ err) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the update beside this panel
+  constexpr int B = kGjB;
+  struct Cand {
+    double v[B];
+    unsigned long long key;
+    int row;
+  };
+  extern __shared__ double pan[];  // B columns of the block's rpb rows
+  __shared__ Cand cand[2][kGjCluster];
+  __shared__ unsigned long long sv[kGjThreads / 32];
   __shared__ int si[kGjThreads / 32];
-  const int p = pivrow[k];
-  const double piv = colk[p];  // a_kk after the exchange
-  const double ip = 1.0 / piv;
-  const int c0 = blockIdx.x * cpb, c1 = min(n, c0 + cpb);
-  for (int t = threadIdx.x; t < c1 - c0; t += blockDim.x) {
-    const size_t o = (size_t)(c0 + t) * n;
-    rk[t] = a[o + k];
-    rp[t] = a[o + p];
-  }
-  __syncthreads();
-  // the owner of column k + 1 updates it first, copies it for the next step and finds its
-  // pivot on the way (largest |a_i,k+1| over i > k, lowest row on ties)
-  const int kn = k + 1;
-  const bool owner = kn < n && kn >= c0 && kn < c1;
-  double best = -1.0;
-  int bi = n;
-  for (int tt = 0; tt < c1 - c0; ++tt) {
-    const int t = owner ? (tt == 0 ? kn - c0 : (tt <= kn - c0 ? tt - 1 : tt)) : tt;
-    const int j = c0 + t;
-    const double r = rp[t] * ip;  // the new row k (row p before the exchange)
-    double* col = a + (size_t)j * n;
-    const bool next = j == kn;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double ci = i == k ? colk[p] : (i == p ? colk[k] : colk[i]);  // column k, exchanged
-      double v;
-      if (j == k) v = i == k ? ip : -ci * ip;
-      else if (i == k) v = r;
-      else v = (i == p ? rk[t] : col[i]) - ci * r;
-      col[i] = v;
-      if (next) {
-        colk_next[i] = v;
-        const double av = fabs(v);
-        if (i > k && av > best) {  // ascending i per thread: the first maximum is kept
-          best = av;
-          bi = i;
-        }
-      }
-    }
-  }
-  if (owner) {
-    // block argmax of (best, bi), lowest index on ties
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sv[threadIdx.x >> 5] = best;
-      si[threadIdx.x >> 5] = bi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double bb = sv[0];
-      int ii = si[0];
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-        if (sv[w] > bb || (sv[w] == bb && si[w] < ii)) {
-          bb = sv[w];
-          ii = si[w];
-        }
-      if (!(bb > 0.0)) {  // a zero or NaN column: flagged, the pivot stays a valid row
-        atomicOr(err, 1);
-        ii = kn;
-      }
-      pivrow[kn] = ii;
-    }
-  }
-}
-
-// Panel form with the panel factored in every block (no exchange between blocks inside a
-// launch).  A launch takes b pivot steps k0 .. k0 + b - 1.  Each block loads those b columns
-// and runs the b steps on them in shared memory: pivot search, exchanged column c_s, and the
-// step on the panel columns not yet pivoted.  It then moves its own columns through the b
-// steps (a panel column from its own step on, where it becomes 1 / pivot in row k and
-// -c_s(i) / pivot elsewhere).  For one column only the rows k_s and p_s follow special
-// formulas; one warp walks those rows (one per lane) through the steps, which gives
-// r_s = x_{p_s} / pivot_s of every step, and every other row takes x <- x - c_s(i) r_s.
-// Every element sees the operations of the one-launch-per-step form in the same order.  A
-// launch reads src and writes every column to dst, so no block overwrites a column that
-// another block of the same launch may still be loading.  The own columns are copied to
-// shared memory asynchronously while the panel is factored.
-constexpr int kGjRpThreads = 256;
-
-// Pivot keys: the bits of |v| as an integer, which order like |v| for every non-NaN v; a NaN
-// gets -1 and is never chosen, as with a floating-point comparison.  The search then runs
-// on the integer units instead of the FP64 pipe.
-__device__ __forceinline__ long long pivot_key(double v) {
-  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
-  return b > 0x7ff0000000000000LL ? -1LL : b;
-}
-
-// (key, index) maximum over a warp, lowest index on ties; every lane holds the result
-__device__ __forceinline__ void rp_warp_argmax(long long& best, int& bi) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob > best || (ob == best && oi < bi)) {
-      best = ob;
-      bi = oi;
-    }
-  }
-}
-
-// the same over the block; after the barrier inside, every lane of warp 0 holds the result
-__device__ __forceinline__ void rp_block_argmax(long long& best, int& bi, long long* sv, int* si) {
-  rp_warp_argmax(best, bi);
-  if ((threadIdx.x & 31) == 0) {
-    sv[threadIdx.x >> 5] = best;
-    si[threadIdx.x >> 5] = bi;
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const int nw = blockDim.x >> 5;
-    best = threadIdx.x < nw ? sv[threadIdx.x] : -1LL;
-    bi = threadIdx.x < nw ? si[threadIdx.x] : 0x7fffffff;
-    rp_warp_argmax(best, bi);
-  }
-}
-
-template <int B, int NT, bool STAGE>
-__global__ void __launch_bounds__(NT) gj_rp_k(int n, int k0, int cpb,
-                                                        const double* __restrict__ src,
-                                                        double* __restrict__ dst,
-                                                        int* __restrict__ pivrow,
-                                                        int* __restrict__ err) {
-  extern __shared__ double rp_smem[];
-  double* pan = rp_smem;                      // B columns of n
-  double* cs = rp_smem + (size_t)B * n;       // c_s of every step, B x n
-  // the block's own columns: a shared copy, or (too large for it) src itself
-  const double* own;
-  __shared__ long long sv[NT / 32];
-  __shared__ int si[NT / 32];
-  __shared__ int sp[B];
-  __shared__ double sip[B], s_xk[B], s_r[B];
-  __shared__ double s_ck, s_cp;
-  __shared__ int srow[2 * B];
-  __shared__ int nspec;
-  __shared__ double rr[kGjMaxCols][B];        // r_s of each own column
-  __shared__ double fin[kGjMaxCols][2 * B];  // final values of its special rows
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  __shared__ double s_r[2][B];
+  __shared__ GjPanel pn;       // the pending panel, then this one
+  __shared__ double rr[B][B];  // pending r_s of each panel column j: rr[s][j]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int me = (int)cluster.block_rank();
   const int bw = min(B, n - k0);
-  const int c0 = blockIdx.x * cpb, c1 = min(n, c0 + cpb);
-  const int ncols = max(0, c1 - c0), nown = ncols * n;
-  if constexpr (STAGE) {
-    double* own_s = rp_smem + (size_t)2 * B * n;
-    for (int e = tid; e < nown; e += nt) {
-      const unsigned d = (unsigned)__cvta_generic_to_shared(own_s + e);
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d),
-                   "l"(src + (size_t)c0 * n + e)
-                   : "memory");
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    own = own_s;
-  } else {
-    own = src + (size_t)c0 * n;
-  }
-  for (int e = tid; e < bw * n; e += nt) pan[e] = src[(size_t)k0 * n + e];
-  __syncthreads();
-  // pivot search of the first panel column (rows k0 .. n - 1; ascending i per thread keeps
-  // the first maximum)
-  long long best = -1;
-  int bi = n;
-  for (int i = k0 + tid; i < n; i += nt) {
-    const long long v = pivot_key(pan[i]);
-    if (v > best) {
-      best = v;
-      bi = i;
-    }
-  }
-  for (int s = 0; s < bw; ++s) {
-    const int k = k0 + s;
-    rp_block_argmax(best, bi, sv, si);
-    if (tid < 32) {
-      if (best <= 0) {  // a zero or NaN column: flagged, the pivot stays a valid row
-        if (blockIdx.x == 0 && tid == 0) atomicOr(err, 1);
-        bi = k;
-      }
-      const double* col = pan + (size_t)s * n;
-      const double ip = 1.0 / col[bi];
-      if (tid == 0) {
-        sp[s] = bi;
-        sip[s] = ip;
-        s_ck = col[k];
-        s_cp = col[bi];
-      }
-      if (tid < bw) {
-        s_xk[tid] = pan[(size_t)tid * n + k];
-        s_r[tid] = pan[(size_t)tid * n + bi] * ip;  // the new row k (row p before the exchange)
-      }
-    }
+  const int i0 = me * rpb, rows = max(0, min(rpb, n - i0));
+  // threads by (row, column group): G groups of rp threads
+  int rp = 32;
+  while (rp < rows && rp < kGjThreads) rp <<= 1;
+  const int G = kGjThreads / rp, gi = tid & (rp - 1), gg = tid / rp;
+  // the pivot step of every own row so far sits behind the panel
+  int* own = reinterpret_cast<int*>(pan + (size_t)B * rpb);
+  for (int i = tid; i < rows; i += kGjThreads) own[i] = pstep[i0 + i];
+  if (pend > 0) {
+    const double* src = reinterpret_cast<const double*>(ppn);
+    double* dst = reinterpret_cast<double*>(&pn);
+    for (int e = tid; e < (int)(sizeof(GjPanel) / 8); e += kGjThreads) dst[e] = src[e];
     __syncthreads();
-    const int p = sp[s];
-    const double ip = sip[s], ck = s_ck, cpv = s_cp;
-    double* c = cs + (size_t)s * n;
-    // c_s (column k with rows k and p exchanged), the step on the panel columns still to be
-    // pivoted and the pivot search of the next one (rows > k), row by row
-    best = -1;
-    bi = n;
-    for (int i = tid; i < n; i += nt) {
-      const double ci = i == k ? cpv : (i == p ? ck : pan[(size_t)s * n + i]);
-      c[i] = ci;
+    const int j = 2 * warp + (lane >> 4), t = lane & 15;
+    const double x = j < bw && t < pend ? a[(size_t)(k0 + j) * n + pn.row[t]] : 0.0;
+    rr[t][j] = gj_forward(x, t, pn, -1, pend);
+  }
+  __syncthreads();
+  for (int i = gi; i < rows; i += rp) {
+    const int kp = own[i] - (k0 - pend);  // its step in the pending panel, if any
+    double c[B];
+    if (pend > 0) {
 #pragma unroll
-      for (int j = 0; j < B; ++j) {
-        if (j >= bw) break;
-        if (j <= s) continue;  // pivoted panel columns are finished by their owner
-        const double v =
-            i == k ? s_r[j] : (i == p ? s_xk[j] : pan[(size_t)j * n + i]) - ci * s_r[j];
-        pan[(size_t)j * n + i] = v;
-        if (j == s + 1 && i > k) {
-          const long long av = pivot_key(v);
-          if (av > best) {
-            best = av;
-            bi = i;
-          }
+      for (int s = 0; s < B; ++s) c[s] = s < pend ? pc[(size_t)s * n + i0 + i] : 0.0;
+    }
+    for (int j = gg; j < bw; j += G) {
+      double x = a[(size_t)(k0 + j) * n + i0 + i];
+      if (pend > 0) {
+        if (kp >= 0) x = rr[kp][j];
+#pragma unroll
+        for (int s = 0; s < B; ++s) x = fma(-c[s], rr[s][j], x);
+      }
+      pan[(size_t)j * rpb + i] = x;
+    }
+  }
+  cluster.sync();  // every block runs before the first one writes into another's shared memory
+  int p = -1;         // pivot row of the current step
+  double myip = 0.0;  // warp 0, lane s: 1 / pivot of step s
+  for (int s = -1; s < bw - 1; ++s) {
+    // step s (none for -1) on column s + 1, and the pivot search there
+    const int jn = s + 1;
+    const double* r = s_r[s & 1];
+    unsigned long long best = 0;
+    int bi = n;
+    for (int i = tid; i < rows; i += kGjThreads) {
+      double v = pan[(size_t)jn * rpb + i];
+      if (s >= 0) {
+        const bool isp = i0 + i == p;
+        if (isp) own[i] = k0 + s;
+        v = isp ? r[jn] : fma(-pan[(size_t)s * rpb + i], r[jn], v);
+        pan[(size_t)jn * rpb + i] = v;
+      }
+      if (own[i] < 0) {
+        const unsigned long long key = pivot_key(v);
+        if (key > best) {
+          best = key;
+          bi = i0 + i;
         }
       }
     }
-  }
-  // the special rows: k0 .. k0 + bw - 1 and the pivot rows, each once
-  if (tid == 0) {
-    int m = 0;
-    for (int s = 0; s < bw; ++s) srow[m++] = k0 + s;
-    for (int s = 0; s < bw; ++s) {
-      bool seen = false;
-      for (int u = 0; u < m; ++u) seen |= srow[u] == sp[s];
-      if (!seen) srow[m++] = sp[s];
+    gj_warp_argmax(best, bi);
+    if (lane == 0) {
+      sv[warp] = best;
+      si[warp] = bi;
     }
-    nspec = m;
-    if (blockIdx.x == 0)
-      for (int s = 0; s < bw; ++s) pivrow[k0 + s] = sp[s];
-  }
-  if constexpr (STAGE) asm volatile("cp.async.wait_all;\n" ::: "memory");
-  __syncthreads();
-  const int m = nspec;
-  // one warp per own column walks its special rows (one per lane) through the b steps
-  for (int t = warp; t < ncols; t += nw) {
-    const int j = c0 + t;
-    // a panel column starts after its own step s0: the inverse's column, 1 / pivot in row
-    // k_s0 and -c_s0(i) / pivot elsewhere
-    const int s0 = j >= k0 && j < k0 + bw ? j - k0 : -1;
-    const int row = lane < m ? srow[lane] : -1;
-    double x = 0.0;
-    if (lane < m) {
-      if (s0 < 0) x = own[(size_t)t * n + row];
-      else x = row == k0 + s0 ? sip[s0] : -cs[(size_t)s0 * n + row] * sip[s0];
-    }
-    for (int s = s0 + 1; s < bw; ++s) {
-      const int k = k0 + s, p = sp[s];
-      const int uk = __ffs(__ballot_sync(0xffffffffu, row == k)) - 1;
-      const int up = __ffs(__ballot_sync(0xffffffffu, row == p)) - 1;
-      const double r = __shfl_sync(0xffffffffu, x, up) * sip[s];  // the new row k
-      const double xk = __shfl_sync(0xffffffffu, x, uk);
-      if (lane == 0) rr[t][s] = r;
-      if (lane < m) {
-        const double ci = cs[(size_t)s * n + row];
-        x = row == k ? r : (row == p ? xk : x) - ci * r;
+    __syncthreads();
+    if (warp == 0) {
+      // the block's candidate with its row of the panel (multipliers up to s, the values after
+      // step s beyond) goes to every block of the cluster, a half-warp a block
+      best = lane < kGjThreads / 32 ? sv[lane] : 0ull;
+      bi = lane < kGjThreads / 32 ? si[lane] : n;
+      gj_warp_argmax(best, bi);
+      const int j = lane & 15;
+      double v = 0.0;
+      if (best > 0ull && j < bw) {
+        v = pan[(size_t)j * rpb + (bi - i0)];
+        if (s >= 0 && j > jn) v = fma(-pan[(size_t)s * rpb + (bi - i0)], r[j], v);
+      }
+#pragma unroll
+      for (int q = 0; q < kGjCluster; q += 2)
+        cluster.map_shared_rank(&cand[jn & 1][me], q + (lane >> 4))->v[j] = v;
+      if (lane < kGjCluster) {
+        Cand* to = cluster.map_shared_rank(&cand[jn & 1][me], lane);
+        to->key = best;
+        to->row = bi;
       }
     }
-    if (lane < m) fin[t][lane] = x;
+    __syncthreads();  // the candidate's row has been read
+    auto token = cluster.barrier_arrive();
+    if (s >= 0) {
+      for (int i = gi; i < rows; i += rp) {
+        const bool isp = i0 + i == p;
+        const double c = -pan[(size_t)s * rpb + i];
+        for (int j = s + 2 + gg; j < bw; j += G) {
+          const double v = pan[(size_t)j * rpb + i];
+          pan[(size_t)j * rpb + i] = isp ? r[j] : fma(c, r[j], v);
+        }
+      }
+    }
+    cluster.barrier_wait(std::move(token));
+    const Cand* cd = cand[jn & 1];
+    // rows ascend with the blocks: the lowest block wins a tie
+    unsigned long long key = lane < kGjCluster ? cd[lane].key : 0ull;
+    int w = lane;
+    gj_warp_argmax(key, w);
+    p = cd[w].row;
+    if (warp == 0) {
+      const double ip = 1.0 / cd[w].v[jn];
+      const double v = lane < B ? cd[w].v[lane] : 0.0;
+      if (lane < B) s_r[jn & 1][lane] = v * ip;
+      if (lane == jn) myip = ip;
+      if (lane < jn) pn.l[jn][lane] = v * myip;
+      if (lane == 0) {
+        pn.ip[jn] = ip;
+        pn.row[jn] = p;
+        // a zero or NaN column: flagged, and the pivot stays a valid row
+        if (me == 0 && key <= 2ull) atomicOr(err, 1);
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < rows; i += kGjThreads) {
+    if (i0 + i == p) own[i] = k0 + bw - 1;
+    // multipliers: a pivot row of this panel starts from its r_s, so its steps up to s are 0
+    const int ks = own[i] - k0;
+    for (int t = 0; t < bw; ++t)
+      oc[(size_t)t * n + i0 + i] = ks >= t ? 0.0 : pan[(size_t)t * rpb + i];
+    step[i0 + i] = own[i];
+  }
+  if (me == 0) {
+    double* dst = reinterpret_cast<double*>(opn);
+    const double* src = reinterpret_cast<const double*>(&pn);
+    for (int e = tid; e < (int)(sizeof(GjPanel) / 8); e += kGjThreads) dst[e] = src[e];
+    if (tid < bw) prow[k0 + tid] = pn.row[tid];
+  }
+}
+
+// dst = src after the steps of the panel at k0: a tile of cpb columns and rpt rows per block.
+__global__ void __launch_bounds__(kGjUpdThreads) gj_update_k(int n, int k0, int cpb, int rpt,
+                                                             const GjPanel* __restrict__ gpn,
+                                                             const double* __restrict__ cc,
+                                                             const int* __restrict__ step,
+                                                             const double* __restrict__ src,
+                                                             double* __restrict__ dst) {
+  constexpr int B = kGjB;
+  __shared__ GjPanel pn;
+  __shared__ double rr[kGjUpdCols][B];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int bw = min(B, n - k0);
+  const int c0 = blockIdx.x * cpb, nc = min(cpb, n - c0);
+  const int r0 = blockIdx.y * rpt, r1 = min(n, r0 + rpt);
+  {
+    const double* g = reinterpret_cast<const double*>(gpn);
+    double* d = reinterpret_cast<double*>(&pn);
+    for (int e = tid; e < (int)(sizeof(GjPanel) / 8); e += kGjUpdThreads) d[e] = g[e];
   }
   __syncthreads();
-  // every row of the own columns: x <- x - c_s(i) r_s over the steps s > s0 (the special
-  // rows are rewritten below)
-  {
-    int t = tid / max(n, 1), i = tid - t * n;
-    for (int e = tid; e < nown; e += nt) {
-      const int j = c0 + t;
-      const int s0 = j >= k0 && j < k0 + bw ? j - k0 : -1;
-      double x;
-      if (s0 < 0) x = own[e];
-      else x = i == k0 + s0 ? sip[s0] : -cs[(size_t)s0 * n + i] * sip[s0];
+  if (2 * (tid >> 5) < nc) {
+    // a panel column s0 starts after its own step: 1 / pivot in its pivot row, -c_s0(i) / pivot
+    // elsewhere
+    const int u = 2 * (tid >> 5) + (lane >> 4), t = lane & 15;
+    const int j = c0 + u, s0 = j >= k0 && j < k0 + bw ? j - k0 : -1;
+    double x = 0.0;
+    if (u < nc && t < bw && t > s0)
+      x = s0 < 0 ? src[(size_t)j * n + pn.row[t]] : -pn.l[t][s0];
+    rr[u][t] = gj_forward(x, t, pn, s0, bw);
+  }
+  __syncthreads();
+  for (int i = r0 + tid; i < r1; i += kGjUpdThreads) {
+    const int ks = step[i] - k0;  // >= 0: a pivot row of this panel
+    double c[B];
+#pragma unroll
+    for (int s = 0; s < B; ++s) c[s] = s < bw ? cc[(size_t)s * n + i] : 0.0;
+    auto start = [&](int t) {
+      const int j = c0 + t, s0 = j >= k0 && j < k0 + bw ? j - k0 : -1;
+      if (ks > s0) return rr[t][ks];
+      if (s0 < 0) return src[(size_t)j * n + i];
+      return ks == s0 ? pn.ip[s0] : -cc[(size_t)s0 * n + i] * pn.ip[s0];
+    };
+    int t = 0;
+    for (; t + 8 <= nc; t += 8) {
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = start(t + u);
 #pragma unroll
       for (int s = 0; s < B; ++s)
-        if (s > s0 && s < bw) x = x - cs[(size_t)s * n + i] * rr[t][s];
-      dst[(size_t)c0 * n + e] = x;
-      i += nt;
-      while (i >= n) {
-        i -= n;
-        ++t;
-      }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = fma(-c[s], rr[t + u][s], x[u]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) dst[(size_t)(c0 + t + u) * n + i] = x[u];
+    }
+    for (; t < nc; ++t) {
+      double x = start(t);
+#pragma unroll
+      for (int s = 0; s < B; ++s) x = fma(-c[s], rr[t][s], x);
+      dst[(size_t)(c0 + t) * n + i] = x;
     }
   }
-  __syncthreads();
-  for (int e = tid; e < ncols * m; e += nt) {
-    const int t = e / m, u = e - t * m;
-    dst[(size_t)(c0 + t) * n + srow[u]] = fin[t][u];
-  }
+  // the grid ends after the panel beside it, so that the next launch follows both
+  if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait();
 }
 
-// inverse(:, j) = work(:, q_j), q: the exchanges undone in reverse order (one thread)
-__global__ void gj_perm_k(int n, const int* __restrict__ pivrow, int* __restrict__ q) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int j = 0; j < n; ++j) q[j] = j;
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = pivrow[k];
-    const int t = q[k];
-    q[k] = q[p];
-    q[p] = t;
-  }
-}
-
-// inverse(i, j) = work(i, q_j), stored by rows: a 32 x 32 tile read along the work's columns
-// and written along the inverse's rows through shared memory (q = NULL: a plain transpose)
+// inverse(k, p_j) = w(p_k, j), stored by rows: a 32 x 32 tile read along the work's columns and
+// written along the inverse's rows through shared memory (step, prow NULL: a plain transpose)
 __global__ void __launch_bounds__(256) gj_gather_k(int n, const double* __restrict__ w,
-                                                   const int* __restrict__ q,
+                                                   const int* __restrict__ step,
+                                                   const int* __restrict__ prow,
                                                    double* __restrict__ inv) {
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int jj = ty; jj < 32; jj += 8) {
     const int j = j0 + jj, i = i0 + tx;
-    if (j < n && i < n) tile[jj][tx] = w[(size_t)(q ? q[j] : j) * n + i];
+    if (j < n && i < n) tile[jj][tx] = w[(size_t)j * n + i];
   }
   __syncthreads();
   for (int ii = ty; ii < 32; ii += 8) {
     const int i = i0 + ii, j = j0 + tx;
-    if (i < n && j < n) inv[(size_t)i * n + j] = tile[tx][ii];
+    if (i < n && j < n)
+      inv[(size_t)(step ? step[i] : i) * n + (prow ? prow[j] : j)] = tile[tx][ii];
   }
 }
 
@@ -597,66 +525,81 @@ void coarse_gs_setup(const DevCsr& A, const double* invd, const unsigned* ids, i
 // A^-1 by Gauss-Jordan elimination of the column-major n x n work array w (overwritten),
 // written by rows to inv; synchronises to read the zero-pivot flag
 static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_t s) {
-  Buf<double> w2, colk;
-  Buf<int> pivrow, q, err;
-  colk.alloc(2 * (size_t)n, s);
-  pivrow.alloc(n, s);
-  q.alloc(n, s);
+  constexpr int B = kGjB;
+  Buf<int> prow, step[2], err;
+  Buf<double> w2, c[2];
+  Buf<GjPanel> pn[2];
+  prow.alloc(n, s);
   err.alloc(1, s);
-  fill_int(err.p, 0, 1, s);
-  // b pivot steps per launch with the panel factored in every block (one block per SM, its
-  // own columns in a contiguous range); the panel and the b exchanged columns must fit
-  // shared memory, else one launch per step
-  const int nsm = sm_count();
-  const int rcpb = (n + nsm - 1) / nsm;
-  // the widest panel (5 .. 2 steps) whose shared arrays fit, with the own columns staged if
-  // possible
-  constexpr size_t kRpSmem = 212u << 10;
-  int B = 0;
-  bool stage = false;
-  for (int b = 5; b >= 2 && !B; --b)
-    if ((size_t)(2 * b + rcpb) * n * sizeof(double) <= kRpSmem) B = b, stage = true;
-  for (int b = 5; b >= 2 && !B; --b)
-    if ((size_t)(2 * b) * n * sizeof(double) <= kRpSmem) B = b;
-  if (B && rcpb <= kGjMaxCols) {
-    const size_t rsm = (size_t)(2 * B + (stage ? rcpb : 0)) * n * sizeof(double);
-    const int rblocks = (n + rcpb - 1) / rcpb;
-    w2.alloc((size_t)n * n, s);
-    auto run = [&](auto kern) {
-      SAAMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-      for (int k0 = 0; k0 < n; k0 += B) {
-        kern<<<rblocks, kGjRpThreads, rsm, s>>>(n, k0, rcpb, w.p, w2.p, pivrow.p, err.p);
-        SAAMG_LAUNCH();
-        w.swap(w2);
-      }
-    };
-    switch (B * 2 + (stage ? 1 : 0)) {
-      case 11: run(gj_rp_k<5, kGjRpThreads, true>); break;
-      case 10: run(gj_rp_k<5, kGjRpThreads, false>); break;
-      case 9: run(gj_rp_k<4, kGjRpThreads, true>); break;
-      case 8: run(gj_rp_k<4, kGjRpThreads, false>); break;
-      case 7: run(gj_rp_k<3, kGjRpThreads, true>); break;
-      case 6: run(gj_rp_k<3, kGjRpThreads, false>); break;
-      case 5: run(gj_rp_k<2, kGjRpThreads, true>); break;
-      default: run(gj_rp_k<2, kGjRpThreads, false>); break;
-    }
-  } else {
-    gj_first_k<<<1, kGjThreads, 0, s>>>(n, w.p, colk.p, pivrow.p, err.p);
-    SAAMG_LAUNCH();
-    // about two blocks per SM, at most kGjMaxCols columns each
-    const int cpb = std::min(kGjMaxCols, std::max(1, (n + 303) / 304));
-    const int blocks = (n + cpb - 1) / cpb;
-    for (int k = 0; k < n; ++k) {
-      gj_step_k<<<blocks, kGjThreads, 0, s>>>(n, k, cpb, w.p, colk.p + (size_t)(k & 1) * n,
-                                              colk.p + (size_t)((k + 1) & 1) * n, pivrow.p,
-                                              err.p);
-      SAAMG_LAUNCH();
-    }
+  w2.alloc((size_t)n * n, s);
+  for (int q = 0; q < 2; ++q) {
+    step[q].alloc(n, s);
+    c[q].alloc((size_t)B * n, s);
+    pn[q].alloc(1, s);
   }
-  gj_perm_k<<<1, 32, 0, s>>>(n, pivrow.p, q.p);
-  SAAMG_LAUNCH();
+  fill_int(err.p, 0, 1, s);
+  fill_int(step[1].p, -1, n, s);  // read by panel 0: no row is pivoted
+  const int rpb = (n + kGjCluster - 1) / kGjCluster;
+  SAAMG_CUDA(cudaFuncSetAttribute(gj_panel_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)kGjPanelSmem));
+  SAAMG_CUDA(cudaFuncSetAttribute(gj_panel_k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  // tile of the update: the fewest clocks of the busiest SM beside the panel's, a tile costing its
+  // multiply-adds (two a clock) and about 6000 clocks of start-up and forward substitution
+  const int nsm = std::max(1, sm_count() - kGjCluster);
+  int cpb = 1, rt = 1;
+  double least = -1.0;
+  for (int r = 1; r <= 16; ++r)
+    for (int k = 1; k <= kGjUpdCols; ++k) {
+      const long long tiles = (long long)((n + k - 1) / k) * r;
+      const double rows = (double)((n + r - 1) / r);
+      const double cost = (double)((tiles + nsm - 1) / nsm) * (k * rows * B / 2.0 + 6000.0);
+      if (least < 0.0 || cost < least) {
+        least = cost;
+        cpb = k;
+        rt = r;
+      }
+    }
+  const int rpt = (n + rt - 1) / rt;
+  const dim3 ugrid((n + cpb - 1) / cpb, rt);
+  // panel q reads the matrix before update q - 1 and the panel q - 1; update q the same matrix as
+  // panel q + 1, and the panel q.  A panel is launched plainly: everything before it has finished.
+  const int panels = (n + B - 1) / B;
+  auto panel = [&](int q) {
+    const int pq = (q & 1) ^ 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = kGjCluster;
+    cfg.blockDim = kGjThreads;
+    cfg.dynamicSmemBytes = kGjPanelSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kGjCluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SAAMG_CUDA(cudaLaunchKernelEx(&cfg, gj_panel_k, n, q * B, rpb, (const double*)w.p,
+                                  q > 0 ? B : 0, (const GjPanel*)pn[pq].p, (const double*)c[pq].p,
+                                  pn[q & 1].p, c[q & 1].p, (const int*)step[pq].p, step[q & 1].p,
+                                  prow.p, err.p));
+    SAAMG_LAUNCH();
+  };
+  panel(0);
+  for (int q = 0; q < panels; ++q) {
+    const bool beside = q + 1 < panels;
+    if (beside) panel(q + 1);
+    auto args = [&](auto&& launch) {
+      launch(n, q * B, cpb, rpt, (const GjPanel*)pn[q & 1].p, (const double*)c[q & 1].p,
+             (const int*)step[q & 1].p, (const double*)w.p, w2.p);
+    };
+    args([&](auto... a) {
+      if (beside) launch_pdl(gj_update_k, ugrid, kGjUpdThreads, kGjUpdSmem, s, a...);
+      else gj_update_k<<<ugrid, kGjUpdThreads, kGjUpdSmem, s>>>(a...);
+    });
+    SAAMG_LAUNCH();
+    w.swap(w2);
+  }
   const dim3 tiles((n + 31) / 32, (n + 31) / 32);
-  gj_gather_k<<<tiles, 256, 0, s>>>(n, w.p, q.p, inv);
+  gj_gather_k<<<tiles, 256, 0, s>>>(n, w.p, step[(panels - 1) & 1].p, prow.p, inv);
   SAAMG_LAUNCH();
   int herr = 0;
   d2h_sync(&herr, err.p, sizeof(int), s);
@@ -681,7 +624,7 @@ void dense_inverse(int n, const double* a, double* inv, cudaStream_t s) {
   Buf<double> w;
   w.alloc((size_t)n * n, s);
   const dim3 tiles((n + 31) / 32, (n + 31) / 32);
-  gj_gather_k<<<tiles, 256, 0, s>>>(n, a, nullptr, w.p);  // rows of a -> columns of w
+  gj_gather_k<<<tiles, 256, 0, s>>>(n, a, nullptr, nullptr, w.p);  // rows of a -> columns of w
   SAAMG_LAUNCH();
   gauss_jordan_inverse(n, w, inv, s);
 }
