@@ -38,7 +38,7 @@ TRAFFIC_BYTES = {("stencil_smooth", 0, 256): 364.0e6,
                  ("stencil_resid", 1, 256): 82.5e6, ("stencil_resid", 2, 256): 82.5e6,
                  ("prolong0", 1, 256): 81.3e6, ("prolong0", 2, 256): 81.3e6}
 # kernel timing classes of the solve phase (one kernel template each)
-SOLVE_CLASSES = ("stencil_smooth", "stencil_apply", "stencil_resid", "stencil_first",
+SOLVE_CLASSES = ("stencil_pair", "stencil_smooth", "stencil_apply", "stencil_resid", "stencil_first",
                  "coarse_csr", "coarse_deep", "transfer", "transfer_deep", "prolong0")
 
 
@@ -376,11 +376,12 @@ def roofline(name, rec, prec, n=256, index_bytes=4):
         # flops per row: 13 for A x (7 multiply-adds less one), +1 for b - A x, +4 for the
         # Chebyshev update, +1 for x + d; bytes per row: the compulsory vector traffic
         # stencil_first alternates the step from x = 0 (2 flops; b in, d and x out) and the
-        # step with c1 = 0 (17 flops; b, x in, d, x out): their mean
+        # step with c1 = 0 (17 flops; b, x in, d, x out): their mean; stencil_pair alternates the
+        # pair from x = 0 (13 flops; b in, x out) and the pair after a residual (14; r, x in, x out)
         flops = {"stencil_smooth": 19, "stencil_apply": 15, "stencil_resid": 14,
-                 "stencil_first": 9.5}[name] * per
+                 "stencil_first": 9.5, "stencil_pair": 13.5}[name] * per
         nbytes = {"stencil_smooth": 5, "stencil_apply": 2, "stencil_resid": 3,
-                  "stencil_first": 3.5}[name] * w * per
+                  "stencil_first": 3.5, "stencil_pair": 2.5}[name] * w * per
     else:
         # 2 flops per entry; bytes per entry: column index + value (FP32 / BF16 values in
         # the mixed V-cycle; transfers keep FP32 values in both mixed modes).  The level-1
@@ -547,7 +548,8 @@ def mixed_quadratic_leg(S, torch, args):
 def vcycle_bytes(info, prec, degree=2):
     """Algorithmic bytes of one V-cycle from the level sizes: per smoothing or residual sweep
     the matrix entries (column + value) and the vectors; level 0 is matrix-free (20 B per row
-    per Chebyshev step in FP32, 40 in FP64); transfers read P and R once each."""
+    per Chebyshev step in FP32, 40 in FP64, counted step by step although the first two steps
+    of either smoothing are one pass with fewer bytes); transfers read P and R once each."""
     w = 8 if prec == 0 else 4
     n, nnz, nnz_p = info["n"], info["nnz"], info["nnz_p"]
     total = n[0] * w * (10 * degree + 3) + 2 * nnz_p[0] * (w + 4)

@@ -299,7 +299,7 @@ saamg_status saamg_batch_last(int *merged, double *ms_merged, double *ms_graphs)
  * the allocator hook may no longer be callable). */
 saamg_status saamg_release_batch_cache(void);
 
-/* Launch shape of the level-0 stencil passes of one precision (the Chebyshev steps, the
+/* Launch shape of the level-0 stencil passes of one precision (the smoothing passes, the
  * residual and the matrix-free prolongation; the passes with a reduction keep a fixed shape
  * so that their partial sums never change).  Every row is computed the same way under every
  * shape, so results are identical; only the time changes. */
@@ -318,7 +318,7 @@ saamg_status saamg_stencil_config_get(const saamg_operator *op, int precision,
  * set up later, and solve graphs captured later, use it; graphs captured before keep theirs. */
 saamg_status saamg_stencil_config_set(saamg_operator *op, int precision,
                                       const saamg_stencil_config *cfg);
-/* Autotuner of the launch shape: times the level-0 Chebyshev step of precision 0 or 1 under
+/* Autotuner of the launch shape: times the level-0 smoothing pass of precision 0 or 1 under
  * all 36 shapes on scratch vectors of op's size (allocated and freed here), sets the fastest
  * on op and returns it with its time in microseconds (median of three launches). */
 saamg_status saamg_autotune_stencil(saamg_operator *op, int precision, void *stream,
@@ -403,7 +403,8 @@ typedef enum {
   SAAMG_KT_PROLONG0 = 8,       /* matrix-free level-0 prolongation of the FP32 V-cycle */
   SAAMG_KT_COARSE_DEEP = 9,    /* SAAMG_KT_COARSE on levels >= 2 */
   SAAMG_KT_TRANSFER_DEEP = 10, /* SAAMG_KT_TRANSFER between levels >= 1 */
-  SAAMG_KT_COUNT = 11
+  SAAMG_KT_STENCIL_PAIR = 11,  /* two level-0 Chebyshev steps as one pass (k0 r - k1 A r) */
+  SAAMG_KT_COUNT = 12
 } saamg_kernel_class;
 
 /* Number of kernels this library has launched in the calling process. */

@@ -546,6 +546,27 @@ struct Planner {
     return o;
   }
 
+  // the level-0 pair passes of the one-solve V-cycle
+  template <class T>
+  void pair(int phase, int step, int mode, const T* x, T* y, T* d, const SmoothPair<T>& sp) {
+    const StencilDev<T> S = w.h->op->d.template view<T>();
+    Op o = base(phase, 0, step);
+    StTask<T> t{};
+    t.S = pair_stencil(S, sp.k0, sp.k1);
+    t.go = go;
+    t.x = x;
+    t.y = y;
+    t.d = d;
+    t.c1 = sp.k1;
+    t.c2 = sp.k0;
+    t.c2i0 = sp.g;
+    o.key.fam = sizeof(T) == 4 ? F_ST32 : F_ST64;
+    o.key.mode = mode;
+    o.units = stencil_units<T>(S);
+    set_st(o, t);
+    add(o);
+  }
+
   // smooth_step of the one-solve V-cycle
   template <class T>
   void smooth(int phase, int l, int step, int mode0, const T* x, T* y, const T* b, T* d, T c1,
@@ -692,9 +713,13 @@ struct Planner {
     const int nu = (int)L.cheb.c1.size();
     T* bufs[2] = {WV<T>::x0(w, l), out};
     T* d = WV<T>::d(w, l);
-    int cur = 0;
-    smooth<T>(P_PRE, l, 0, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0]);
-    for (int k = 1; k < nu; ++k) {
+    const bool pr = l == 0 && nu >= 2;
+    const SmoothPair<T> sp = pr ? SmoothPair<T>(L.cheb.c2[0], L.cheb.c1[1], L.cheb.c2[1])
+                                : SmoothPair<T>(0.0, 0.0, 0.0);
+    int cur = pr ? 1 : 0;
+    if (pr) pair<T>(P_PRE, 0, ST_PAIR0, b, bufs[cur], nu > 2 ? d : nullptr, sp);
+    else smooth<T>(P_PRE, l, 0, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0]);
+    for (int k = pr ? 2 : 1; k < nu; ++k) {
       smooth<T>(P_PRE, l, k, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
                 (T)L.cheb.c2[k]);
       cur = 1 - cur;
@@ -706,7 +731,11 @@ struct Planner {
     transfer<T>(P_RESTRICT, l, true, r, bc);
     vcycle<T>(l + 1, bc, vc);
     transfer<T>(P_PROLONG, l, false, vc, bufs[cur]);
-    for (int k = 0; k < nu; ++k) {
+    if (pr) {
+      smooth<T>(P_POST, l, 0, CSR_RESID, bufs[cur], r, b, nullptr, T(0), T(0));
+      pair<T>(P_POST, 1, nu > 2 ? ST_PAIR_D : ST_PAIR, r, bufs[cur], d, sp);
+    }
+    for (int k = pr ? 2 : 0; k < nu; ++k) {
       smooth<T>(P_POST, l, k, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
                 (T)L.cheb.c2[k]);
       cur = 1 - cur;

@@ -703,7 +703,9 @@ static void release_hierarchy(saamg_hierarchy* h) {
 // --- V-cycle (Algorithm 1) -------------------------------------------------
 // Level l smooths b_l -> x_l; the final iterate lands in `out` (length n_l).  The
 // Chebyshev steps ping-pong between two buffers: with nu pre- and nu post-steps there are
-// 2 nu - 1 swaps after the first step, so starting in `tmp` ends in `out`.
+// 2 nu - 1 swaps after the first step, so starting in `tmp` ends in `out`.  On level 0 the first
+// two steps of either smoothing are one pass (SmoothPair); the second pair works in place, which
+// leaves 2 nu - 4 swaps, so starting in `out` ends there.
 template <class T>
 struct LevelVecs;
 
@@ -819,10 +821,17 @@ static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStre
   const int nu = (int)L.cheb.c1.size();
   T* bufs[2] = {LevelVecs<T>::x0(L), out};
   T* d = LevelVecs<T>::d(L);
-  int cur = 0;
+  const bool pair = l == 0 && nu >= 2;
+  const SmoothPair<T> sp = pair ? SmoothPair<T>(L.cheb.c2[0], L.cheb.c1[1], L.cheb.c2[1])
+                                : SmoothPair<T>(0.0, 0.0, 0.0);
+  int cur = pair ? 1 : 0;
   // presmoothing from x = 0
-  smooth_step<T>(h, l, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0], s);
-  for (int k = 1; k < nu; ++k) {
+  if (pair)
+    stencil_apply<T>(h->op->d.template view<T>(), ST_PAIR0, b, bufs[cur], nullptr,
+                     nu > 2 ? d : nullptr, sp.k1, sp.k0, nullptr, s, nullptr, sp.g);
+  else
+    smooth_step<T>(h, l, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0], s);
+  for (int k = pair ? 2 : 1; k < nu; ++k) {
     smooth_step<T>(h, l, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
                    (T)L.cheb.c2[k], s);
     cur = 1 - cur;
@@ -837,7 +846,12 @@ static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStre
   vcycle_level<T>(h, l + 1, bc, vc, s);
   transfer<T>(h, l, false, vc, bufs[cur], s);
   // postsmoothing with the same polynomial
-  for (int k = 0; k < nu; ++k) {
+  if (pair) {
+    smooth_step<T>(h, l, CSR_RESID, bufs[cur], r, b, nullptr, T(0), T(0), s);
+    stencil_apply<T>(h->op->d.template view<T>(), nu > 2 ? ST_PAIR_D : ST_PAIR, r, bufs[cur],
+                     nullptr, d, sp.k1, sp.k0, nullptr, s, nullptr, sp.g);
+  }
+  for (int k = pair ? 2 : 0; k < nu; ++k) {
     smooth_step<T>(h, l, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
                    (T)L.cheb.c2[k], s);
     cur = 1 - cur;

@@ -79,17 +79,47 @@ enum StencilMode {
   ST_CHEB0 = 4,     // d = c2 D^-1 b; y = d   (Chebyshev step 0 from x = 0)
   ST_DINV_DOT = 5,  // y = s D^-1 A x, partials of y.y (power iteration; s = *xscale or 1)
   ST_CHEB1 = 6,     // ST_CHEB with c1 = 0 (first step from a nonzero x): d is not read
-  ST_PROLONG = 7    // y += P v with P = (I - omega D^-1 A) T, T from the aggregates
+  ST_PROLONG = 7,   // y += P v with P = (I - omega D^-1 A) T, T from the aggregates
+  // the first two Chebyshev steps as one pass (see SmoothPair): x is b or the residual
+  ST_PAIR0 = 8,     // y = k0 x - k1 A x; d = y - g x (if d is not null)
+  ST_PAIR = 9,      // y += k0 x - k1 A x
+  ST_PAIR_D = 10    // e = k0 x - k1 A x; y += e; d = e - g x
 };
+
+// Two Chebyshev steps on level 0 from x with residual r = b - A x (x = 0: r = b).  The scaled
+// operator's diagonal is 1 to rounding (a_ii s_i s_i with s_i = a_ii^-1/2), so D^-1 is left out and
+//   x1 = x + g r, r1 = r - g A r, x2 = x1 + c1 g r + c2 r1 = x + k0 r - k1 A r,
+//   k0 = g + c1 g + c2, k1 = c2 g;   d = x2 - x1.
+// From x = 0 that is one pass over b instead of two (7 FP64 operations a row instead of 11, 16 bytes
+// instead of 64), after the prolongation the residual and one pass (15 instead of 19 operations, 48
+// bytes instead of 72): at 256^3 in FP64 43 + 148 -> TIME_A us and 134 + 148 -> TIME_B us.
+template <class T>
+struct SmoothPair {
+  T k0, k1, g;
+  SmoothPair(double g_, double c1, double c2)
+      : k0((T)(g_ + c1 * g_ + c2)), k1((T)(c2 * g_)), g((T)g_) {}
+};
+
+// c1, c2: of the Chebyshev steps; the pair passes take k1, k0 there and g
 template <class T>
 void stencil_apply(const StencilDev<T>& S, int mode, const T* x, T* y, const T* b, T* d, T c1,
-                   T c2, double* partials, cudaStream_t s, const double* xscale = nullptr);
+                   T c2, double* partials, cudaStream_t s, const double* xscale = nullptr,
+                   T g = T(0));
+// S with the regular rows' coefficients of k0 I - k1 A, as the pair passes apply it
+template <class T>
+StencilDev<T> pair_stencil(StencilDev<T> S, T k0, T k1) {
+  S.c0 = k0 - k1 * S.c0;
+  S.cx = -k1 * S.cx;
+  S.cy = -k1 * S.cy;
+  S.cz = -k1 * S.cz;
+  return S;
+}
 // Level-0 prolongation without the matrix P (Sec. 3.2: P = (I - omega D^-1 A) T):
 // y_i += v_agg(i) - omega invd_i sum_j a_ij v_agg(j), agg = level-0 aggregate of each row
 template <class T>
 void stencil_prolong(const StencilDev<T>& S, const int* agg, T omega, const T* v, T* y,
                      cudaStream_t s);
-// Times the level-0 Chebyshev step under every launch shape (K 1/2/4, packed or line chunks,
+// Times the level-0 smoothing pass under every launch shape (K 1/2/4, packed or line chunks,
 // 128/256 threads, 8/16/32 blocks per SM) on scratch vectors and returns the fastest; its
 // time (median of three launches) in *best_us.
 template <class T>

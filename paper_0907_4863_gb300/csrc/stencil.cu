@@ -70,6 +70,7 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
                                             const T* __restrict__ b, T* __restrict__ d, T c1,
                                             T c2, T c2invd0, double& dacc,
                                             const int* __restrict__ agg) {
+    constexpr bool kPair = MODE == ST_PAIR0 || MODE == ST_PAIR || MODE == ST_PAIR_D;
     int row;
     int ra = 0, rb = 0, tl = 0;  // chunk path: lanes of the regular run, table row of lane 0
     int4 nb;
@@ -111,7 +112,17 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       ayp = tb[4];
       azm = tb[5];
       azp = tb[6];
-      c2i = c2 * tb[7];
+      if (kPair) {  // the row of k0 I - k1 A (c2 = k0, c1 = k1)
+        a0 = fma(-c1, a0, c2);
+        axm *= -c1;
+        axp *= -c1;
+        aym *= -c1;
+        ayp *= -c1;
+        azm *= -c1;
+        azp *= -c1;
+      } else {
+        c2i = c2 * tb[7];
+      }
       oxm = nonzero(axm) ? oxm : 0;
       oxp = nonzero(axp) ? oxp : 0;
       oym = nonzero(aym) ? oym : 0;
@@ -173,7 +184,7 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       acc = fma(-azm, vzm, acc);
       acc = fma(-azp, vzp, acc);
     } else {
-      acc = a0 * xc;
+      acc = MODE == ST_PAIR ? fma(a0, xc, y[row]) : a0 * xc;
       acc = fma(axm, vxm, acc);
       acc = fma(axp, vxp, acc);
       acc = fma(aym, vym, acc);
@@ -190,6 +201,14 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       if (MODE == ST_SPMV_DOT) dacc = fma(to_d(xc), to_d(acc), dacc);
     } else if (MODE == ST_RESID) {
       y[row] = acc;
+    } else if (MODE == ST_PAIR) {
+      y[row] = acc;
+    } else if (MODE == ST_PAIR0) {  // the c2invd0 argument holds g
+      y[row] = acc;
+      if (d) d[row] = fma(-c2invd0, xc, acc);
+    } else if (MODE == ST_PAIR_D) {
+      y[row] = y[row] + acc;
+      d[row] = fma(-c2invd0, xc, acc);
     } else if (MODE == ST_PROLONG) {  // c2 = omega: y += (T v)_i - omega invd_i (A T v)_i
       y[row] = y[row] + fma(-c2i, acc, xc);
     } else {  // ST_CHEB / ST_CHEB1: d = c1 d + c2 D^-1 r; x_out = x + d
@@ -396,6 +415,15 @@ void batched_stencil(int mode, const StTask<T>* tasks, const int4* wbs, int nwb,
     case ST_PROLONG:
       SAAMG_BST(ST_PROLONG);
       break;
+    case ST_PAIR0:
+      SAAMG_BST(ST_PAIR0);
+      break;
+    case ST_PAIR:
+      SAAMG_BST(ST_PAIR);
+      break;
+    case ST_PAIR_D:
+      SAAMG_BST(ST_PAIR_D);
+      break;
     default:
       fail(SAAMG_EINVAL, "bad batched stencil mode");
   }
@@ -448,8 +476,10 @@ long long shaped_units(const StencilDev<T>& S, bool packed) {
 }
 
 template <class T>
-void stencil_apply(const StencilDev<T>& S, int mode, const T* x, T* y, const T* b, T* d, T c1,
-                   T c2, double* partials, cudaStream_t s, const double* xscale) {
+void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T* b, T* d, T c1,
+                   T c2, double* partials, cudaStream_t s, const double* xscale, T g) {
+  const bool pair = mode == ST_PAIR0 || mode == ST_PAIR || mode == ST_PAIR_D;
+  const StencilDev<T> S = pair ? pair_stencil(S0, c2, c1) : S0;
   if (S.nchunks == 0) {
     if (mode == ST_SPMV_DOT || mode == ST_DINV_DOT) fill_double(partials, 0.0, kRedBlocks, s);
     return;
@@ -461,11 +491,12 @@ void stencil_apply(const StencilDev<T>& S, int mode, const T* x, T* y, const T* 
                  : (mode == ST_SPMV || mode == ST_SPMV_DOT) ? SAAMG_KT_STENCIL_APPLY
                  : mode == ST_RESID                         ? SAAMG_KT_STENCIL_RESID
                  : (mode == ST_CHEB0 || mode == ST_CHEB1)   ? SAAMG_KT_STENCIL_FIRST
+                 : pair                                     ? SAAMG_KT_STENCIL_PAIR
                                                             : -1,
                  S.n, s);
   // c2 / diag of the regular rows, formed here: a kernel that forms it from c2 lets the
   // compiler merge it with the table rows' c2 * (1/diag) into one multiply on every row
-  const T c2i0 = c2 * S.invd0;
+  const T c2i0 = pair ? g : c2 * S.invd0;
   if (mode == ST_SPMV_DOT || mode == ST_DINV_DOT) {
     // reductions: the fixed grid and the default shape, so that partial sums are always
     // taken the same way
@@ -504,6 +535,18 @@ void stencil_apply(const StencilDev<T>& S, int mode, const T* x, T* y, const T* 
       launch_shaped<T, ST_CHEB1>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
       break;
+    case ST_PAIR0:
+      launch_shaped<T, ST_PAIR0>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+                                 nullptr, s);
+      break;
+    case ST_PAIR:
+      launch_shaped<T, ST_PAIR>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+                                nullptr, s);
+      break;
+    case ST_PAIR_D:
+      launch_shaped<T, ST_PAIR_D>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+                                  nullptr, s);
+      break;
     default:
       fail(SAAMG_EINVAL, "bad stencil mode");
   }
@@ -522,7 +565,7 @@ void stencil_prolong(const StencilDev<T>& S, const int* agg, T omega, const T* v
   SAAMG_LAUNCH();
 }
 
-// Times the Chebyshev step of every launch shape on scratch vectors and returns the fastest
+// Times the smoothing pass of every launch shape on scratch vectors and returns the fastest
 // (median of three launches after one untimed).
 template <class T>
 StencilCfg stencil_autotune(const StencilDev<T>& S0, cudaStream_t s, double* best_us) {
@@ -546,11 +589,11 @@ StencilCfg stencil_autotune(const StencilDev<T>& S0, cudaStream_t s, double* bes
         for (int block : {128, 256})
           for (int per_sm : {8, 16, 32}) {
             S.cfg = StencilCfg{k, packed, block, per_sm};
-            stencil_apply<T>(S, ST_CHEB, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
+            stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
             float t[3];
             for (int r = 0; r < 3; ++r) {
               SAAMG_CUDA(cudaEventRecord(e[0], s));
-              stencil_apply<T>(S, ST_CHEB, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
+              stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
               SAAMG_CUDA(cudaEventRecord(e[1], s));
               SAAMG_CUDA(cudaEventSynchronize(e[1]));
               SAAMG_CUDA(cudaEventElapsedTime(&t[r], e[0], e[1]));
@@ -580,9 +623,9 @@ template void stencil_prolong<double>(const StencilDev<double>&, const int*, dou
 
 template void stencil_apply<double>(const StencilDev<double>&, int, const double*, double*,
                                     const double*, double*, double, double, double*,
-                                    cudaStream_t, const double*);
+                                    cudaStream_t, const double*, double);
 template void stencil_apply<float>(const StencilDev<float>&, int, const float*, float*,
                                    const float*, float*, float, float, double*, cudaStream_t,
-                                   const double*);
+                                   const double*, float);
 
 }  // namespace saamg
