@@ -33,7 +33,7 @@ namespace saamg {
 namespace {
 
 constexpr int kWarps = 8;         // warps per block of the batched kernels
-constexpr int kWarpUnits = 4;     // warp-sized units per warp and work block
+constexpr int kWarpUnits = 4;     // warp-sized units per warp and work block, at least
 constexpr int kBlockUnits = 4;    // 256-element units per work block (vector kernels)
 constexpr int kMaxLanes = 8;      // concurrent sub-batches of a batch
 constexpr int kLaneSolves = 32;   // solves per lane (about)
@@ -61,6 +61,7 @@ struct VTask {  // the CG recursion of one solve
   int* go;
   int n;
   PcgCtl* ctl;
+  const double* bhat;
   double* x;
   double* r;
   double* p;
@@ -94,7 +95,7 @@ __device__ __forceinline__ void load_task(const Task* __restrict__ tasks, int t,
 
 // --- sparse-matrix kernels --------------------------------------------------------------------
 template <class TV, class TM, int G, int MODE>
-__global__ void __launch_bounds__(256, 5) bcsr_k(const MTask* __restrict__ tasks,
+__global__ void __launch_bounds__(256, 4) bcsr_k(const MTask* __restrict__ tasks,
                                               const int4* __restrict__ wbs, int nwb) {
   __shared__ MTask sk;
   const int lane = threadIdx.x & 31, gl = lane % G, warp = threadIdx.x >> 5;
@@ -102,12 +103,30 @@ __global__ void __launch_bounds__(256, 5) bcsr_k(const MTask* __restrict__ tasks
   double dacc = 0.0;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     SAAMG_WORK_BLOCK(MTask)
-    for (int u = B.y + warp; u < B.z; u += kWarps) {
-    const int row = u * kRows + lane / G;
-    rows::csr_group_row<TV, TM, G, MODE>(row, row < k.n, gl, k.rowptr, k.col,
-                                         (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
-                                         (const TV*)k.b, (TV*)k.d, (const TV*)k.invd, (TV)k.c1,
-                                         (TV)k.c2, dacc);
+    if (MODE == CSR_CHEB0) {
+      for (int u = B.y + warp; u < B.z; u += kWarps) {
+        const int row = u * kRows + lane / G;
+        rows::csr_group_row<TV, TM, G, MODE>(row, row < k.n, gl, k.rowptr, k.col,
+                                             (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
+                                             (const TV*)k.b, (TV*)k.d, (const TV*)k.invd, (TV)k.c1,
+                                             (TV)k.c2, dacc);
+      }
+    } else {
+      // four row groups a warp step, their loads in flight together
+      constexpr int NR = G < 4 ? G : 4;
+      for (int u = B.y + warp; u < B.z; u += NR * kWarps) {
+        int row[NR];
+        bool active[NR];
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+          row[q] = (u + q * kWarps) * kRows + lane / G;
+          active[q] = u + q * kWarps < B.z && row[q] < k.n;
+        }
+        rows::csr_group_rows<TV, TM, G, MODE, NR>(row, active, gl, k.rowptr, k.col,
+                                                  (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
+                                                  (const TV*)k.b, (TV*)k.d, (const TV*)k.invd,
+                                                  (TV)k.c1, (TV)k.c2);
+      }
     }
   }
 }
@@ -228,6 +247,32 @@ __global__ void __launch_bounds__(256) bupdate_k(const VTask* __restrict__ tasks
   }
 }
 
+// Partials of a vector's square around the loop: b'b into part2 and r'r into part1, with the FP32
+// copy of r (the prologue), or q'q of the recomputed residual into part0 (the epilogue).
+enum Square { SQ_B, SQ_R, SQ_Q };
+
+__global__ void __launch_bounds__(256) bsquare_k(const VTask* __restrict__ tasks, int ntasks,
+                                                 int which) {
+  const int lane = threadIdx.x & 31;
+  const long long npairs = (long long)ntasks * kRedBlocks;
+  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long pr = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs;
+       pr += nwarps) {
+    const VTask& k = tasks[pr / kRedBlocks];
+    const int b = (int)(pr % kRedBlocks);
+    const double* v = which == SQ_B ? k.bhat : (which == SQ_R ? k.r : k.q);
+    double* part = which == SQ_B ? k.part2 : (which == SQ_R ? k.part1 : k.part0);
+    double t = 0.0;
+    if (b * kRedThreads < k.n) {
+      float* copy = which == SQ_R ? k.r32 : nullptr;
+      if (copy)
+        rows::virt_block(b, k.n, lane, [&](int i, int) { copy[i] = (float)v[i]; });
+      t = rows::dot_block_warp<double, double>(b, k.n, v, v, lane);
+    }
+    if (lane == 0) part[b] = t;
+  }
+}
+
 int resident_blocks(const void* kernel);
 
 inline int grid_pairs(int ntasks, const void* kernel) {  // blocks of 8 warps, a warp per pair
@@ -286,6 +331,12 @@ __global__ void __launch_bounds__(kRedThreads) binit_k(const VTask* __restrict__
     ctl->beta = 0.0;
     *k.go = !ctl->converged && !ctl->breakdown && k.maxit > 0;
   }
+}
+
+__global__ void __launch_bounds__(kRedThreads) bstore_true_k(const VTask* __restrict__ tasks) {
+  const VTask& k = tasks[blockIdx.x];
+  const double rr = rows::sum_fixed(k.part0);
+  if (threadIdx.x == 0) k.ctl->rr_true = rr;
 }
 
 __global__ void __launch_bounds__(kRedThreads) bbeta_k(const VTask* __restrict__ tasks) {
@@ -484,6 +535,15 @@ void work_blocks(const std::vector<int>& units, int per, std::vector<int4>& out)
       out.push_back(make_int4((int)t, u, std::min(units[t], u + per), 0));
 }
 
+// Warp-sized units per work block: about ten blocks per SM (each costs a task load and two
+// barriers), 32 to 128 units.
+int units_per_block(const std::vector<int>& units) {
+  long long total = 0;
+  for (int u : units) total += u;
+  const long long step = kWarps * kWarpUnits, want = total / (10LL * sm_count());
+  return (int)std::max(step, std::min(4 * step, (want + step - 1) / step * step));
+}
+
 // --- planning ---------------------------------------------------------------------------------
 enum Phase { P_PRE = 0, P_RESID, P_RESTRICT, P_COARSE, P_PROLONG, P_POST, P_COPY };
 
@@ -502,7 +562,7 @@ struct SolveWork {
   Buf<double> bhat, xhat, r, z, p, q;
   Buf<float> z32, r32;
   Buf<double> part0, part1, part2;
-  Buf<PcgCtl> ctl;
+  PcgCtl* ctl = nullptr;  // in its lane's array
   std::vector<Buf<double>> dx0, dx1, db, dd, dr;
   std::vector<Buf<float>> fx0, fx1, fb, fd, fr;
 };
@@ -767,7 +827,8 @@ struct Group {
 // so that one lane's short, latency-bound launches overlap another's).
 struct Lane {
   std::vector<int> sol;       // global indices of its solves
-  Buf<int> go;                // loop flags, one per solve of the lane
+  Buf<int> go;                // loop flags, one per solve of the lane, and a last one that is 1
+  Buf<PcgCtl> ctl;            // CG scalars, one per solve of the lane
   Buf<unsigned char> tasks;   // every task table and work-block list of the loop body
   Buf<VTask> vtasks;
   std::vector<Group> groups;            // the V-cycle launches, in order
@@ -780,6 +841,11 @@ struct Lane {
   Buf<int4> vall_off;          // all solves of the lane: work blocks (zero)
   int vall_units = 0;
   Buf<StTask<double>> dot_tasks;  // A p with p'Ap partials
+  // before and after the loop: gather / scatter, and the residuals b - A x into r and into q
+  Buf<BoxTask> box;
+  Buf<StTask<double>> res_tasks;  // m into r, then m into q
+  Buf<int4> pro_wbs;              // work blocks: gather, scatter, residual
+  int n_gather = 0, n_scatter = 0, n_resid = 0;
   long long k_body = 0;
 };
 
@@ -788,7 +854,8 @@ struct BatchEngine {
   std::vector<std::unique_ptr<Lane>> lanes;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  PcgCtl* res = nullptr;  // pinned host copies of every solve's scalars after a run
+  PcgCtl* res = nullptr;  // pinned host copies of the scalars after a run, lane by lane
+  mutable std::vector<PcgCtl> by_solve;  // the same in the order of the solves
   long long k_fixed = 0;
   ~BatchEngine() {
     if (exec) cudaGraphExecDestroy(exec);
@@ -827,7 +894,6 @@ void alloc_work(SolveWork& w, cudaStream_t s) {
   w.part0.alloc(kRedBlocks, s);
   w.part1.alloc(kRedBlocks, s);
   w.part2.alloc(kRedBlocks, s);
-  w.ctl.alloc(1, s);
   const int nl = (int)h->lev.size();
   if (mx) {
     w.fx0.resize(nl);
@@ -882,10 +948,13 @@ long long slot_of(const Op& o, int lmax, int numax) {
 namespace {
 
 // Plans the lane's V-cycles, merges their operations and uploads every task table.
-void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work, double rtol,
-                cudaStream_t s) {
+void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
+                const double* const* rho, double* const* phi, double rtol, cudaStream_t s) {
   const int m = (int)L.sol.size();
-  L.go.alloc(m, s);
+  L.go.alloc(m + 1, s);
+  fill_int(L.go.p + m, 1, 1, s);
+  L.ctl.alloc(m, s);
+  for (int i = 0; i < m; ++i) work[L.sol[i]]->ctl = L.ctl.p + i;
   std::vector<Op> ops;
   int lmax = 0, numax = 0;
   for (int i = 0; i < m; ++i) {
@@ -934,7 +1003,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work, double r
       units.push_back(o.units);
     }
     std::vector<int4> wb;
-    work_blocks(units, kWarps * kWarpUnits, wb);
+    work_blocks(units, units_per_block(units), wb);
     g.nwb = (int)wb.size();
     align(16);
     g.wb_off = host.size();
@@ -954,7 +1023,8 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work, double r
     VTask& t = vt[i];
     t.go = L.go.p + i;
     t.n = h->op->d.n;
-    t.ctl = w.ctl.p;
+    t.ctl = w.ctl;
+    t.bhat = w.bhat.p;
     t.x = w.xhat.p;
     t.r = w.r.p;
     t.p = w.p.p;
@@ -1025,6 +1095,91 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work, double r
     SAAMG_CUDA(cudaMemcpyAsync(L.dot_tasks.p, dt.data(), sizeof(StTask<double>) * m,
                                cudaMemcpyHostToDevice, s));
   }
+  {
+    std::vector<BoxTask> box(m);
+    std::vector<StTask<double>> rt(2 * m);
+    std::vector<int> ug, us, ur;
+    for (int i = 0; i < m; ++i) {
+      SolveWork& w = *work[L.sol[i]];
+      const OperatorData& od = w.h->op->d;
+      BoxTask& t = box[i];
+      t.g = od.g;
+      t.lines = od.lines.p;
+      t.chunks = od.chunks.p;
+      t.scale = od.scale.p;
+      t.rho = rho[L.sol[i]];
+      t.phi = phi[L.sol[i]];
+      t.bhat = w.bhat.p;
+      t.xhat = w.xhat.p;
+      t.p = w.p.p;
+      t.nbox = (size_t)od.g.nx * od.g.ny * od.g.nz;
+      StTask<double> r{};
+      r.S = od.view<double>();
+      r.go = L.go.p + m;
+      r.x = w.xhat.p;
+      r.b = w.bhat.p;
+      r.y = w.r.p;
+      rt[i] = r;
+      r.y = w.q.p;
+      rt[m + i] = r;
+      ug.push_back(od.nchunks);
+      us.push_back((int)((t.nbox + 255) / 256));
+      ur.push_back(stencil_units<double>(r.S));
+    }
+    std::vector<int4> wb;
+    work_blocks(ug, units_per_block(ug), wb);
+    L.n_gather = (int)wb.size();
+    work_blocks(us, kBlockUnits, wb);
+    L.n_scatter = (int)wb.size() - L.n_gather;
+    work_blocks(ur, units_per_block(ur), wb);
+    L.n_resid = (int)wb.size() - L.n_gather - L.n_scatter;
+    L.box.alloc(m, s);
+    L.res_tasks.alloc(2 * m, s);
+    L.pro_wbs.alloc(wb.size(), s);
+    SAAMG_CUDA(cudaMemcpyAsync(L.box.p, box.data(), sizeof(BoxTask) * m, cudaMemcpyHostToDevice, s));
+    SAAMG_CUDA(cudaMemcpyAsync(L.res_tasks.p, rt.data(), sizeof(StTask<double>) * 2 * m,
+                               cudaMemcpyHostToDevice, s));
+    SAAMG_CUDA(cudaMemcpyAsync(L.pro_wbs.p, wb.data(), sizeof(int4) * wb.size(),
+                               cudaMemcpyHostToDevice, s));
+  }
+}
+
+// Partials of a square of every solve of the lane.
+void lane_square(Lane& L, Square which, cudaStream_t s) {
+  const int m = (int)L.sol.size();
+  bsquare_k<<<grid_pairs(m, reinterpret_cast<const void*>(bsquare_k)), 256, 0, s>>>(L.vtasks.p, m,
+                                                                                   which);
+  SAAMG_LAUNCH();
+}
+
+// The one-solve graph's prologue for every solve of the lane: b and x from the box, p = 0, b'b,
+// r = b - A x, r'r, the scalars and the loop condition.
+void lane_prologue(Lane& L, cudaGraphConditionalHandle cond, cudaStream_t s) {
+  const int m = (int)L.sol.size();
+  batched_gather(L.box.p, L.pro_wbs.p, L.n_gather, s);
+  lane_square(L, SQ_B, s);
+  batched_stencil<double>(ST_RESID, L.res_tasks.p, L.pro_wbs.p + L.n_gather + L.n_scatter,
+                          L.n_resid, s);
+  lane_square(L, SQ_R, s);
+  binit_k<<<m, kRedThreads, 0, s>>>(L.vtasks.p);
+  SAAMG_LAUNCH();
+  bzero_k<<<grid_wb(L.vall_units, reinterpret_cast<const void*>(bzero_k)), 256, 0, s>>>(
+      L.vtasks.p, L.vall_off.p, L.vall_units);
+  SAAMG_LAUNCH();
+  bany_k<<<1, 256, 0, s>>>(L.go.p, m, cond);
+  SAAMG_LAUNCH();
+}
+
+// Its epilogue: the recomputed residual, the scalars to the host, phi.
+void lane_epilogue(Lane& L, PcgCtl* res, cudaStream_t s) {
+  const int m = (int)L.sol.size();
+  batched_stencil<double>(ST_RESID, L.res_tasks.p + m, L.pro_wbs.p + L.n_gather + L.n_scatter,
+                          L.n_resid, s);
+  lane_square(L, SQ_Q, s);
+  bstore_true_k<<<m, kRedThreads, 0, s>>>(L.vtasks.p);
+  SAAMG_LAUNCH();
+  SAAMG_CUDA(cudaMemcpyAsync(res, L.ctl.p, sizeof(PcgCtl) * m, cudaMemcpyDeviceToHost, s));
+  batched_scatter(L.box.p, L.pro_wbs.p + L.n_gather, L.n_scatter, s);
 }
 
 // One pass of the lane's loop body on stream s.
@@ -1114,7 +1269,7 @@ BatchEngine* batch_engine_build(saamg_hierarchy* const* hs, const double* const*
   for (auto& sol : make_lanes(hs, count, nlanes)) {
     e->lanes.emplace_back(new Lane());
     e->lanes.back()->sol = sol;
-    build_lane(*e->lanes.back(), e->work, rtol, s);
+    build_lane(*e->lanes.back(), e->work, rho, phi, rtol, s);
   }
   SAAMG_CUDA(cudaStreamSynchronize(s));
   SAAMG_CUDA(cudaMallocHost(&e->res, sizeof(PcgCtl) * count));
@@ -1139,32 +1294,12 @@ BatchEngine* batch_engine_build(saamg_hierarchy* const* hs, const double* const*
     evs.push_back(fork);
     SAAMG_CUDA(cudaEventRecord(fork, cs));
     std::vector<cudaGraph_t> bodies(e->lanes.size());
+    size_t done = 0;  // solves of the lanes before
     for (size_t li = 0; li < e->lanes.size(); ++li) {
       Lane& L = *e->lanes[li];
       cudaStream_t ls = stream_of(2 + 2 * (int)li);
       SAAMG_CUDA(cudaStreamWaitEvent(ls, fork, 0));
-      const int m = (int)L.sol.size();
-      // prologue of every solve (the one-solve graph's prologue, per solve)
-      for (int j : L.sol) {
-        SolveWork& w = *e->work[j];
-        saamg_hierarchy* h = hs[j];
-        const OperatorData& od = h->op->d;
-        const int n = od.n;
-        const StencilDev<double> S = od.view<double>();
-        gather_rhs(od, rho[j], phi[j], w.bhat.p, w.xhat.p, ls);
-        dot_partials<double, double>(n, w.bhat.p, w.bhat.p, w.part2.p, ls);
-        stencil_apply<double>(S, ST_RESID, w.xhat.p, w.r.p, w.bhat.p, nullptr, 0.0, 0.0, nullptr, ls);
-        if (h->prm.precision != SAAMG_PREC_FP64) to_float(w.r.p, w.r32.p, n, ls);
-        dot_partials<double, double>(n, w.r.p, w.r.p, w.part1.p, ls);
-        SAAMG_CUDA(cudaMemsetAsync(w.p.p, 0, sizeof(double) * n, ls));
-      }
-      binit_k<<<m, kRedThreads, 0, ls>>>(L.vtasks.p);
-      SAAMG_LAUNCH();
-      bzero_k<<<grid_wb(L.vall_units, reinterpret_cast<const void*>(bzero_k)), 256, 0, ls>>>(
-          L.vtasks.p, L.vall_off.p, L.vall_units);
-      SAAMG_LAUNCH();
-      bany_k<<<1, 256, 0, ls>>>(L.go.p, m, conds[li]);
-      SAAMG_LAUNCH();
+      lane_prologue(L, conds[li], ls);
       // the while node
       cudaStreamCaptureStatus st;
       cudaGraph_t cg = nullptr;
@@ -1180,17 +1315,8 @@ BatchEngine* batch_engine_build(saamg_hierarchy* const* hs, const double* const*
       SAAMG_CUDA(cudaGraphAddNode(&cnode, cg, deps, nullptr, nd, &cp));
       bodies[li] = cp.conditional.phGraph_out[0];
       SAAMG_CUDA(cudaStreamUpdateCaptureDependencies(ls, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-      // epilogue of every solve: recomputed residual, result copy, scatter
-      for (int j : L.sol) {
-        SolveWork& w = *e->work[j];
-        const OperatorData& od = hs[j]->op->d;
-        const StencilDev<double> S = od.view<double>();
-        stencil_apply<double>(S, ST_RESID, w.xhat.p, w.q.p, w.bhat.p, nullptr, 0.0, 0.0, nullptr, ls);
-        dot_partials<double, double>(od.n, w.q.p, w.q.p, w.part0.p, ls);
-        pcg_store_true(w.part0.p, w.ctl.p, ls);
-        SAAMG_CUDA(cudaMemcpyAsync(&e->res[j], w.ctl.p, sizeof(PcgCtl), cudaMemcpyDeviceToHost, ls));
-        scatter_solution(od, w.xhat.p, phi[j], ls);
-      }
+      lane_epilogue(L, e->res + done, ls);
+      done += L.sol.size();
       cudaEvent_t join;
       SAAMG_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
       evs.push_back(join);
@@ -1238,13 +1364,20 @@ void batch_engine_launch(BatchEngine* e, cudaStream_t s) {
   SAAMG_CUDA(cudaGraphLaunch(e->exec, s));
 }
 
-const PcgCtl* batch_engine_results(const BatchEngine* e) { return e->res; }
+const PcgCtl* batch_engine_results(const BatchEngine* e) {
+  e->by_solve.resize(e->work.size());
+  size_t at = 0;
+  for (const auto& L : e->lanes)
+    for (int j : L->sol) e->by_solve[j] = e->res[at++];
+  return e->by_solve.data();
+}
 
 long long batch_engine_kernels(const BatchEngine* e) {
   long long k = e->k_fixed;
+  size_t at = 0;
   for (const auto& L : e->lanes) {
     int passes = 0;
-    for (int j : L->sol) passes = std::max(passes, e->res[j].iters);
+    for (size_t i = 0; i < L->sol.size(); ++i) passes = std::max(passes, e->res[at++].iters);
     k += (long long)passes * L->k_body;
   }
   return k;

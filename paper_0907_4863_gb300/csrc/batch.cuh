@@ -49,7 +49,7 @@ BatchEngine* batch_engine_build(saamg_hierarchy* const* hs, const double* const*
                                 cudaStream_t (*stream_of)(int));
 // Enqueues one run of the batch on s (gather, PCG of every solve, scatter).
 void batch_engine_launch(BatchEngine* e, cudaStream_t s);
-// Every solve's CG scalars after the last run (pinned host memory; valid once s is idle).
+// Every solve's CG scalars after the last run (call once s is idle; valid until the next call).
 const PcgCtl* batch_engine_results(const BatchEngine* e);
 // Kernels the last run executed.
 long long batch_engine_kernels(const BatchEngine* e);

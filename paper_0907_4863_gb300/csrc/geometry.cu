@@ -576,20 +576,16 @@ __global__ void fill_table_k(const LineInfo* __restrict__ lines, const int2* __r
   }
 }
 
-// Box -> compact right-hand side and initial guess.
-__global__ void gather_k(GeomParams g, const LineInfo* __restrict__ lines,
-                         const int2* __restrict__ chunks, int nchunks,
-                         const double* __restrict__ scale, const double* __restrict__ rho,
-                         const double* __restrict__ phi0, double* __restrict__ bhat,
-                         double* __restrict__ xhat) {
-  int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (c >= nchunks) return;
-  int2 ch = chunks[c];
+// Box -> compact right-hand side and initial guess, one row of a chunk; the row, or -1.
+__device__ __forceinline__ int gather_row(const GeomParams& g, const LineInfo* __restrict__ lines,
+                                          int2 ch, int lane, const double* __restrict__ scale,
+                                          const double* __restrict__ rho,
+                                          const double* __restrict__ phi0,
+                                          double* __restrict__ bhat, double* __restrict__ xhat) {
   int L = ch.x;
   LineInfo me = lines[L];
   int i = me.lo + ch.y + lane;
-  if (i > me.hi) return;
+  if (i > me.hi) return -1;
   int row = me.start + ch.y + lane;
   int k = L / g.ny;
   size_t box = (size_t)i + (size_t)g.nx * (size_t)L;
@@ -598,24 +594,61 @@ __global__ void gather_k(GeomParams g, const LineInfo* __restrict__ lines,
   double si = scale[row];
   bhat[row] = si * (bf * rho[box]);
   if (xhat) xhat[row] = phi0 ? phi0[box] / si : 0.0;
+  return row;
+}
+
+__global__ void gather_k(GeomParams g, const LineInfo* __restrict__ lines,
+                         const int2* __restrict__ chunks, int nchunks,
+                         const double* __restrict__ scale, const double* __restrict__ rho,
+                         const double* __restrict__ phi0, double* __restrict__ bhat,
+                         double* __restrict__ xhat) {
+  int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  int lane = threadIdx.x & 31;
+  if (c >= nchunks) return;
+  gather_row(g, lines, chunks[c], lane, scale, rho, phi0, bhat, xhat);
+}
+
+__global__ void __launch_bounds__(256) bgather_k(const BoxTask* __restrict__ tasks,
+                                                 const int4* __restrict__ wbs) {
+  const int4 B = wbs[blockIdx.x];
+  const BoxTask& k = tasks[B.x];
+  const int lane = threadIdx.x & 31;
+  for (int u = B.y + (threadIdx.x >> 5); u < B.z; u += blockDim.x >> 5) {
+    const int row = gather_row(k.g, k.lines, k.chunks[u], lane, k.scale, k.rho, k.phi, k.bhat,
+                               k.xhat);
+    if (row >= 0) k.p[row] = 0.0;
+  }
+}
+
+// The scaled-back unknown of box node b, 0 outside its line's run.
+__device__ __forceinline__ double scatter_node(int nx, const LineInfo* __restrict__ lines,
+                                               const double* __restrict__ scale,
+                                               const double* __restrict__ xhat, size_t b) {
+  const int L = (int)(b / (size_t)nx);
+  const int i = (int)(b - (size_t)L * nx);
+  const LineInfo me = lines[L];
+  if (i < me.lo || i > me.hi) return 0.0;
+  const int row = me.start + (i - me.lo);
+  return scale[row] * xhat[row];
 }
 
 // Every node of the box: the scaled-back unknown on its line run, 0 elsewhere (one pass that
 // writes each element once, so phi may be a box array in device or in pinned host memory).
-__global__ void scatter_full_k(const GeomParams g, const LineInfo* __restrict__ lines,
+__global__ void scatter_full_k(int nx, const LineInfo* __restrict__ lines,
                                const double* __restrict__ scale, const double* __restrict__ xhat,
                                size_t nbox, double* __restrict__ phi) {
   for (size_t b = blockIdx.x * (size_t)blockDim.x + threadIdx.x; b < nbox;
-       b += (size_t)gridDim.x * blockDim.x) {
-    const int L = (int)(b / (size_t)g.nx);
-    const int i = (int)(b - (size_t)L * g.nx);
-    const LineInfo me = lines[L];
-    double v = 0.0;
-    if (i >= me.lo && i <= me.hi) {
-      const int row = me.start + (i - me.lo);
-      v = scale[row] * xhat[row];
-    }
-    phi[b] = v;
+       b += (size_t)gridDim.x * blockDim.x)
+    phi[b] = scatter_node(nx, lines, scale, xhat, b);
+}
+
+__global__ void __launch_bounds__(256) bscatter_k(const BoxTask* __restrict__ tasks,
+                                                  const int4* __restrict__ wbs) {
+  const int4 B = wbs[blockIdx.x];
+  const BoxTask& k = tasks[B.x];
+  for (int u = B.y; u < B.z; ++u) {
+    const size_t b = (size_t)u * 256 + threadIdx.x;
+    if (b < k.nbox) k.phi[b] = scatter_node(k.g.nx, k.lines, k.scale, k.xhat, b);
   }
 }
 
@@ -1086,7 +1119,19 @@ void scatter_solution(const OperatorData& op, const double* xhat, double* phi, c
   if (nbox == 0) return;
   const size_t need = (nbox + 255) / 256;
   const int blocks = (int)(need < (size_t)sm_count() * 16 ? need : (size_t)sm_count() * 16);
-  scatter_full_k<<<blocks, 256, 0, s>>>(op.g, op.lines.p, op.scale.p, xhat, nbox, phi);
+  scatter_full_k<<<blocks, 256, 0, s>>>(op.g.nx, op.lines.p, op.scale.p, xhat, nbox, phi);
+  SAAMG_LAUNCH();
+}
+
+void batched_gather(const BoxTask* tasks, const int4* wbs, int nwb, cudaStream_t s) {
+  if (nwb <= 0) return;
+  bgather_k<<<nwb, 256, 0, s>>>(tasks, wbs);
+  SAAMG_LAUNCH();
+}
+
+void batched_scatter(const BoxTask* tasks, const int4* wbs, int nwb, cudaStream_t s) {
+  if (nwb <= 0) return;
+  bscatter_k<<<nwb, 256, 0, s>>>(tasks, wbs);
   SAAMG_LAUNCH();
 }
 

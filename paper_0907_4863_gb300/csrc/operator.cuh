@@ -66,6 +66,24 @@ void stencil_diag_inverse(const OperatorData& op, double* invd, float* invd32, c
 // xhat (compact) -> phi (box) = s_i * xhat at unknowns, 0 elsewhere
 void scatter_solution(const OperatorData& op, const double* xhat, double* phi, cudaStream_t s);
 
+// gather_rhs (with phi as the initial guess; p = 0 as well) and scatter_solution of many solves:
+// one launch over work blocks (task, first unit, end unit).  A unit is a chunk (gather) or 256 box
+// nodes (scatter); every node is computed as in the one-solve launches.
+struct BoxTask {
+  GeomParams g;
+  const LineInfo* lines;
+  const int2* chunks;
+  const double* scale;
+  const double* rho;
+  double* phi;
+  double* bhat;
+  double* xhat;
+  double* p;
+  size_t nbox;
+};
+void batched_gather(const BoxTask* tasks, const int4* wbs, int nwb, cudaStream_t s);
+void batched_scatter(const BoxTask* tasks, const int4* wbs, int nwb, cudaStream_t s);
+
 // E = -grad phi on the box (phi and E box arrays; E is 0 outside the unknowns)
 void field_gradient(const OperatorData& op, const double* phi, double* ex, double* ey,
                     double* ez, cudaStream_t s);

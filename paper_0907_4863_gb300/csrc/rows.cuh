@@ -84,6 +84,83 @@ __device__ __forceinline__ void csr_group_row(int row, bool active, int gl,
   }
 }
 
+// NR <= G rows of a group at a time, as csr_group_row computes each: the rows' bounds, the first
+// two entries of every lane, their x and the update's operands are loaded for all rows before the
+// first is summed, and lane q of the group applies MODE to row q (the butterfly leaves the same
+// sum in every lane).  A warp that takes many short rows of many matrices waits for one chain of
+// loads instead of NR (each row is a lane's entry or two, then the shuffles).
+template <class TV, class TM, int G, int MODE, int NR>
+__device__ __forceinline__ void csr_group_rows(const int row[NR], const bool active[NR], int gl,
+                                               const int* __restrict__ rowptr,
+                                               const int* __restrict__ col,
+                                               const TM* __restrict__ val,
+                                               const TV* __restrict__ x, TV* __restrict__ y,
+                                               const TV* __restrict__ b, TV* __restrict__ d,
+                                               const TV* __restrict__ invd, TV c1, TV c2) {
+  static_assert(NR <= G, "a lane per row");
+  int p[NR], p1[NR], er = -1;
+#pragma unroll
+  for (int q = 0; q < NR; ++q) {
+    p[q] = active[q] ? rowptr[row[q]] + gl : 0;
+    p1[q] = active[q] ? rowptr[row[q] + 1] : 0;
+    if (gl == q && active[q]) er = row[q];
+  }
+  TV bv = TV(0), dv = TV(0), iv = TV(0), xv = TV(0);
+  if (er >= 0) {
+    if (MODE == CSR_RESID || MODE == CSR_CHEB) bv = b[er];
+    if (MODE == CSR_CHEB) {
+      iv = invd[er];
+      xv = x[er];
+      if (c1 != TV(0)) dv = d[er];
+    }
+    if (MODE == CSR_ADD) xv = y[er];
+  }
+  int k[NR][2];
+  TV a[NR][2], acc[NR];
+#pragma unroll
+  for (int q = 0; q < NR; ++q)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const bool on = p[q] + e * G < p1[q];
+      k[q][e] = on ? col[p[q] + e * G] : -1;
+      a[q][e] = on ? (TV)ldv(val, p[q] + e * G) : TV(0);
+    }
+#pragma unroll
+  for (int q = 0; q < NR; ++q) {
+    TV xe[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) xe[e] = k[q][e] >= 0 ? x[k[q][e]] : TV(0);
+    acc[q] = TV(0);
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (k[q][e] >= 0) acc[q] += a[q][e] * xe[e];
+  }
+#pragma unroll
+  for (int q = 0; q < NR; ++q)
+    for (int e = p[q] + 2 * G; e < p1[q]; e += G) acc[q] += (TV)ldv(val, e) * x[col[e]];
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < NR; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o, G);
+  TV s = acc[0];
+#pragma unroll
+  for (int q = 1; q < NR; ++q)
+    if (gl == q) s = acc[q];
+  if (er < 0) return;
+  if (MODE == CSR_SPMV) {
+    y[er] = s;
+  } else if (MODE == CSR_RESID) {
+    y[er] = bv - s;
+  } else if (MODE == CSR_ADD) {
+    y[er] = xv + s;
+  } else {  // CSR_CHEB
+    const TV t = iv * (bv - s);
+    const TV w = (c1 == TV(0)) ? c2 * t : fma(c2, t, c1 * dv);
+    d[er] = w;
+    y[er] = xv + w;
+  }
+}
+
 // --- CSR, a thread per short row ------------------------------------------------------------
 constexpr int kShortWin = 6;
 
@@ -321,42 +398,55 @@ __device__ __forceinline__ double update_block(int blk, int n, double a, double*
 }
 
 // --- the same blocks emulated by one warp ---------------------------------------------------
-// A warp can stand in for a block of kRedThreads = 8 x 32 threads: lane l runs the loops of
-// the block's threads 32 w + l (w = 0..7, the block's warps) one after the other with its own
-// accumulator each, every accumulator is reduced by the warp's xor tree (the block's per-warp
-// reduction), and the eight sums are added in warp order (the block's final loop).  The
-// result has the bits of the block's partial, in every lane, without shared memory or
-// barriers, and eight of these run side by side in a block.
+// A warp can stand in for a block of kRedThreads = 8 x 32 threads: lane l holds the accumulators
+// of the block's threads 32 w + l (w = 0..7, the block's warps), every accumulator is reduced by
+// the warp's xor tree (the block's per-warp reduction), and the eight sums are added in warp
+// order (the block's final loop).  The result has the bits of the block's partial, in every
+// lane, without shared memory or barriers, and eight of these run side by side in a block.
 constexpr int kVirtWarps = kRedThreads / 32;
 
-__device__ __forceinline__ double warp_tree(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// The eight xor trees (16, 8, 4, 2, 1) at once: at the first three levels a lane keeps half of its
+// accumulators and passes the other half on, so a tree level is 4, 2, 1, 1, 1 additions for all
+// eight instead of 8 each (an FP64 instruction holds a quarter of the SM for 64 clocks, whatever
+// its lanes do); each sum adds the same two numbers as the plain tree.
+__device__ __forceinline__ double warp_tree8(const double v[kVirtWarps], int lane) {
+  double u[4], w[2];
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    u[q] = (h16 ? v[q + 4] : v[q]) + __shfl_xor_sync(0xffffffffu, h16 ? v[q] : v[q + 4], 16);
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    w[q] = (h8 ? u[q + 2] : u[q]) + __shfl_xor_sync(0xffffffffu, h8 ? u[q] : u[q + 2], 8);
+  double s = (h4 ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, h4 ? w[0] : w[1], 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  double t = 0.0;
+#pragma unroll
+  for (int a = 0; a < kVirtWarps; ++a)
+    t += __shfl_sync(0xffffffffu, s, ((a >> 2) & 1) * 16 + ((a >> 1) & 1) * 8 + (a & 1) * 4);
+  return t;
+}
+
+// f(i, w) for every element i of the block's threads 32 w + lane, in each thread's order
+template <class F>
+__device__ __forceinline__ void virt_block(int blk, int n, int lane, F&& f) {
+  for (int base = blk * kRedThreads; base < n; base += kRedBlocks * kRedThreads) {
+#pragma unroll
+    for (int w = 0; w < kVirtWarps; ++w) {
+      if (base + 32 * w >= n) break;  // uniform
+      const int i = base + 32 * w + lane;
+      if (i < n) f(i, w);
+    }
+  }
 }
 
 template <class TA, class TB>
 __device__ __forceinline__ double dot_block_warp(int blk, int n, const TA* __restrict__ a,
                                                  const TB* __restrict__ b, int lane) {
-  const int st = kRedBlocks * kRedThreads;
-  double t = 0.0;
-#pragma unroll
-  for (int w = 0; w < kVirtWarps; ++w) {
-    double acc = 0.0;
-    int i = blk * kRedThreads + 32 * w + lane;
-    for (; i + 3 * st < n; i += 4 * st) {
-      const double a0 = (double)a[i], a1 = (double)a[i + st], a2 = (double)a[i + 2 * st],
-                   a3 = (double)a[i + 3 * st];
-      const double b0 = (double)b[i], b1 = (double)b[i + st], b2 = (double)b[i + 2 * st],
-                   b3 = (double)b[i + 3 * st];
-      acc += a0 * b0;
-      acc += a1 * b1;
-      acc += a2 * b2;
-      acc += a3 * b3;
-    }
-    for (; i < n; i += st) acc += (double)a[i] * (double)b[i];
-    t += warp_tree(acc);
-  }
-  return t;
+  double acc[kVirtWarps] = {};
+  virt_block(blk, n, lane, [&](int i, int w) { acc[w] += (double)a[i] * (double)b[i]; });
+  return warp_tree8(acc, lane);
 }
 
 template <class TZ>
@@ -364,29 +454,14 @@ __device__ __forceinline__ void dot2_block_warp(int blk, int n, const double* __
                                                 const TZ* __restrict__ z,
                                                 const double* __restrict__ q, int lane,
                                                 double& t1, double& t2) {
-  const int st = kRedBlocks * kRedThreads;
-  t1 = 0.0;
-  t2 = 0.0;
-#pragma unroll
-  for (int w = 0; w < kVirtWarps; ++w) {
-    double a1 = 0.0, a2 = 0.0;
-    int i = blk * kRedThreads + 32 * w + lane;
-    for (; i + st < n; i += 2 * st) {
-      const double z0 = (double)z[i], z1 = (double)z[i + st];
-      const double r0 = r[i], r1 = r[i + st], q0 = q[i], q1 = q[i + st];
-      a1 += r0 * z0;
-      a2 += z0 * q0;
-      a1 += r1 * z1;
-      a2 += z1 * q1;
-    }
-    for (; i < n; i += st) {
-      const double zi = (double)z[i];
-      a1 += r[i] * zi;
-      a2 += zi * q[i];
-    }
-    t1 += warp_tree(a1);
-    t2 += warp_tree(a2);
-  }
+  double a1[kVirtWarps] = {}, a2[kVirtWarps] = {};
+  virt_block(blk, n, lane, [&](int i, int w) {
+    const double zi = (double)z[i];
+    a1[w] += r[i] * zi;
+    a2[w] += zi * q[i];
+  });
+  t1 = warp_tree8(a1, lane);
+  t2 = warp_tree8(a2, lane);
 }
 
 __device__ __forceinline__ double update_block_warp(int blk, int n, double a,
@@ -395,20 +470,15 @@ __device__ __forceinline__ double update_block_warp(int blk, int n, double a,
                                                     const double* __restrict__ p,
                                                     const double* __restrict__ q,
                                                     float* __restrict__ r32, int lane) {
-  double t = 0.0;
-#pragma unroll
-  for (int w = 0; w < kVirtWarps; ++w) {
-    double acc = 0.0;
-    for (int i = blk * kRedThreads + 32 * w + lane; i < n; i += kRedBlocks * kRedThreads) {
-      x[i] = x[i] + a * p[i];
-      double ri = r[i] - a * q[i];
-      r[i] = ri;
-      if (r32) r32[i] = (float)ri;
-      acc += ri * ri;
-    }
-    t += warp_tree(acc);
-  }
-  return t;
+  double acc[kVirtWarps] = {};
+  virt_block(blk, n, lane, [&](int i, int w) {
+    x[i] = x[i] + a * p[i];
+    const double ri = r[i] - a * q[i];
+    r[i] = ri;
+    if (r32) r32[i] = (float)ri;
+    acc[w] += ri * ri;
+  });
+  return warp_tree8(acc, lane);
 }
 
 }  // namespace rows

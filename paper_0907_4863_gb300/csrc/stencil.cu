@@ -340,12 +340,15 @@ __global__ void __launch_bounds__(256, 4) bstencil_k(const StTask<T>* __restrict
 // q = A p with p'q partials, FP64: every (task t, block b) pair computes block b of the
 // one-solve launch (kRedBlocks blocks of 8 warps, one chunk per warp step) for task t,
 // emulated by one warp: lane l runs the rows of lane l of the block's warps w = 0..7 in turn,
-// each warp's sum of its own accumulator by the xor tree, the eight added in warp order --
-// the bits of the one-solve partial.  A pair without chunks stores 0.
+// leaves each warp's accumulator in shared memory, and the eight are reduced together by the
+// block's trees (rows::warp_tree8) -- the bits of the one-solve partial.  A pair without chunks
+// stores 0.
 __global__ void __launch_bounds__(256) bstencil_dot_k(const StTask<double>* __restrict__ tasks,
                                                       int ntasks) {
+  constexpr int wpb = rows::kVirtWarps;
+  __shared__ double sacc[8][wpb][32];
   const int lane = threadIdx.x & 31;
-  constexpr int wpb = 8;
+  double(*mine)[32] = sacc[threadIdx.x >> 5];
   const int nw = kRedBlocks * wpb;
   const long long npairs = (long long)ntasks * kRedBlocks;
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(256) bstencil_dot_k(const StTask<double>* __re
       if (lane == 0) k.part[b] = 0.0;
       continue;
     }
-    double t = 0.0;
+#pragma unroll 2
     for (int w = 0; w < wpb; ++w) {
       double dacc = 0.0;
       for (int c = b * wpb + w; c < nch; c += nw) {
@@ -371,8 +374,12 @@ __global__ void __launch_bounds__(256) bstencil_dot_k(const StTask<double>* __re
           stencil_row<double, ST_SPMV_DOT, true>(k.S, c, lane, k.x, k.y, k.b, k.d, k.c1, k.c2,
                                                  k.c2i0, dacc, k.agg);
       }
-      t += rows::warp_tree(dacc);
+      mine[w][lane] = dacc;  // read back by the same lane
     }
+    double v[wpb];
+#pragma unroll
+    for (int w = 0; w < wpb; ++w) v[w] = mine[w][lane];
+    const double t = rows::warp_tree8(v, lane);
     if (lane == 0) k.part[b] = t;
   }
 }
