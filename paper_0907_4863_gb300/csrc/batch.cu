@@ -33,7 +33,7 @@ namespace saamg {
 namespace {
 
 constexpr int kWarps = 8;         // warps per block of the batched kernels
-constexpr int kWarpUnits = 4;     // warp-sized units per warp and work block, at least
+constexpr int kWarpUnits = 4;     // warp-sized units per warp and work block
 constexpr int kBlockUnits = 4;    // 256-element units per work block (vector kernels)
 constexpr int kMaxLanes = 8;      // concurrent sub-batches of a batch
 constexpr int kLaneSolves = 32;   // solves per lane (about)
@@ -71,6 +71,7 @@ struct VTask {  // the CG recursion of one solve
   double* part0;
   double* part1;
   double* part2;
+  double* partq;  // p'q, by the chunks of A p (its last block may hold rows where a vector's has none)
   int rule, maxit;
   double rtol;
 };
@@ -192,40 +193,32 @@ __global__ void __launch_bounds__(256, 5) bcopy_k(const MTask* __restrict__ task
 // --- CG vector kernels ----------------------------------------------------------------------
 // Every (task t, block b) pair computes block b of the one-solve grid (kRedBlocks blocks of
 // kRedThreads) for task t, emulated by one warp (rows::*_block_warp), so each partial has the
-// one-solve bits; warps take pairs in turn.  A pair past the vector's end only stores its
-// partial, 0 (what the one-solve block sums).
+// one-solve bits; warps take pairs in turn.  The list holds the blocks with elements only (the
+// partials of the others stay 0, what the one-solve block sums): over all blocks of all tasks in
+// turn, the warps' stride was a multiple of kRedBlocks, and the warps of the last blocks, which a
+// vector of fewer than 155,648 elements does not reach, had no work at all.
 #define SAAMG_WARP_PAIRS                                                          \
   const int lane = threadIdx.x & 31;                                              \
-  const long long npairs = (long long)ntasks * kRedBlocks;                        \
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);              \
-  for (long long pr = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;    \
-       pr < npairs; pr += nwarps) {                                               \
-    const VTask& k = tasks[pr / kRedBlocks];                                      \
-    const int b = (int)(pr % kRedBlocks);                                         \
+  const int nwarps = gridDim.x * (blockDim.x >> 5);                               \
+  for (int pr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs; pr += nwarps) { \
+    const int2 tb = pairs[pr];                                                    \
+    const VTask& k = tasks[tb.x];                                                 \
+    const int b = tb.y;                                                           \
     if (!*k.go) continue;
 
 template <class TZ>
-__global__ void __launch_bounds__(256) bdot_rz_k(const VTask* __restrict__ tasks, int ntasks) {
+__global__ void __launch_bounds__(256) bdot_rz_k(const VTask* __restrict__ tasks,
+                                                 const int2* __restrict__ pairs, int npairs) {
   SAAMG_WARP_PAIRS
-    if (b * kRedThreads >= k.n) {
-      if (lane == 0) k.part0[b] = 0.0;
-      continue;
-    }
     const double t = rows::dot_block_warp<double, TZ>(b, k.n, k.r, (const TZ*)k.z, lane);
     if (lane == 0) k.part0[b] = t;
   }
 }
 
 template <class TZ>
-__global__ void __launch_bounds__(256) bdot2_k(const VTask* __restrict__ tasks, int ntasks) {
+__global__ void __launch_bounds__(256) bdot2_k(const VTask* __restrict__ tasks,
+                                               const int2* __restrict__ pairs, int npairs) {
   SAAMG_WARP_PAIRS
-    if (b * kRedThreads >= k.n) {
-      if (lane == 0) {
-        k.part0[b] = 0.0;
-        k.part2[b] = 0.0;
-      }
-      continue;
-    }
     double t1, t2;
     rows::dot2_block_warp<TZ>(b, k.n, k.r, (const TZ*)k.z, k.q, lane, t1, t2);
     if (lane == 0) {
@@ -235,12 +228,9 @@ __global__ void __launch_bounds__(256) bdot2_k(const VTask* __restrict__ tasks, 
   }
 }
 
-__global__ void __launch_bounds__(256) bupdate_k(const VTask* __restrict__ tasks, int ntasks) {
+__global__ void __launch_bounds__(256) bupdate_k(const VTask* __restrict__ tasks,
+                                                 const int2* __restrict__ pairs, int npairs) {
   SAAMG_WARP_PAIRS
-    if (b * kRedThreads >= k.n) {
-      if (lane == 0) k.part1[b] = 0.0;
-      continue;
-    }
     const double t =
         rows::update_block_warp(b, k.n, k.ctl->alpha, k.x, k.r, k.p, k.q, k.r32, lane);
     if (lane == 0) k.part1[b] = t;
@@ -251,34 +241,28 @@ __global__ void __launch_bounds__(256) bupdate_k(const VTask* __restrict__ tasks
 // copy of r (the prologue), or q'q of the recomputed residual into part0 (the epilogue).
 enum Square { SQ_B, SQ_R, SQ_Q };
 
-__global__ void __launch_bounds__(256) bsquare_k(const VTask* __restrict__ tasks, int ntasks,
+__global__ void __launch_bounds__(256) bsquare_k(const VTask* __restrict__ tasks,
+                                                 const int2* __restrict__ pairs, int npairs,
                                                  int which) {
   const int lane = threadIdx.x & 31;
-  const long long npairs = (long long)ntasks * kRedBlocks;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long pr = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs;
-       pr += nwarps) {
-    const VTask& k = tasks[pr / kRedBlocks];
-    const int b = (int)(pr % kRedBlocks);
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  for (int pr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs; pr += nwarps) {
+    const int2 tb = pairs[pr];
+    const VTask& k = tasks[tb.x];
+    const int b = tb.y;
     const double* v = which == SQ_B ? k.bhat : (which == SQ_R ? k.r : k.q);
     double* part = which == SQ_B ? k.part2 : (which == SQ_R ? k.part1 : k.part0);
-    double t = 0.0;
-    if (b * kRedThreads < k.n) {
-      float* copy = which == SQ_R ? k.r32 : nullptr;
-      if (copy)
-        rows::virt_block(b, k.n, lane, [&](int i, int) { copy[i] = (float)v[i]; });
-      t = rows::dot_block_warp<double, double>(b, k.n, v, v, lane);
-    }
+    float* copy = which == SQ_R ? k.r32 : nullptr;
+    if (copy) rows::virt_block(b, k.n, lane, [&](int i, int) { copy[i] = (float)v[i]; });
+    const double t = rows::dot_block_warp<double, double>(b, k.n, v, v, lane);
     if (lane == 0) part[b] = t;
   }
 }
 
 int resident_blocks(const void* kernel);
 
-inline int grid_pairs(int ntasks, const void* kernel) {  // blocks of 8 warps, a warp per pair
-  return (int)std::max<long long>(
-      1, std::min<long long>(((long long)ntasks * kRedBlocks + 7) / 8,
-                             (long long)sm_count() * resident_blocks(kernel)));
+inline int grid_pairs(int npairs, const void* kernel) {  // blocks of 8 warps, a warp per pair
+  return std::max(1, std::min((npairs + 7) / 8, sm_count() * resident_blocks(kernel)));
 }
 
 // p = z + beta p; a unit is 256 elements
@@ -363,7 +347,7 @@ __global__ void __launch_bounds__(kRedThreads) balpha_k(const VTask* __restrict_
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
   PcgCtl* ctl = k.ctl;
-  const double pq = rows::sum_fixed(k.part0);
+  const double pq = rows::sum_fixed(k.partq);
   if (threadIdx.x == 0) {
     ctl->pq = pq;
     double a = ctl->rz / pq;
@@ -535,15 +519,6 @@ void work_blocks(const std::vector<int>& units, int per, std::vector<int4>& out)
       out.push_back(make_int4((int)t, u, std::min(units[t], u + per), 0));
 }
 
-// Warp-sized units per work block: about ten blocks per SM (each costs a task load and two
-// barriers), 32 to 128 units.
-int units_per_block(const std::vector<int>& units) {
-  long long total = 0;
-  for (int u : units) total += u;
-  const long long step = kWarps * kWarpUnits, want = total / (10LL * sm_count());
-  return (int)std::max(step, std::min(4 * step, (want + step - 1) / step * step));
-}
-
 // --- planning ---------------------------------------------------------------------------------
 enum Phase { P_PRE = 0, P_RESID, P_RESTRICT, P_COARSE, P_PROLONG, P_POST, P_COPY };
 
@@ -561,7 +536,7 @@ struct SolveWork {
   saamg_hierarchy* h = nullptr;
   Buf<double> bhat, xhat, r, z, p, q;
   Buf<float> z32, r32;
-  Buf<double> part0, part1, part2;
+  Buf<double> part;       // part0, part1, part2, partq; 0 in the blocks that hold nothing
   PcgCtl* ctl = nullptr;  // in its lane's array
   std::vector<Buf<double>> dx0, dx1, db, dd, dr;
   std::vector<Buf<float>> fx0, fx1, fb, fd, fr;
@@ -838,6 +813,12 @@ struct Lane {
   Buf<int4> vsub_off;          // per subset: work blocks of 256-element units (direction)
   std::vector<int> vsub_units; // work blocks of each subset
   std::vector<size_t> vsub_offpos;  // first work block of each subset
+  // (task, block) pairs of the reductions: all solves, then each subset, then A p
+  Buf<int2> pairs;
+  int n_all = 0, n_dot = 0;
+  std::vector<int> n_sub;
+  size_t dot_off = 0;
+  std::vector<size_t> sub_off;
   Buf<int4> vall_off;          // all solves of the lane: work blocks (zero)
   int vall_units = 0;
   Buf<StTask<double>> dot_tasks;  // A p with p'Ap partials
@@ -891,9 +872,8 @@ void alloc_work(SolveWork& w, cudaStream_t s) {
   } else {
     w.z.alloc(n, s);
   }
-  w.part0.alloc(kRedBlocks, s);
-  w.part1.alloc(kRedBlocks, s);
-  w.part2.alloc(kRedBlocks, s);
+  w.part.alloc(4 * kRedBlocks, s);
+  SAAMG_CUDA(cudaMemsetAsync(w.part.p, 0, w.part.bytes(), s));
   const int nl = (int)h->lev.size();
   if (mx) {
     w.fx0.resize(nl);
@@ -1003,7 +983,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       units.push_back(o.units);
     }
     std::vector<int4> wb;
-    work_blocks(units, units_per_block(units), wb);
+    work_blocks(units, kWarps * kWarpUnits, wb);
     g.nwb = (int)wb.size();
     align(16);
     g.wb_off = host.size();
@@ -1031,9 +1011,10 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
     t.q = w.q.p;
     t.z = mx ? (const void*)w.z32.p : (const void*)w.z.p;
     t.r32 = mx ? w.r32.p : nullptr;
-    t.part0 = w.part0.p;
-    t.part1 = w.part1.p;
-    t.part2 = w.part2.p;
+    t.part0 = w.part.p;
+    t.part1 = w.part.p + kRedBlocks;
+    t.part2 = w.part.p + 2 * kRedBlocks;
+    t.partq = w.part.p + 3 * kRedBlocks;
     t.rule = h->prm.beta_rule;
     t.maxit = h->prm.maxit;
     t.rtol = rtol;
@@ -1070,6 +1051,28 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
     SAAMG_CUDA(cudaMemcpyAsync(L.vsub_off.p, wbs.data(), sizeof(int4) * wbs.size(),
                                cudaMemcpyHostToDevice, s));
   {
+    std::vector<int2> pr;
+    auto blocks = [](int n) { return std::min(kRedBlocks, (n + kRedThreads - 1) / kRedThreads); };
+    auto add = [&](int task, int nb) {
+      for (int b = 0; b < nb; ++b) pr.push_back(make_int2(task, b));
+    };
+    for (int i = 0; i < m; ++i) add(i, blocks(vt[i].n));
+    L.n_all = (int)pr.size();
+    for (int kind : L.vsub_kind) {
+      L.sub_off.push_back(pr.size());
+      for (size_t q = 0; q < L.vsets[kind].size(); ++q) add((int)q, blocks(vt[L.vsets[kind][q]].n));
+      L.n_sub.push_back((int)(pr.size() - L.sub_off.back()));
+    }
+    L.dot_off = pr.size();
+    for (int i = 0; i < m; ++i)
+      add(i, stencil_dot_blocks(work[L.sol[i]]->h->op->d.view<double>()));
+    L.n_dot = (int)(pr.size() - L.dot_off);
+    L.pairs.alloc(std::max<size_t>(pr.size(), 1), s);
+    if (!pr.empty())
+      SAAMG_CUDA(cudaMemcpyAsync(L.pairs.p, pr.data(), sizeof(int2) * pr.size(),
+                                 cudaMemcpyHostToDevice, s));
+  }
+  {
     std::vector<int> units;
     for (int i = 0; i < m; ++i) units.push_back((vt[i].n + 255) / 256);
     std::vector<int4> all;
@@ -1088,7 +1091,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       t.go = L.go.p + i;
       t.x = w.p.p;
       t.y = w.q.p;
-      t.part = w.part0.p;
+      t.part = w.part.p + 3 * kRedBlocks;
       dt[i] = t;
     }
     L.dot_tasks.alloc(m, s);
@@ -1127,11 +1130,11 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       ur.push_back(stencil_units<double>(r.S));
     }
     std::vector<int4> wb;
-    work_blocks(ug, units_per_block(ug), wb);
+    work_blocks(ug, kWarps * kWarpUnits, wb);
     L.n_gather = (int)wb.size();
     work_blocks(us, kBlockUnits, wb);
     L.n_scatter = (int)wb.size() - L.n_gather;
-    work_blocks(ur, units_per_block(ur), wb);
+    work_blocks(ur, kWarps * kWarpUnits, wb);
     L.n_resid = (int)wb.size() - L.n_gather - L.n_scatter;
     L.box.alloc(m, s);
     L.res_tasks.alloc(2 * m, s);
@@ -1146,9 +1149,8 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
 
 // Partials of a square of every solve of the lane.
 void lane_square(Lane& L, Square which, cudaStream_t s) {
-  const int m = (int)L.sol.size();
-  bsquare_k<<<grid_pairs(m, reinterpret_cast<const void*>(bsquare_k)), 256, 0, s>>>(L.vtasks.p, m,
-                                                                                   which);
+  bsquare_k<<<grid_pairs(L.n_all, reinterpret_cast<const void*>(bsquare_k)), 256, 0, s>>>(
+      L.vtasks.p, L.pairs.p, L.n_all, which);
   SAAMG_LAUNCH();
 }
 
@@ -1190,20 +1192,17 @@ void lane_body(Lane& L, cudaGraphConditionalHandle cond, cudaStream_t s) {
                  reinterpret_cast<const int4*>(L.tasks.p + gr.wb_off), gr.nwb, s);
   for (size_t q = 0; q < L.vsub.size(); ++q) {
     const int kind = L.vsub_kind[q];
-    const int nt = (int)L.vsets[kind].size();
     const VTask* t = L.vsub[q].p;
+    const int2* pr = L.pairs.p + L.sub_off[q];
+    const int np = L.n_sub[q];
     if (kind == 0)
-      bdot_rz_k<double><<<grid_pairs(nt, reinterpret_cast<const void*>(bdot_rz_k<double>)), 256, 0,
-                          s>>>(t, nt);
+      bdot_rz_k<double><<<grid_pairs(np, reinterpret_cast<const void*>(bdot_rz_k<double>)), 256, 0, s>>>(t, pr, np);
     else if (kind == 1)
-      bdot2_k<double><<<grid_pairs(nt, reinterpret_cast<const void*>(bdot2_k<double>)), 256, 0,
-                        s>>>(t, nt);
+      bdot2_k<double><<<grid_pairs(np, reinterpret_cast<const void*>(bdot2_k<double>)), 256, 0, s>>>(t, pr, np);
     else if (kind == 2)
-      bdot_rz_k<float><<<grid_pairs(nt, reinterpret_cast<const void*>(bdot_rz_k<float>)), 256, 0,
-                         s>>>(t, nt);
+      bdot_rz_k<float><<<grid_pairs(np, reinterpret_cast<const void*>(bdot_rz_k<float>)), 256, 0, s>>>(t, pr, np);
     else
-      bdot2_k<float><<<grid_pairs(nt, reinterpret_cast<const void*>(bdot2_k<float>)), 256, 0,
-                       s>>>(t, nt);
+      bdot2_k<float><<<grid_pairs(np, reinterpret_cast<const void*>(bdot2_k<float>)), 256, 0, s>>>(t, pr, np);
     SAAMG_LAUNCH();
   }
   bbeta_k<<<m, kRedThreads, 0, s>>>(L.vtasks.p);
@@ -1220,10 +1219,11 @@ void lane_body(Lane& L, cudaGraphConditionalHandle cond, cudaStream_t s) {
                             256, 0, s>>>(L.vsub[q].p, wb, nwb);
     SAAMG_LAUNCH();
   }
-  batched_stencil_dot(L.dot_tasks.p, m, s);
+  batched_stencil_dot(L.dot_tasks.p, L.pairs.p + L.dot_off, L.n_dot, s);
   balpha_k<<<m, kRedThreads, 0, s>>>(L.vtasks.p);
   SAAMG_LAUNCH();
-  bupdate_k<<<grid_pairs(m, reinterpret_cast<const void*>(bupdate_k)), 256, 0, s>>>(L.vtasks.p, m);
+  bupdate_k<<<grid_pairs(L.n_all, reinterpret_cast<const void*>(bupdate_k)), 256, 0, s>>>(
+      L.vtasks.p, L.pairs.p, L.n_all);
   SAAMG_LAUNCH();
   bcheck_k<<<m, kRedThreads, 0, s>>>(L.vtasks.p);
   SAAMG_LAUNCH();

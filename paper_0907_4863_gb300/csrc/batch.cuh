@@ -32,9 +32,12 @@ int stencil_units(const StencilDev<T>& S);
 // the units.
 template <class T>
 void batched_stencil(int mode, const StTask<T>* tasks, const int4* wbs, int nwb, cudaStream_t s);
-// q = A p with the partials of p'q (FP64 CG product): kRedBlocks blocks per task, the
-// one-solve launch's grid, so every partial has the same bits.
-void batched_stencil_dot(const StTask<double>* tasks, int ntasks, cudaStream_t s);
+// q = A p with the partials of p'q (FP64 CG product): blocks of the one-solve launch's grid of
+// kRedBlocks, so every partial has the same bits; pairs: (task, block) of the blocks with rows,
+// the first stencil_dot_blocks(S) of each task.
+int stencil_dot_blocks(const StencilDev<double>& S);
+void batched_stencil_dot(const StTask<double>* tasks, const int2* pairs, int npairs,
+                         cudaStream_t s);
 
 struct PcgCtl;
 

@@ -341,28 +341,22 @@ __global__ void __launch_bounds__(256, 4) bstencil_k(const StTask<T>* __restrict
 // one-solve launch (kRedBlocks blocks of 8 warps, one chunk per warp step) for task t,
 // emulated by one warp: lane l runs the rows of lane l of the block's warps w = 0..7 in turn,
 // leaves each warp's accumulator in shared memory, and the eight are reduced together by the
-// block's trees (rows::warp_tree8) -- the bits of the one-solve partial.  A pair without chunks
-// stores 0.
+// block's trees (rows::warp_tree8) -- the bits of the one-solve partial.
 __global__ void __launch_bounds__(256) bstencil_dot_k(const StTask<double>* __restrict__ tasks,
-                                                      int ntasks) {
+                                                      const int2* __restrict__ pairs, int npairs) {
   constexpr int wpb = rows::kVirtWarps;
   __shared__ double sacc[8][wpb][32];
   const int lane = threadIdx.x & 31;
   double(*mine)[32] = sacc[threadIdx.x >> 5];
   const int nw = kRedBlocks * wpb;
-  const long long npairs = (long long)ntasks * kRedBlocks;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long pr = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs;
-       pr += nwarps) {
-    const StTask<double>& k = tasks[pr / kRedBlocks];
-    const int b = (int)(pr % kRedBlocks);
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  for (int pr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < npairs; pr += nwarps) {
+    const int2 tb = pairs[pr];
+    const StTask<double>& k = tasks[tb.x];
+    const int b = tb.y;
     if (!*k.go) continue;
     const int nreg = (k.S.nrun + 31) / 32;
     const int nch = nreg + (k.S.ntable + 31) / 32;
-    if (b * wpb >= nch) {
-      if (lane == 0) k.part[b] = 0.0;
-      continue;
-    }
 #pragma unroll 2
     for (int w = 0; w < wpb; ++w) {
       double dacc = 0.0;
@@ -440,15 +434,18 @@ void batched_stencil(int mode, const StTask<T>* tasks, const int4* wbs, int nwb,
 template void batched_stencil<float>(int, const StTask<float>*, const int4*, int, cudaStream_t);
 template void batched_stencil<double>(int, const StTask<double>*, const int4*, int, cudaStream_t);
 
-void batched_stencil_dot(const StTask<double>* tasks, int ntasks, cudaStream_t s) {
-  if (ntasks <= 0) return;
-  const long long pairs = (long long)ntasks * kRedBlocks;
+int stencil_dot_blocks(const StencilDev<double>& S) {
+  return std::min(kRedBlocks, (stencil_units<double>(S) + rows::kVirtWarps - 1) / rows::kVirtWarps);
+}
+
+void batched_stencil_dot(const StTask<double>* tasks, const int2* pairs, int npairs,
+                         cudaStream_t s) {
+  if (npairs <= 0) return;
   int nb = 0;
   SAAMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &nb, reinterpret_cast<const void*>(bstencil_dot_k), 256, 0));
-  const int blocks =
-      (int)std::min<long long>((pairs + 7) / 8, (long long)sm_count() * std::max(nb, 1));
-  bstencil_dot_k<<<blocks, 256, 0, s>>>(tasks, ntasks);
+  const int blocks = std::min((npairs + 7) / 8, sm_count() * std::max(nb, 1));
+  bstencil_dot_k<<<blocks, 256, 0, s>>>(tasks, pairs, npairs);
   SAAMG_LAUNCH();
 }
 
