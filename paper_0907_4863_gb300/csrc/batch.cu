@@ -76,29 +76,17 @@ struct VTask {  // the CG recursion of one solve
   double rtol;
 };
 
-// Copies task t into shared memory (the whole block takes part).
-template <class Task>
-__device__ __forceinline__ void load_task(const Task* __restrict__ tasks, int t, Task& sk) {
-  const int* src = reinterpret_cast<const int*>(tasks + t);
-  int* dst = reinterpret_cast<int*>(&sk);
-  for (int i = threadIdx.x; i < (int)(sizeof(Task) / 4); i += blockDim.x) dst[i] = src[i];
-}
-
-// Every work-block kernel starts a work block the same way: the task into shared memory, and
-// nothing to do when its solve has ended.
+// Every work-block kernel starts a work block the same way: its warps read the task through L1
+// (nothing is staged and no warp waits for another), and nothing is done when its solve has ended.
 #define SAAMG_WORK_BLOCK(TaskT)            \
   const int4 B = wbs[wb];                  \
-  __syncthreads();                         \
-  load_task<TaskT>(tasks, B.x, sk);        \
-  __syncthreads();                         \
-  if (!*sk.go) continue;                   \
-  const TaskT& k = sk;
+  const TaskT& k = tasks[B.x];             \
+  if (!*k.go) continue;
 
 // --- sparse-matrix kernels --------------------------------------------------------------------
 template <class TV, class TM, int G, int MODE>
 __global__ void __launch_bounds__(256, 4) bcsr_k(const MTask* __restrict__ tasks,
                                               const int4* __restrict__ wbs, int nwb) {
-  __shared__ MTask sk;
   const int lane = threadIdx.x & 31, gl = lane % G, warp = threadIdx.x >> 5;
   constexpr int kRows = 32 / G;
   double dacc = 0.0;
@@ -135,7 +123,6 @@ __global__ void __launch_bounds__(256, 4) bcsr_k(const MTask* __restrict__ tasks
 template <class TV, class TM, int MODE>
 __global__ void __launch_bounds__(256, 5) bshort_k(const MTask* __restrict__ tasks,
                                                 const int4* __restrict__ wbs, int nwb) {
-  __shared__ MTask sk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     SAAMG_WORK_BLOCK(MTask)
@@ -151,7 +138,6 @@ __global__ void __launch_bounds__(256, 5) bshort_k(const MTask* __restrict__ tas
 template <class TV, class TM, int MODE, bool REL>
 __global__ void __launch_bounds__(256, 5) bsell_k(const MTask* __restrict__ tasks,
                                                const int4* __restrict__ wbs, int nwb) {
-  __shared__ MTask sk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double dacc = 0.0;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
@@ -167,7 +153,6 @@ __global__ void __launch_bounds__(256, 5) bsell_k(const MTask* __restrict__ task
 template <class TV>
 __global__ void __launch_bounds__(256, 5) bgemv_k(const MTask* __restrict__ tasks,
                                                const int4* __restrict__ wbs, int nwb) {
-  __shared__ MTask sk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     SAAMG_WORK_BLOCK(MTask)
@@ -179,7 +164,6 @@ __global__ void __launch_bounds__(256, 5) bgemv_k(const MTask* __restrict__ task
 template <class T>
 __global__ void __launch_bounds__(256, 5) bcopy_k(const MTask* __restrict__ tasks,
                                                const int4* __restrict__ wbs, int nwb) {
-  __shared__ MTask sk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     SAAMG_WORK_BLOCK(MTask)

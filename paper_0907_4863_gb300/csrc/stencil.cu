@@ -290,30 +290,20 @@ __host__ __device__ constexpr int kChunks() {
   return sizeof(T) == 4 ? 2 : 1;
 }
 
-// Batched form: a block takes one work block (task, first chunk, end chunk) at a time and
-// copies the task into shared memory; its warps take two chunks at a time, as the one-solve
-// FP32 launch does, and apply each exactly as the one-solve launch applies it.
-template <class T>
-__device__ __forceinline__ void load_task(const StTask<T>* __restrict__ tasks, int t,
-                                          StTask<T>& sk) {
-  const int* src = reinterpret_cast<const int*>(tasks + t);
-  int* dst = reinterpret_cast<int*>(&sk);
-  for (int i = threadIdx.x; i < (int)(sizeof(StTask<T>) / 4); i += blockDim.x) dst[i] = src[i];
-}
-
+// Batched form: a block takes one work block (task, first chunk, end chunk) at a time; its warps
+// read the task through L1 and take two chunks at a time, as the one-solve FP32 launch does, and
+// apply each exactly as the one-solve launch applies it.  No warp waits for another: staging the
+// task in shared memory put two barriers and a dependent load before every 1024 rows.
 template <class T, int MODE>
 __global__ void __launch_bounds__(256, 4) bstencil_k(const StTask<T>* __restrict__ tasks,
                                                   const int4* __restrict__ wbs, int nwb) {
-  __shared__ StTask<T> sk;
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   constexpr int K = kChunks<T>();
   double dacc = 0.0;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     const int4 B = wbs[wb];
-    __syncthreads();  // the previous work block is done with sk
-    load_task<T>(tasks, B.x, sk);
-    __syncthreads();
+    const StTask<T>& sk = tasks[B.x];
     if (!*sk.go) continue;  // uniform across the block
     const int nreg = packed_rows<T>() ? (sk.S.nrun + 31) / 32 : sk.S.nchunks;
     for (int c0 = B.y + (threadIdx.x >> 5) * K; c0 < B.z; c0 += wpb * K) {
