@@ -54,6 +54,7 @@ struct MTask {  // a sparse-matrix, coarse-solve or copy operation of one solve
   const void* b;
   void* d;
   const void* invd;
+  void* y2;
   double c1, c2;
 };
 
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(256, 4) bcsr_k(const MTask* __restrict__ tasks
         rows::csr_group_rows<TV, TM, G, MODE, NR>(row, active, gl, k.rowptr, k.col,
                                                   (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
                                                   (const TV*)k.b, (TV*)k.d, (const TV*)k.invd,
-                                                  (TV)k.c1, (TV)k.c2);
+                                                  (TV)k.c1, (TV)k.c2, (TV*)k.y2);
       }
     }
   }
@@ -175,12 +176,12 @@ __global__ void __launch_bounds__(256, 5) bcopy_k(const MTask* __restrict__ task
 }
 
 // --- CG vector kernels ----------------------------------------------------------------------
-// Every (task t, block b) pair computes block b of the one-solve grid (kRedBlocks blocks of
+// Every (task t, block b) pair computes block b of the one-solve grid (kVecBlocks blocks of
 // kRedThreads) for task t, emulated by one warp (rows::*_block_warp), so each partial has the
 // one-solve bits; warps take pairs in turn.  The list holds the blocks with elements only (the
 // partials of the others stay 0, what the one-solve block sums): over all blocks of all tasks in
-// turn, the warps' stride was a multiple of kRedBlocks, and the warps of the last blocks, which a
-// vector of fewer than 155,648 elements does not reach, had no work at all.
+// turn, the warps' stride was a multiple of their number, and the warps of the last blocks, which
+// a short vector does not reach, had no work at all.
 #define SAAMG_WARP_PAIRS                                                          \
   const int lane = threadIdx.x & 31;                                              \
   const int nwarps = gridDim.x * (blockDim.x >> 5);                               \
@@ -283,78 +284,40 @@ __global__ void __launch_bounds__(256, 5) bzero_k(const VTask* __restrict__ task
 // --- CG scalars: a block per task -------------------------------------------------------------
 __global__ void __launch_bounds__(kRedThreads) binit_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
-  PcgCtl* ctl = k.ctl;
-  const double bb = rows::sum_fixed(k.part2);
-  const double rr = rows::sum_fixed(k.part1);
+  const double bb = rows::sum_fixed(k.part2, kVecBlocks);
+  const double rr = rows::sum_fixed(k.part1, kVecBlocks);
   if (threadIdx.x == 0) {
-    ctl->rtol = k.rtol;
-    ctl->bb = bb;
-    ctl->rr = rr;
-    ctl->tol2 = (ctl->rtol * ctl->rtol) * bb;
-    ctl->iters = 0;
-    ctl->breakdown = !(isfinite(bb) && isfinite(rr));
-    ctl->converged = (bb == 0.0) || rr <= ctl->tol2;
-    ctl->rz = 0.0;
-    ctl->alpha = 0.0;
-    ctl->beta = 0.0;
-    *k.go = !ctl->converged && !ctl->breakdown && k.maxit > 0;
+    k.ctl->rtol = k.rtol;
+    *k.go = finish_init(k.ctl, bb, rr, k.maxit);
   }
 }
 
 __global__ void __launch_bounds__(kRedThreads) bstore_true_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
-  const double rr = rows::sum_fixed(k.part0);
+  const double rr = rows::sum_fixed(k.part0, kVecBlocks);
   if (threadIdx.x == 0) k.ctl->rr_true = rr;
 }
 
 __global__ void __launch_bounds__(kRedThreads) bbeta_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
-  PcgCtl* ctl = k.ctl;
-  const double rz = rows::sum_fixed(k.part0);
-  const double zq = k.rule == 1 ? rows::sum_fixed(k.part2) : 0.0;
-  if (threadIdx.x == 0) {
-    double b = 0.0;
-    if (ctl->iters > 0) b = (k.rule == 1) ? (-ctl->alpha * zq) / ctl->rz : rz / ctl->rz;
-    if (!isfinite(b) || !isfinite(rz)) {
-      ctl->breakdown = 1;
-      b = 0.0;
-    }
-    ctl->rz_new = rz;
-    ctl->zq = zq;
-    ctl->beta = b;
-    ctl->rz = rz;
-  }
+  const double rz = rows::sum_fixed(k.part0, kVecBlocks);
+  const double zq = k.rule == 1 ? rows::sum_fixed(k.part2, kVecBlocks) : 0.0;
+  if (threadIdx.x == 0) finish_beta(k.ctl, rz, zq, k.rule);
 }
 
 __global__ void __launch_bounds__(kRedThreads) balpha_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
-  PcgCtl* ctl = k.ctl;
-  const double pq = rows::sum_fixed(k.partq);
-  if (threadIdx.x == 0) {
-    ctl->pq = pq;
-    double a = ctl->rz / pq;
-    if (!(pq != 0.0) || !isfinite(a)) {
-      ctl->breakdown = 1;
-      a = 0.0;
-    }
-    ctl->alpha = a;
-  }
+  const double pq = rows::sum_fixed(k.partq, kRedBlocks);
+  if (threadIdx.x == 0) finish_alpha(k.ctl, pq);
 }
 
 __global__ void __launch_bounds__(kRedThreads) bcheck_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
-  PcgCtl* ctl = k.ctl;
-  const double rr = rows::sum_fixed(k.part1);
-  if (threadIdx.x == 0) {
-    ctl->rr = rr;
-    ctl->iters += 1;
-    if (!isfinite(rr)) ctl->breakdown = 1;
-    ctl->converged = rr <= ctl->tol2;
-    *k.go = !ctl->converged && !ctl->breakdown && ctl->iters < k.maxit;
-  }
+  const double rr = rows::sum_fixed(k.part1, kVecBlocks);
+  if (threadIdx.x == 0) *k.go = finish_check(k.ctl, rr, k.maxit);
 }
 
 // The loop goes on while any solve goes on.
@@ -409,6 +372,7 @@ template <class TV, class TM, int G>
 void launch_csr_g(int mode, const MTask* t, const int4* wbs, int nwb, cudaStream_t s) {
   switch (mode) {
     case CSR_SPMV: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_SPMV>)); break;
+    case CSR_SPMV_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_SPMV_CHEB0>)); break;
     case CSR_RESID: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_RESID>)); break;
     case CSR_CHEB: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_CHEB>)); break;
     case CSR_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_CHEB0>)); break;
@@ -688,7 +652,8 @@ struct Planner {
     }
     const DevCsr& M = restrict_ ? L.R : L.P;
     if (M.n == 0) return;
-    const int mode = restrict_ ? CSR_SPMV : CSR_ADD;
+    const bool first = restrict_ && restriction_smooths(h, l, dbl);
+    const int mode = restrict_ ? (first ? CSR_SPMV_CHEB0 : CSR_SPMV) : CSR_ADD;
     const double avg = M.n ? (double)M.nnz / M.n : 0.0;
     const int g = csr_plan(mode, M.n, avg, dbl);
     o.key.tv = dbl ? 0 : 1;
@@ -700,6 +665,13 @@ struct Planner {
     o.m.val = dbl ? (const void*)M.val.p : (const void*)(restrict_ ? L.R32.p : L.P32.p);
     o.m.x = x;
     o.m.y = y;
+    if (first) {
+      const Level& N = *h->lev[l + 1];
+      o.m.d = WV<T>::d(w, l + 1);
+      o.m.y2 = WV<T>::x0(w, l + 1);
+      o.m.invd = dbl ? (const void*)N.invd.p : (const void*)N.invd32.p;
+      o.m.c2 = (double)(T)N.cheb.c2[0];
+    }
     if (g == 0) {
       o.key.fam = F_SHORT;
       o.units = (M.n + 31) / 32;
@@ -737,7 +709,8 @@ struct Planner {
                                 : SmoothPair<T>(0.0, 0.0, 0.0);
     int cur = pr ? 1 : 0;
     if (pr) pair<T>(P_PRE, 0, ST_PAIR0, b, bufs[cur], nu > 2 ? d : nullptr, sp);
-    else smooth<T>(P_PRE, l, 0, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0]);
+    else if (l == 0 || !restriction_smooths(h, l - 1, sizeof(T) == 8))
+      smooth<T>(P_PRE, l, 0, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0]);
     for (int k = pr ? 2 : 1; k < nu; ++k) {
       smooth<T>(P_PRE, l, k, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
                 (T)L.cheb.c2[k]);
@@ -856,7 +829,7 @@ void alloc_work(SolveWork& w, cudaStream_t s) {
   } else {
     w.z.alloc(n, s);
   }
-  w.part.alloc(4 * kRedBlocks, s);
+  w.part.alloc(3 * kVecBlocks + kRedBlocks, s);
   SAAMG_CUDA(cudaMemsetAsync(w.part.p, 0, w.part.bytes(), s));
   const int nl = (int)h->lev.size();
   if (mx) {
@@ -996,9 +969,9 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
     t.z = mx ? (const void*)w.z32.p : (const void*)w.z.p;
     t.r32 = mx ? w.r32.p : nullptr;
     t.part0 = w.part.p;
-    t.part1 = w.part.p + kRedBlocks;
-    t.part2 = w.part.p + 2 * kRedBlocks;
-    t.partq = w.part.p + 3 * kRedBlocks;
+    t.part1 = w.part.p + kVecBlocks;
+    t.part2 = w.part.p + 2 * kVecBlocks;
+    t.partq = w.part.p + 3 * kVecBlocks;
     t.rule = h->prm.beta_rule;
     t.maxit = h->prm.maxit;
     t.rtol = rtol;
@@ -1036,7 +1009,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
                                cudaMemcpyHostToDevice, s));
   {
     std::vector<int2> pr;
-    auto blocks = [](int n) { return std::min(kRedBlocks, (n + kRedThreads - 1) / kRedThreads); };
+    auto blocks = [](int n) { return std::min(kVecBlocks, (n + kRedThreads - 1) / kRedThreads); };
     auto add = [&](int task, int nb) {
       for (int b = 0; b < nb; ++b) pr.push_back(make_int2(task, b));
     };
@@ -1075,7 +1048,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       t.go = L.go.p + i;
       t.x = w.p.p;
       t.y = w.q.p;
-      t.part = w.part.p + 3 * kRedBlocks;
+      t.part = w.part.p + 3 * kVecBlocks;
       dt[i] = t;
     }
     L.dot_tasks.alloc(m, s);

@@ -338,9 +338,9 @@ static void alloc_pcg_vectors(saamg_hierarchy* h, int n, cudaStream_t s) {
     h->z32.alloc(n, s);
     h->r32.alloc(n, s);
   }
-  h->part0.alloc(kRedBlocks, s);
-  h->part1.alloc(kRedBlocks, s);
-  h->part2.alloc(kRedBlocks, s);
+  h->part0.alloc(kVecBlocks, s);
+  h->part1.alloc(kVecBlocks, s);
+  h->part2.alloc(kVecBlocks, s);
   h->ctl.alloc(1, s);
 }
 
@@ -764,35 +764,57 @@ void level_csr<float>(saamg_hierarchy* h, int l, int mode, const float* x, float
   }
 }
 
+// Values of P_l / R_l and D^-1 of level l in the working precision
 template <class T>
-static void transfer(saamg_hierarchy* h, int l, bool restrict_, const T* x, T* y, cudaStream_t s);
-
+static const T* transfer_values(const Level& L, bool restrict_);
 template <>
-void transfer<double>(saamg_hierarchy* h, int l, bool restrict_, const double* x, double* y,
-                      cudaStream_t s) {
+const double* transfer_values<double>(const Level& L, bool restrict_) {
+  return restrict_ ? L.R.val.p : L.P.val.p;
+}
+template <>
+const float* transfer_values<float>(const Level& L, bool restrict_) {
+  return restrict_ ? L.R32.p : L.P32.p;
+}
+template <class T>
+static const T* level_invd(const Level& L);
+template <>
+const double* level_invd<double>(const Level& L) { return L.invd.p; }
+template <>
+const float* level_invd<float>(const Level& L) { return L.invd32.p; }
+
+// b_{l+1} = R_l r; where level l + 1 smooths, its first step from zero goes with it (x0 and d of
+// that level).  Returns whether it did.
+template <class T>
+static bool restrict_residual(saamg_hierarchy* h, int l, const T* r, cudaStream_t s) {
   Level& L = *h->lev[l];
-  const DevCsr& M = restrict_ ? L.R : L.P;
-  csr_apply<double, double>(restrict_ ? CSR_SPMV : CSR_ADD, M.n, M.rowptr.p, M.col.p, M.val.p,
-                            M.n ? (double)M.nnz / M.n : 0.0, x, y, nullptr, nullptr, nullptr, 0.0,
-                            0.0, nullptr, s, l == 0 ? SAAMG_KT_TRANSFER : SAAMG_KT_TRANSFER_DEEP);
+  Level& N = *h->lev[l + 1];
+  const DevCsr& M = L.R;
+  const double avg = M.n ? (double)M.nnz / M.n : 0.0;
+  const bool first = restriction_smooths(h, l, sizeof(T) == 8);
+  csr_apply<T, T>(first ? CSR_SPMV_CHEB0 : CSR_SPMV, M.n, M.rowptr.p, M.col.p,
+                  transfer_values<T>(L, true), avg, r, LevelVecs<T>::b(N), nullptr,
+                  first ? LevelVecs<T>::d(N) : nullptr, first ? level_invd<T>(N) : nullptr, T(0),
+                  first ? (T)N.cheb.c2[0] : T(0), nullptr, s,
+                  l == 0 ? SAAMG_KT_TRANSFER : SAAMG_KT_TRANSFER_DEEP, nullptr,
+                  first ? LevelVecs<T>::x0(N) : nullptr);
+  return first;
 }
 
-template <>
-void transfer<float>(saamg_hierarchy* h, int l, bool restrict_, const float* x, float* y,
-                     cudaStream_t s) {
+// x += P_l v
+template <class T>
+static void prolong(saamg_hierarchy* h, int l, const T* v, T* x, cudaStream_t s) {
   Level& L = *h->lev[l];
-  if (l == 0 && !restrict_) {
+  if (l == 0 && sizeof(T) == 4) {
     // level 0, FP32: the prolongation from the stencil and the aggregates (about 12 bytes per
     // row instead of the 39 of the CSR matrix); FP64 keeps the CSR, which needs fewer FP64
     // operations per row
-    stencil_prolong<float>(h->op->d.template view<float>(), L.agg.p, (float)L.omega, x, y, s);
+    stencil_prolong<T>(h->op->d.template view<T>(), L.agg.p, (T)L.omega, v, x, s);
     return;
   }
-  const DevCsr& M = restrict_ ? L.R : L.P;
-  const float* v = restrict_ ? L.R32.p : L.P32.p;
-  csr_apply<float, float>(restrict_ ? CSR_SPMV : CSR_ADD, M.n, M.rowptr.p, M.col.p, v,
-                          M.n ? (double)M.nnz / M.n : 0.0, x, y, nullptr, nullptr, nullptr, 0.0f,
-                          0.0f, nullptr, s, l == 0 ? SAAMG_KT_TRANSFER : SAAMG_KT_TRANSFER_DEEP);
+  const DevCsr& M = L.P;
+  csr_apply<T, T>(CSR_ADD, M.n, M.rowptr.p, M.col.p, transfer_values<T>(L, false),
+                  M.n ? (double)M.nnz / M.n : 0.0, v, x, nullptr, nullptr, nullptr, T(0), T(0),
+                  nullptr, s, l == 0 ? SAAMG_KT_TRANSFER : SAAMG_KT_TRANSFER_DEEP);
 }
 
 template <class T>
@@ -811,7 +833,8 @@ static void smooth_step(saamg_hierarchy* h, int l, int mode0, const T* x, T* y, 
 }
 
 template <class T>
-static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStream_t s) {
+static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStream_t s,
+                         bool first_done = false) {
   const int nl = (int)h->lev.size();
   Level& L = *h->lev[l];
   if (l == nl - 1) {
@@ -829,7 +852,7 @@ static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStre
   if (pair)
     stencil_apply<T>(h->op->d.template view<T>(), ST_PAIR0, b, bufs[cur], nullptr,
                      nu > 2 ? d : nullptr, sp.k1, sp.k0, nullptr, s, nullptr, sp.g);
-  else
+  else if (!first_done)
     smooth_step<T>(h, l, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0], s);
   for (int k = pair ? 2 : 1; k < nu; ++k) {
     smooth_step<T>(h, l, CSR_CHEB, bufs[cur], bufs[1 - cur], b, d, (T)L.cheb.c1[k],
@@ -842,9 +865,9 @@ static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStre
   Level& N = *h->lev[l + 1];
   T* bc = LevelVecs<T>::b(N);
   T* vc = (l + 1 == nl - 1) ? LevelVecs<T>::x0(N) : LevelVecs<T>::x1(N);
-  transfer<T>(h, l, true, r, bc, s);
-  vcycle_level<T>(h, l + 1, bc, vc, s);
-  transfer<T>(h, l, false, vc, bufs[cur], s);
+  const bool first = restrict_residual<T>(h, l, r, s);
+  vcycle_level<T>(h, l + 1, bc, vc, s, first);
+  prolong<T>(h, l, vc, bufs[cur], s);
   // postsmoothing with the same polynomial
   if (pair) {
     smooth_step<T>(h, l, CSR_RESID, bufs[cur], r, b, nullptr, T(0), T(0), s);
@@ -874,127 +897,19 @@ static void apply_preconditioner(saamg_hierarchy* h, const double* r, double* z,
   }
 }
 
-// r'z (and z'q for the Polak-Ribiere rule) of the new preconditioned residual
-static void rz_partials(saamg_hierarchy* h, const double* r, const double* z, const double* q,
-                        cudaStream_t s) {
-  const int n = h->op->d.n;
-  const bool pr = h->prm.beta_rule == 1;
-  if (mixed(h)) {
-    if (pr) dot2_partials<float>(n, r, h->z32.p, q, h->part0.p, h->part2.p, s);
-    else dot_partials<double, float>(n, r, h->z32.p, h->part0.p, s);
-  } else {
-    if (pr) dot2_partials<double>(n, r, z, q, h->part0.p, h->part2.p, s);
-    else dot_partials<double, double>(n, r, z, h->part0.p, s);
-  }
+static saamg_status info_from_ctl(const PcgCtl& c, saamg_solve_info* info) {
+  const double bn = std::sqrt(c.bb);
+  info->iters = c.iters;
+  info->converged = (c.converged && !c.breakdown) ? 1 : 0;
+  info->relres = bn > 0 ? std::sqrt(c.rr) / bn : 0.0;
+  info->relres_true = bn > 0 ? std::sqrt(c.rr_true) / bn : 0.0;
+  if (c.breakdown) return SAAMG_NUMERICAL;
+  return info->converged ? SAAMG_OK : SAAMG_NOT_CONVERGED;
 }
 
 // --- PCG --------------------------------------------------------------------
-static int pcg_impl(saamg_hierarchy* h, double rtol, cudaStream_t s, saamg_solve_info* info) {
-  const OperatorData& od = h->op->d;
-  const int n = od.n;
-  const bool mx = mixed(h);
-  double* x = h->xhat.p;
-  double* r = h->r.p;
-  double* p = h->p.p;
-  double* q = h->q.p;
-  double* z = h->z.p;
-  PcgCtl* ctl = h->ctl.p;
-  PcgCtl* hc = static_cast<PcgCtl*>(h->host.need(sizeof(PcgCtl)));
-  const StencilDev<double> S = od.view<double>();
-  info->iters = 0;
-  info->converged = 0;
-  info->relres = 0;
-  info->relres_true = 0;
-  if (n == 0) {
-    info->converged = 1;
-    return SAAMG_OK;
-  }
-  // ||b||
-  dot_partials<double, double>(n, h->bhat.p, h->bhat.p, h->part0.p, s);
-  Buf<double>& sc = h->scratch;
-  if (!sc.p) sc.alloc(4, s);
-  sum_partials(h->part0.p, kRedBlocks, sc.p, s);
-  double bb = 0;
-  d2h_sync(&bb, sc.p, sizeof(double), s);
-  if (!std::isfinite(bb)) fail(SAAMG_NUMERICAL, "right-hand side holds NaN or Inf");
-  if (bb == 0.0) {
-    SAAMG_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * n, s));
-    info->converged = 1;
-    return SAAMG_OK;
-  }
-  const double bnorm = std::sqrt(bb);
-  // r = b - A x
-  stencil_apply<double>(S, ST_RESID, x, r, h->bhat.p, nullptr, 0.0, 0.0, nullptr, s);
-  PcgCtl init{};
-  init.tol2 = (rtol * bnorm) * (rtol * bnorm);
-  SAAMG_CUDA(cudaMemcpyAsync(ctl, &init, sizeof(PcgCtl), cudaMemcpyHostToDevice, s));
-  dot_partials<double, double>(n, r, r, h->part0.p, s);
-  pcg_check(h->part0.p, ctl, s);  // counts one; reset below
-  d2h_sync(hc, ctl, sizeof(PcgCtl), s);
-  double rr = hc->rr;
-  if (!std::isfinite(rr)) fail(SAAMG_NUMERICAL, "initial residual holds NaN or Inf");
-  init.rr = rr;
-  init.iters = 0;
-  SAAMG_CUDA(cudaMemcpyAsync(ctl, &init, sizeof(PcgCtl), cudaMemcpyHostToDevice, s));
-  int status = SAAMG_NOT_CONVERGED;
-  if (rr <= init.tol2) {
-    status = SAAMG_OK;
-    info->converged = 1;
-  } else {
-    apply_preconditioner(h, r, z, h->z32.p, s);
-    if (mx) {
-      vec_copy_to_double<float>(n, h->z32.p, p, s);
-      dot_partials<double, float>(n, r, h->z32.p, h->part0.p, s);
-    } else {
-      vec_copy_to_double<double>(n, z, p, s);
-      dot_partials<double, double>(n, r, z, h->part0.p, s);
-    }
-    pcg_beta(h->part0.p, nullptr, -1, ctl, s);  // rz of the first direction
-    for (int it = 1; it <= h->prm.maxit; ++it) {
-      stencil_apply<double>(S, ST_SPMV_DOT, p, q, nullptr, nullptr, 0.0, 0.0, h->part0.p, s);
-      pcg_alpha(h->part0.p, ctl, s);
-      pcg_update(n, x, r, p, q, ctl, h->part1.p, s, mx ? h->r32.p : nullptr);
-      pcg_check(h->part1.p, ctl, s);
-      d2h_sync(hc, ctl, sizeof(PcgCtl), s);
-      info->iters = hc->iters;
-      if (hc->breakdown) {
-        status = SAAMG_NUMERICAL;
-        break;
-      }
-      if (hc->converged) {
-        status = SAAMG_OK;
-        info->converged = 1;
-        break;
-      }
-      apply_preconditioner(h, r, z, h->z32.p, s, true);
-      rz_partials(h, r, z, q, s);
-      pcg_beta(h->part0.p, h->prm.beta_rule == 1 ? h->part2.p : nullptr, h->prm.beta_rule, ctl, s);
-      if (mx) pcg_direction<float>(n, h->z32.p, p, ctl, s);
-      else pcg_direction<double>(n, z, p, ctl, s);
-    }
-  }
-  d2h_sync(hc, ctl, sizeof(PcgCtl), s);
-  info->relres = std::sqrt(hc->rr) / bnorm;
-  // true residual of the scaled system
-  stencil_apply<double>(S, ST_RESID, x, q, h->bhat.p, nullptr, 0.0, 0.0, nullptr, s);
-  dot_partials<double, double>(n, q, q, h->part0.p, s);
-  sum_partials(h->part0.p, kRedBlocks, sc.p, s);
-  double tr = 0;
-  d2h_sync(&tr, sc.p, sizeof(double), s);
-  info->relres_true = std::sqrt(tr) / bnorm;
-  if (status == SAAMG_NUMERICAL) g_last_error = "saamg_solve: breakdown (NaN/Inf or p'Ap = 0)";
-  return status;
-}
-
-// --- device-loop PCG ------------------------------------------------------------
-// The whole solve of Sec. 3.1 as one CUDA graph: a prologue (||b||, r = b - A x, the loop
-// condition), a conditional while node whose body is one PCG pass (V-cycle, beta,
-// direction, A p, alpha, update, convergence test that clears the condition), and an
-// epilogue (true residual).  Pointers and Chebyshev coefficients are fixed at capture, the
-// tolerance is read from the device scalars, so one capture serves every right-hand side.
-__global__ void set_rtol_k(PcgCtl* ctl, double rtol) { ctl->rtol = rtol; }
-
-static void pcg_pass(saamg_hierarchy* h, cudaGraphConditionalHandle cond, cudaStream_t s) {
+// One pass: z = M r, beta, direction, A p with alpha, update with the convergence test.
+static void pcg_pass(saamg_hierarchy* h, const cudaGraphConditionalHandle* cond, cudaStream_t s) {
   const OperatorData& od = h->op->d;
   const int n = od.n;
   const StencilDev<double> S = od.view<double>();
@@ -1004,16 +919,78 @@ static void pcg_pass(saamg_hierarchy* h, cudaGraphConditionalHandle cond, cudaSt
   double* q = h->q.p;
   PcgCtl* ctl = h->ctl.p;
   apply_preconditioner(h, r, h->z.p, h->z32.p, s, true);
-  rz_partials(h, r, h->z.p, q, s);
-  pcg_graph_beta(h->part0.p, rule == 1 ? h->part2.p : nullptr, rule, ctl, s);
-  if (mixed(h)) pcg_direction<float>(n, h->z32.p, p, ctl, s);
-  else pcg_direction<double>(n, h->z.p, p, ctl, s);
-  stencil_apply<double>(S, ST_SPMV_DOT, p, q, nullptr, nullptr, 0.0, 0.0, h->part0.p, s);
-  pcg_alpha(h->part0.p, ctl, s);
-  pcg_update(n, h->xhat.p, r, p, q, ctl, h->part1.p, s, mixed(h) ? h->r32.p : nullptr);
-  pcg_graph_check(h->part1.p, ctl, cond, h->prm.maxit, s);
+  if (mixed(h)) {
+    pcg_beta<float>(n, r, h->z32.p, q, h->part0.p, h->part2.p, rule, ctl, s);
+    pcg_direction<float>(n, h->z32.p, p, ctl, s);
+  } else {
+    pcg_beta<double>(n, r, h->z.p, q, h->part0.p, h->part2.p, rule, ctl, s);
+    pcg_direction<double>(n, h->z.p, p, ctl, s);
+  }
+  stencil_apply<double>(S, ST_SPMV_DOT, p, q, nullptr, nullptr, 0.0, 0.0, h->part0.p, s, nullptr,
+                        0.0, ctl);
+  pcg_update(n, h->xhat.p, r, p, q, ctl, h->part1.p, mixed(h) ? h->r32.p : nullptr, cond,
+             h->prm.maxit, s);
 }
 
+// Prologue: ||b||, r = b - A x, ||r||, p = 0, the scalars (and the loop condition of a graph).
+static void pcg_prologue(saamg_hierarchy* h, const cudaGraphConditionalHandle* cond,
+                         cudaStream_t s) {
+  const OperatorData& od = h->op->d;
+  const int n = od.n;
+  dot_partials<double, double>(n, h->bhat.p, h->bhat.p, h->part2.p, s);
+  stencil_apply<double>(od.view<double>(), ST_RESID, h->xhat.p, h->r.p, h->bhat.p, nullptr, 0.0,
+                        0.0, nullptr, s);
+  if (mixed(h)) to_float(h->r.p, h->r32.p, n, s);  // the first pass's V-cycle input
+  dot_partials<double, double>(n, h->r.p, h->r.p, h->part1.p, s);
+  SAAMG_CUDA(cudaMemsetAsync(h->p.p, 0, sizeof(double) * n, s));
+  pcg_init(h->part2.p, h->part1.p, h->ctl.p, cond, h->prm.maxit, h->xhat.p, n, s);
+}
+
+// Epilogue: the recomputed residual.
+static void pcg_epilogue(saamg_hierarchy* h, cudaStream_t s) {
+  const OperatorData& od = h->op->d;
+  stencil_apply<double>(od.view<double>(), ST_RESID, h->xhat.p, h->q.p, h->bhat.p, nullptr, 0.0,
+                        0.0, nullptr, s);
+  dot_partials<double, double>(od.n, h->q.p, h->q.p, h->part0.p, s);
+  pcg_store_true(h->part0.p, od.n, h->ctl.p, s);
+}
+
+__global__ void set_rtol_k(PcgCtl* ctl, double rtol) { ctl->rtol = rtol; }
+
+// The host-driven loop (device_loop = 0): the launches of the device loop in the same order, with
+// the scalars read back after every pass.
+static int pcg_impl(saamg_hierarchy* h, double rtol, cudaStream_t s, saamg_solve_info* info) {
+  info->iters = 0;
+  info->converged = 0;
+  info->relres = 0;
+  info->relres_true = 0;
+  if (h->op->d.n == 0) {
+    info->converged = 1;
+    return SAAMG_OK;
+  }
+  PcgCtl* ctl = h->ctl.p;
+  PcgCtl* hc = static_cast<PcgCtl*>(h->host.need(sizeof(PcgCtl)));
+  set_rtol_k<<<1, 1, 0, s>>>(ctl, rtol);
+  SAAMG_LAUNCH();
+  pcg_prologue(h, nullptr, s);
+  d2h_sync(hc, ctl, sizeof(PcgCtl), s);
+  while (!hc->converged && !hc->breakdown && hc->iters < h->prm.maxit) {
+    pcg_pass(h, nullptr, s);
+    d2h_sync(hc, ctl, sizeof(PcgCtl), s);
+  }
+  pcg_epilogue(h, s);
+  d2h_sync(hc, ctl, sizeof(PcgCtl), s);
+  const saamg_status st = info_from_ctl(*hc, info);
+  if (st == SAAMG_NUMERICAL) g_last_error = "saamg_solve: breakdown (NaN/Inf or p'Ap = 0)";
+  return st;
+}
+
+// --- device-loop PCG ------------------------------------------------------------
+// The whole solve of Sec. 3.1 as one CUDA graph: a prologue (||b||, r = b - A x, the loop
+// condition), a conditional while node whose body is one PCG pass (V-cycle, beta,
+// direction, A p, alpha, update, convergence test that clears the condition), and an
+// epilogue (true residual).  Pointers and Chebyshev coefficients are fixed at capture, the
+// tolerance is read from the device scalars, so one capture serves every right-hand side.
 // Kernels of a captured solve: `fixed` run once per graph launch, `body` once per PCG pass.
 struct GraphKernels {
   long long fixed = 0, body = 0;
@@ -1049,15 +1026,7 @@ static GraphKernels capture_pcg(saamg_hierarchy* h, cudaGraphConditionalHandle c
                                 cudaStream_t s, cudaStream_t body_s) {
   CaptureCount counting;
   const long long k0 = captured();
-  const OperatorData& od = h->op->d;
-  const int n = od.n;
-  const StencilDev<double> S = od.view<double>();
-  dot_partials<double, double>(n, h->bhat.p, h->bhat.p, h->part2.p, s);
-  stencil_apply<double>(S, ST_RESID, h->xhat.p, h->r.p, h->bhat.p, nullptr, 0.0, 0.0, nullptr, s);
-  if (mixed(h)) to_float(h->r.p, h->r32.p, n, s);  // the first pass's V-cycle input
-  dot_partials<double, double>(n, h->r.p, h->r.p, h->part1.p, s);
-  SAAMG_CUDA(cudaMemsetAsync(h->p.p, 0, sizeof(double) * n, s));
-  pcg_graph_init(h->part2.p, h->part1.p, h->ctl.p, cond, h->prm.maxit, h->xhat.p, n, s);
+  pcg_prologue(h, &cond, s);
   cudaStreamCaptureStatus st;
   cudaGraph_t cg = nullptr;
   const cudaGraphNode_t* deps = nullptr;
@@ -1072,13 +1041,11 @@ static GraphKernels capture_pcg(saamg_hierarchy* h, cudaGraphConditionalHandle c
   SAAMG_CUDA(cudaGraphAddNode(&cnode, cg, deps, nullptr, nd, &cp));
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   SAAMG_CUDA(cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-  stencil_apply<double>(S, ST_RESID, h->xhat.p, h->q.p, h->bhat.p, nullptr, 0.0, 0.0, nullptr, s);
-  dot_partials<double, double>(n, h->q.p, h->q.p, h->part0.p, s);
-  pcg_store_true(h->part0.p, h->ctl.p, s);
+  pcg_epilogue(h, s);
   const long long k1 = captured();
   SAAMG_CUDA(cudaStreamBeginCaptureToGraph(body_s, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   try {
-    pcg_pass(h, cond, body_s);
+    pcg_pass(h, &cond, body_s);
   } catch (...) {
     cudaGraph_t junk = nullptr;
     cudaStreamEndCapture(body_s, &junk);
@@ -1146,16 +1113,6 @@ static void solve_async_impl(saamg_hierarchy* h, const double* rho, double* phi,
   SAAMG_CUDA(cudaMemcpyAsync(host_out, h->ctl.p, sizeof(PcgCtl), cudaMemcpyDeviceToHost, s));
   scatter_solution(od, h->xhat.p, phi, s);
   SAAMG_CUDA(cudaEventRecord(h->done, s));
-}
-
-static saamg_status info_from_ctl(const PcgCtl& c, saamg_solve_info* info) {
-  const double bn = std::sqrt(c.bb);
-  info->iters = c.iters;
-  info->converged = (c.converged && !c.breakdown) ? 1 : 0;
-  info->relres = bn > 0 ? std::sqrt(c.rr) / bn : 0.0;
-  info->relres_true = bn > 0 ? std::sqrt(c.rr_true) / bn : 0.0;
-  if (c.breakdown) return SAAMG_NUMERICAL;
-  return info->converged ? SAAMG_OK : SAAMG_NOT_CONVERGED;
 }
 
 static void recompute_cheb(saamg_hierarchy* h, int degree) {

@@ -18,7 +18,8 @@ __global__ void __launch_bounds__(256) csr_k(int n, const int* __restrict__ rowp
                                              TV* __restrict__ y, const TV* __restrict__ b,
                                              TV* __restrict__ d, const TV* __restrict__ invd,
                                              TV c1, TV c2, double* __restrict__ partials,
-                                             const double* __restrict__ xscale) {
+                                             const double* __restrict__ xscale,
+                                             TV* __restrict__ y2) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int gl = lane % G;
@@ -31,7 +32,7 @@ __global__ void __launch_bounds__(256) csr_k(int n, const int* __restrict__ rowp
   for (int wbase = warp * kRowsPerWarp; wbase < n; wbase += nwarps * kRowsPerWarp) {
     const int row = wbase + lane / G;
     rows::csr_group_row<TV, TM, G, MODE>(row, row < n, gl, rowptr, col, val, x, y, b, d, invd,
-                                         c1, c2, dacc);
+                                         c1, c2, dacc, y2);
   }
   if (MODE == CSR_SPMV_DINV_DOT) {
     const double t = rows::block_sum(dacc);
@@ -59,7 +60,7 @@ __global__ void __launch_bounds__(256) csr_short_k(int n, const int* __restrict_
 template <class TV, class TM, int G>
 void launch_g(int mode, int n, const int* rowptr, const int* col, const TM* val, const TV* x,
               TV* y, const TV* b, TV* d, const TV* invd, TV c1, TV c2, double* partials,
-              cudaStream_t s, const double* xscale) {
+              cudaStream_t s, const double* xscale, TV* y2) {
   int blocks;
   if (mode == CSR_SPMV_DINV_DOT) {
     blocks = kRedBlocks;
@@ -70,7 +71,7 @@ void launch_g(int mode, int n, const int* rowptr, const int* col, const TM* val,
 #define SAAMG_CSR_CASE(M)                                                                  \
   case M:                                                                                  \
     launch_pdl(csr_k<TV, TM, G, M>, blocks, 256, 0, s, n, rowptr, col, val, x, y, b, d,   \
-               invd, c1, c2, partials, xscale);                                            \
+               invd, c1, c2, partials, xscale, y2);                                        \
     break;
   switch (mode) {
     SAAMG_CSR_CASE(CSR_SPMV)
@@ -79,6 +80,7 @@ void launch_g(int mode, int n, const int* rowptr, const int* col, const TM* val,
     SAAMG_CSR_CASE(CSR_CHEB0)
     SAAMG_CSR_CASE(CSR_ADD)
     SAAMG_CSR_CASE(CSR_SPMV_DINV_DOT)
+    SAAMG_CSR_CASE(CSR_SPMV_CHEB0)
     default:
       fail(SAAMG_EINVAL, "bad csr mode");
   }
@@ -127,7 +129,7 @@ int csr_plan(int mode, int n, double avg_nnz, bool dbl) {
   int g = dbl ? (avg_nnz <= 10.0 ? 2 : (avg_nnz <= 48.0 ? 4 : 8))
               : (avg_nnz <= 6.0 ? 2 : (avg_nnz <= 20.0 ? 4 : (avg_nnz <= 64.0 ? 8 : 16)));
   int gpar = 1;
-  while (gpar < 32 && (long long)n * gpar < 150000) gpar <<= 1;
+  while (gpar < 32 && (long long)n * gpar < (dbl ? 150000 : 40000)) gpar <<= 1;
   // no more lanes than the row length needs: one entry per lane in FP32; in FP64, where a
   // warp-wide shuffle-add costs a full FP64 issue slot, up to 8 entries per lane (a level of
   // 9 k rows of 61 entries: 13.9 -> 9.8 us per smoothing step with 8 instead of 32 lanes)
@@ -140,7 +142,7 @@ int csr_plan(int mode, int n, double avg_nnz, bool dbl) {
 template <class TV, class TM>
 void csr_apply(int mode, int n, const int* rowptr, const int* col, const TM* val, double avg_nnz,
                const TV* x, TV* y, const TV* b, TV* d, const TV* invd, TV c1, TV c2,
-               double* partials, cudaStream_t s, int kclass, const double* xscale) {
+               double* partials, cudaStream_t s, int kclass, const double* xscale, TV* y2) {
   if (n <= 0) {
     if (mode == CSR_SPMV_DINV_DOT) fill_double(partials, 0.0, kRedBlocks, s);
     return;
@@ -164,35 +166,36 @@ void csr_apply(int mode, int n, const int* rowptr, const int* col, const TM* val
   }
   switch (g) {
     case 2:
-      launch_g<TV, TM, 2>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale);
+      launch_g<TV, TM, 2>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale, y2);
       break;
     case 4:
-      launch_g<TV, TM, 4>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale);
+      launch_g<TV, TM, 4>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale, y2);
       break;
     case 8:
-      launch_g<TV, TM, 8>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale);
+      launch_g<TV, TM, 8>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s, xscale, y2);
       break;
     case 16:
       launch_g<TV, TM, 16>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s,
-                           xscale);
+                           xscale, y2);
       break;
     default:
       launch_g<TV, TM, 32>(mode, n, rowptr, col, val, x, y, b, d, invd, c1, c2, partials, s,
-                           xscale);
+                           xscale, y2);
   }
 }
 
 template void csr_apply<double, double>(int, int, const int*, const int*, const double*, double,
                                         const double*, double*, const double*, double*,
                                         const double*, double, double, double*, cudaStream_t, int,
-                                        const double*);
+                                        const double*, double*);
 template void csr_apply<float, float>(int, int, const int*, const int*, const float*, double,
                                       const float*, float*, const float*, float*, const float*,
-                                      float, float, double*, cudaStream_t, int, const double*);
+                                      float, float, double*, cudaStream_t, int, const double*,
+                                      float*);
 template void csr_apply<float, __nv_bfloat16>(int, int, const int*, const int*,
                                               const __nv_bfloat16*, double, const float*, float*,
                                               const float*, float*, const float*, float, float,
-                                              double*, cudaStream_t, int, const double*);
+                                              double*, cudaStream_t, int, const double*, float*);
 
 void csr_diag_inverse(const DevCsr& A, double* invd, float* invd32, cudaStream_t s) {
   if (A.n == 0) return;

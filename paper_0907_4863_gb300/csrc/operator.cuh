@@ -110,7 +110,8 @@ enum StencilMode {
 //   k0 = g + c1 g + c2, k1 = c2 g;   d = x2 - x1.
 // From x = 0 that is one pass over b instead of two (7 FP64 operations a row instead of 11, 16 bytes
 // instead of 64), after the prolongation the residual and one pass (15 instead of 19 operations, 48
-// bytes instead of 72): at 256^3 in FP64 43 + 148 -> TIME_A us and 134 + 148 -> TIME_B us.
+// bytes instead of 72).  Measured at 256^3 in FP64: 43 + 148 us from zero and 134 + 148 after the
+// prolongation became 117 (the mean of the pair passes) and 107 + 117.
 template <class T>
 struct SmoothPair {
   T k0, k1, g;
@@ -118,11 +119,13 @@ struct SmoothPair {
       : k0((T)(g_ + c1 * g_ + c2)), k1((T)(c2 * g_)), g((T)g_) {}
 };
 
-// c1, c2: of the Chebyshev steps; the pair passes take k1, k0 there and g
+// c1, c2: of the Chebyshev steps; the pair passes take k1, k0 there and g.  ctl (ST_SPMV_DOT): the
+// last block forms the CG step length from the partials.
+struct PcgCtl;
 template <class T>
 void stencil_apply(const StencilDev<T>& S, int mode, const T* x, T* y, const T* b, T* d, T c1,
                    T c2, double* partials, cudaStream_t s, const double* xscale = nullptr,
-                   T g = T(0));
+                   T g = T(0), PcgCtl* ctl = nullptr);
 // S with the regular rows' coefficients of k0 I - k1 A, as the pair passes apply it
 template <class T>
 StencilDev<T> pair_stencil(StencilDev<T> S, T k0, T k1) {

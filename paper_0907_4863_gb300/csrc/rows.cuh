@@ -26,7 +26,7 @@ __device__ __forceinline__ void csr_group_row(int row, bool active, int gl,
                                               const TV* __restrict__ x, TV* __restrict__ y,
                                               const TV* __restrict__ b, TV* __restrict__ d,
                                               const TV* __restrict__ invd, TV c1, TV c2,
-                                              double& dacc) {
+                                              double& dacc, TV* __restrict__ y2 = nullptr) {
   TV acc = TV(0);
   if (MODE != CSR_CHEB0 && active) {
     const int p0 = rowptr[row], p1 = rowptr[row + 1];
@@ -72,6 +72,11 @@ __device__ __forceinline__ void csr_group_row(int row, bool active, int gl,
       const TV dv = (c1 == TV(0)) ? c2 * t : fma(c2, t, c1 * d[row]);
       d[row] = dv;
       y[row] = x[row] + dv;
+    } else if (MODE == CSR_SPMV_CHEB0) {
+      const TV dv = c2 * (invd[row] * acc);
+      y[row] = acc;
+      d[row] = dv;
+      y2[row] = dv;
     } else if (MODE == CSR_CHEB0) {
       const TV dv = c2 * (invd[row] * b[row]);
       d[row] = dv;
@@ -96,7 +101,8 @@ __device__ __forceinline__ void csr_group_rows(const int row[NR], const bool act
                                                const TM* __restrict__ val,
                                                const TV* __restrict__ x, TV* __restrict__ y,
                                                const TV* __restrict__ b, TV* __restrict__ d,
-                                               const TV* __restrict__ invd, TV c1, TV c2) {
+                                               const TV* __restrict__ invd, TV c1, TV c2,
+                                               TV* __restrict__ y2) {
   static_assert(NR <= G, "a lane per row");
   int p[NR], p1[NR], er = -1;
 #pragma unroll
@@ -114,6 +120,7 @@ __device__ __forceinline__ void csr_group_rows(const int row[NR], const bool act
       if (c1 != TV(0)) dv = d[er];
     }
     if (MODE == CSR_ADD) xv = y[er];
+    if (MODE == CSR_SPMV_CHEB0) iv = invd[er];
   }
   int k[NR][2];
   TV a[NR][2], acc[NR];
@@ -149,6 +156,11 @@ __device__ __forceinline__ void csr_group_rows(const int row[NR], const bool act
   if (er < 0) return;
   if (MODE == CSR_SPMV) {
     y[er] = s;
+  } else if (MODE == CSR_SPMV_CHEB0) {
+    const TV w = c2 * (iv * s);
+    y[er] = s;
+    d[er] = w;
+    y2[er] = w;
   } else if (MODE == CSR_RESID) {
     y[er] = bv - s;
   } else if (MODE == CSR_ADD) {
@@ -290,11 +302,12 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
-// Single-block ordered sum of kRedBlocks partials (kRedThreads threads), valid in all threads.
-__device__ __forceinline__ double sum_fixed(const double* part) {
+// Ordered sum of `count` partials by one block of kRedThreads threads, valid in all threads.  The
+// partials are read through L2: blocks of the same launch may have written them.
+__device__ __forceinline__ double sum_fixed(const double* part, int count) {
   __shared__ double sh[kRedThreads];
   double acc = 0.0;
-  for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) acc += part[i];
+  for (int i = threadIdx.x; i < count; i += blockDim.x) acc += __ldcg(part + i);
   sh[threadIdx.x] = acc;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -306,13 +319,13 @@ __device__ __forceinline__ double sum_fixed(const double* part) {
   return r;
 }
 
-// Block `blk` of a fixed grid of kRedBlocks x kRedThreads: its partial of sum a_i b_i (loads
+// Block `blk` of a fixed grid of kVecBlocks x kRedThreads: its partial of sum a_i b_i (loads
 // of four grid strides in flight, the multiply-adds in index order).  Valid in thread 0.
 template <class TA, class TB>
 __device__ __forceinline__ double dot_block(int blk, int n, const TA* __restrict__ a,
                                             const TB* __restrict__ b) {
   double acc = 0.0;
-  const int st = kRedBlocks * kRedThreads;
+  const int st = kVecBlocks * kRedThreads;
   int i = blk * kRedThreads + threadIdx.x;
   for (; i + 3 * st < n; i += 4 * st) {
     const double a0 = (double)a[i], a1 = (double)a[i + st], a2 = (double)a[i + 2 * st],
@@ -336,7 +349,7 @@ __device__ __forceinline__ void dot2_block(int blk, int n, const double* __restr
                                            const double* __restrict__ q, double& t1,
                                            double& t2) {
   double a1 = 0.0, a2 = 0.0;
-  const int st = kRedBlocks * kRedThreads;
+  const int st = kVecBlocks * kRedThreads;
   int i = blk * kRedThreads + threadIdx.x;
   // loads of four grid strides in flight (the fixed grid holds half the warps an SM can)
   for (; i + 3 * st < n; i += 4 * st) {
@@ -370,26 +383,10 @@ __device__ __forceinline__ double update_block(int blk, int n, double a, double*
                                                const double* __restrict__ q,
                                                float* __restrict__ r32) {
   double acc = 0.0;
-  const int st = kRedBlocks * kRedThreads;
-  int i = blk * kRedThreads + threadIdx.x;
-  // two grid strides per step, every load before the stores
-  for (; i + st < n; i += 2 * st) {
-    const double x0 = x[i], x1 = x[i + st], p0 = p[i], p1 = p[i + st];
-    const double rv0 = r[i], rv1 = r[i + st], q0 = q[i], q1 = q[i + st];
-    x[i] = x0 + a * p0;
-    const double ri0 = rv0 - a * q0;
-    r[i] = ri0;
-    if (r32) r32[i] = (float)ri0;
-    acc += ri0 * ri0;
-    x[i + st] = x1 + a * p1;
-    const double ri1 = rv1 - a * q1;
-    r[i + st] = ri1;
-    if (r32) r32[i + st] = (float)ri1;
-    acc += ri1 * ri1;
-  }
-  for (; i < n; i += st) {
-    x[i] = x[i] + a * p[i];
-    double ri = r[i] - a * q[i];
+  for (int i = blk * kRedThreads + threadIdx.x; i < n; i += kVecBlocks * kRedThreads) {
+    const double xi = x[i], pi = p[i], rv = r[i], qi = q[i];
+    x[i] = xi + a * pi;
+    const double ri = rv - a * qi;
     r[i] = ri;
     if (r32) r32[i] = (float)ri;
     acc += ri * ri;
@@ -431,7 +428,7 @@ __device__ __forceinline__ double warp_tree8(const double v[kVirtWarps], int lan
 // f(i, w) for every element i of the block's threads 32 w + lane, in each thread's order
 template <class F>
 __device__ __forceinline__ void virt_block(int blk, int n, int lane, F&& f) {
-  for (int base = blk * kRedThreads; base < n; base += kRedBlocks * kRedThreads) {
+  for (int base = blk * kRedThreads; base < n; base += kVecBlocks * kRedThreads) {
 #pragma unroll
     for (int w = 0; w < kVirtWarps; ++w) {
       if (base + 32 * w >= n) break;  // uniform

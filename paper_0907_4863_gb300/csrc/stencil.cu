@@ -15,6 +15,7 @@
 
 #include "operator.cuh"
 #include "batch.cuh"
+#include "pcg.cuh"
 #include "rows.cuh"
 
 namespace saamg {
@@ -234,9 +235,9 @@ template <class T, int MODE, int K, bool PACKED>
 __global__ void __launch_bounds__(256) stencil_k(StencilDev<T> S, const T* __restrict__ x,
                                                  T* __restrict__ y, const T* __restrict__ b,
                                                  T* __restrict__ d, T c1, T c2, T c2invd0,
-                                                 double* __restrict__ partials,
+                                                 double* partials,
                                                  const double* __restrict__ xscale,
-                                                 const int* __restrict__ agg) {
+                                                 const int* __restrict__ agg, PcgCtl* ctl) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
@@ -279,6 +280,11 @@ __global__ void __launch_bounds__(256) stencil_k(StencilDev<T> S, const T* __res
       double t = 0.0;
       for (int w = 0; w < wpb; ++w) t += sh[w];
       partials[blockIdx.x] = t;
+    }
+    if (MODE == ST_SPMV_DOT && ctl) {  // CG: the last block adds the partials and forms alpha
+      if (!last_block(&ctl->tick[1])) return;
+      const double pq = rows::sum_fixed(partials, gridDim.x);
+      if (threadIdx.x == 0) finish_alpha(ctl, pq);
     }
   }
 }
@@ -450,7 +456,7 @@ void launch_shaped(const StencilCfg& cfg, long long units, int blocks_cap, const
 #define SAAMG_SHAPE(KK, PP)                                                                  \
   if (cfg.k == KK && (cfg.packed != 0) == PP) {                                              \
     launch_pdl(stencil_k<T, MODE, KK, PP>, blocks, cfg.block, 0, s, S, x, y, b, d, c1, c2,   \
-               c2i0, partials, xscale, agg);                                                 \
+               c2i0, partials, xscale, agg, (PcgCtl*)nullptr);                               \
     return;                                                                                  \
   }
   SAAMG_SHAPE(1, false)
@@ -471,7 +477,8 @@ long long shaped_units(const StencilDev<T>& S, bool packed) {
 
 template <class T>
 void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T* b, T* d, T c1,
-                   T c2, double* partials, cudaStream_t s, const double* xscale, T g) {
+                   T c2, double* partials, cudaStream_t s, const double* xscale, T g,
+                   PcgCtl* ctl) {
   const bool pair = mode == ST_PAIR0 || mode == ST_PAIR || mode == ST_PAIR_D;
   const StencilDev<T> S = pair ? pair_stencil(S0, c2, c1) : S0;
   if (S.nchunks == 0) {
@@ -496,12 +503,16 @@ void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T*
     // taken the same way
     constexpr bool P = packed_rows<T>();
     const int* no_agg = nullptr;
+    // with ctl the last block adds the partials of the blocks that have chunks; the others' are 0
+    const int wide = kRedThreads / 32 * kChunks<T>();
+    const int blocks = ctl ? std::min(kRedBlocks, (stencil_units<T>(S) + wide - 1) / wide)
+                           : kRedBlocks;
     if (mode == ST_SPMV_DOT)
-      launch_pdl(stencil_k<T, ST_SPMV_DOT, kChunks<T>(), P>, kRedBlocks, kRedThreads, 0, s, S, x,
-                 y, b, d, c1, c2, c2i0, partials, xscale, no_agg);
+      launch_pdl(stencil_k<T, ST_SPMV_DOT, kChunks<T>(), P>, blocks, kRedThreads, 0, s, S, x,
+                 y, b, d, c1, c2, c2i0, partials, xscale, no_agg, ctl);
     else
       launch_pdl(stencil_k<T, ST_DINV_DOT, kChunks<T>(), P>, kRedBlocks, kRedThreads, 0, s, S, x,
-                 y, b, d, c1, c2, c2i0, partials, xscale, no_agg);
+                 y, b, d, c1, c2, c2i0, partials, xscale, no_agg, (PcgCtl*)nullptr);
     SAAMG_LAUNCH();
     return;
   }
@@ -617,9 +628,9 @@ template void stencil_prolong<double>(const StencilDev<double>&, const int*, dou
 
 template void stencil_apply<double>(const StencilDev<double>&, int, const double*, double*,
                                     const double*, double*, double, double, double*,
-                                    cudaStream_t, const double*, double);
+                                    cudaStream_t, const double*, double, PcgCtl*);
 template void stencil_apply<float>(const StencilDev<float>&, int, const float*, float*,
                                    const float*, float*, float, float, double*, cudaStream_t,
-                                   const double*, float);
+                                   const double*, float, PcgCtl*);
 
 }  // namespace saamg
