@@ -9,6 +9,7 @@
 #include "pic.cuh"
 
 #include "divc.cuh"
+#include "softmul.cuh"
 
 namespace saamg {
 
@@ -67,6 +68,13 @@ __device__ __forceinline__ void split_coord_fixed(double u, int& c, unsigned lon
     c = f != 0ull ? -c - 1 : -c;
     f = 0ull - f;
   }
+}
+
+// Whether split_coord_fixed's fraction of u holds all of u's bits: u is 0 or at least 2^-11, so
+// that neither a bit below 2^-64 is cut nor, for u < 0, a rounding of 1 + u left out.
+__device__ __forceinline__ bool fraction_exact(double u) {
+  const long long b = __double_as_longlong(u);
+  return b == 0 || b >= 0x3f40000000000000LL;
 }
 
 __global__ void abs_sum_k(int n, const double* __restrict__ q, double* __restrict__ part) {
@@ -212,11 +220,16 @@ __global__ void __launch_bounds__(256) fixed_to_double_k(size_t n, const int* __
   }
 }
 
+// Components of the field whose products run on the integer units, the others' on the FP64 pipe:
+// 10^7 particles on 256^3 took 1101, 951, 1026 and 1139 us with 0, 1, 2 and 3.
+constexpr int kGatherSoft = 1;
+
 // Bitwise the reference's sums: ((wx wy) wz) E added in its corner order, every product and sum
-// rounded.  Those 12 + 45 FP64 instructions, and 18-24 for the three coordinates, bind the kernel
-// (FP64 pipe 84 % busy at two lanes per clock and SM, L2 29 %); full divisions by the spacings and
-// floor() made 10^7 particles on 256^3 take 2019 instead of 1656 us.  All eight nodal values of a
-// component are loaded before they are used.
+// rounded -- 12 + 24 products and 24 sums a particle.  On the FP64 pipe alone they took 1656 us for
+// 10^7 particles on 256^3 (pipe 84 % busy, L2 29 %); here the cell and the weights of a particle
+// inside the box are integer arithmetic (softmul.cuh, the bits of the FP64 operations), and so are
+// the products of kGatherSoft components, which run beside the sums on the other pipe.  A
+// particle at the box's edge, and operands that are not normal numbers, take the FP64 operations.
 __global__ void __launch_bounds__(256) cic_gather_k(Lattice g, const double* __restrict__ ex,
                                                     const double* __restrict__ ey,
                                                     const double* __restrict__ ez, int np,
@@ -233,23 +246,28 @@ __global__ void __launch_bounds__(256) cic_gather_k(Lattice g, const double* __r
                uz = lattice_coord(zp, g.oz, g.hz);
   double s[3] = {0.0, 0.0, 0.0};
   if (coord_near(ux) && coord_near(uy) && coord_near(uz)) {
-    int ci, cj, ck;
-    double fx, fy, fz;
-    split_coord(ux, ci, fx);
-    split_coord(uy, cj, fy);
-    split_coord(uz, ck, fz);
     const double* E[3] = {ex, ey, ez};
-    const double wx[2] = {__dadd_rn(1.0, -fx), fx}, wy[2] = {__dadd_rn(1.0, -fy), fy},
-                 wz[2] = {__dadd_rn(1.0, -fz), fz};
-    double wxy[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wxy[q] = __dmul_rn(wx[q & 1], wy[q >> 1]);
-    const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
     const long long sy = g.nx, sz = (long long)g.nx * g.ny;
-    if (ci >= 0 && cj >= 0 && ck >= 0 && ci + 1 < g.nx && cj + 1 < g.ny && ck + 1 < g.nz) {
-      double w[8];
+    int ci, cj, ck;
+    unsigned long long hx, hy, hz;
+    split_coord_fixed(ux, ci, hx);
+    split_coord_fixed(uy, cj, hy);
+    split_coord_fixed(uz, ck, hz);
+    if (fraction_exact(ux) && fraction_exact(uy) && fraction_exact(uz) && ci + 1 < g.nx &&
+        cj + 1 < g.ny && ck + 1 < g.nz) {
+      const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
+      Unpacked w[8];
+      {
+        const Unpacked wx[2] = {unpack_complement(hx), unpack_fraction(hx)};
+        const Unpacked wy[2] = {unpack_complement(hy), unpack_fraction(hy)};
+        const Unpacked wz[2] = {unpack_complement(hz), unpack_fraction(hz)};
 #pragma unroll
-      for (int q = 0; q < 8; ++q) w[q] = __dmul_rn(wxy[q & 3], wz[q >> 2]);
+        for (int q = 0; q < 4; ++q) {
+          const Unpacked wxy = mul_unpacked(wx[q & 1], wy[q >> 1]);
+          w[q] = mul_unpacked(wxy, wz[0]);
+          w[q + 4] = mul_unpacked(wxy, wz[1]);
+        }
+      }
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         const double* e = E[k] + v0;
@@ -257,20 +275,36 @@ __global__ void __launch_bounds__(256) cic_gather_k(Lattice g, const double* __r
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           t[q] = e[(q & 1) + ((q >> 1) & 1) * sy + (q >> 2) * sz];
-        double a = __dmul_rn(w[0], t[0]);
+        double a = 0.0;
 #pragma unroll
-        for (int q = 1; q < 8; ++q) a = __dadd_rn(a, __dmul_rn(w[q], t[q]));
+        for (int q = 0; q < 8; ++q) {
+          double m;
+          bool ok = false;
+          if (k < kGatherSoft)
+            m = __longlong_as_double(
+                (long long)mul_bits(w[q], (uint64_t)__double_as_longlong(t[q]), ok));
+          if (!ok) m = __dmul_rn(__longlong_as_double((long long)pack_bits(w[q])), t[q]);
+          a = q == 0 ? m : __dadd_rn(a, m);
+        }
         // the reference starts from +0, which no sum of zeros of either sign leaves
         s[k] = (static_cast<unsigned long long>(__double_as_longlong(a)) << 1) == 0ull ? 0.0 : a;
       }
     } else {
-#pragma unroll
+      double fx, fy, fz;
+      split_coord(ux, ci, fx);
+      split_coord(uy, cj, fy);
+      split_coord(uz, ck, fz);
+      const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
+      const double wx[2] = {__dadd_rn(1.0, -fx), fx}, wy[2] = {__dadd_rn(1.0, -fy), fy},
+                   wz[2] = {__dadd_rn(1.0, -fz), fz};
+#pragma unroll 1
       for (int q = 0; q < 8; ++q) {
         const int i = q & 1, j = (q >> 1) & 1, k = q >> 2;
         if (ci + i < 0 || cj + j < 0 || ck + k < 0 || ci + i >= g.nx || cj + j >= g.ny ||
             ck + k >= g.nz)
           continue;
-        const double w = __dmul_rn(wxy[q & 3], wz[k]);
+        const double w = __dmul_rn(__dmul_rn(i ? wx[1] : wx[0], j ? wy[1] : wy[0]),
+                                   k ? wz[1] : wz[0]);
         const long long v = v0 + i + j * sy + k * sz;
 #pragma unroll
         for (int d = 0; d < 3; ++d) s[d] = __dadd_rn(s[d], __dmul_rn(w, E[d][v]));
