@@ -43,13 +43,20 @@ void set_last_error(const std::string& msg);
 // Programmatic dependent launch.  The solve's kernels are launched with launch_pdl, so the
 // launch of a kernel is prepared while the kernel before it on the stream runs; its blocks wait
 // at pdl_wait (their first statement, before any memory access) until that kernel has finished
-// and its writes are visible.  No kernel signals its dependents early: measured at 256^3, an
-// early signal (at kernel entry) made the solve 5-8 % slower, none 0.8-1.3 % faster than plain
-// launches.  The order and the results of the work are those of plain launches; pdl_wait does
-// nothing in a kernel launched without the attribute.  SAAMG_PDL=0 in the environment turns
-// the attribute off.
+// and its writes are visible.  A kernel of at most kPdlEarlyBlocks blocks (two per SM: all of them
+// are resident) lets its dependents in at its own entry, so their blocks are in place when it
+// ends; a larger one does not, because blocks that only wait take the slots of its own later
+// blocks (with 1216 the solve at 256^3 took 27.4 instead of 25.4 ms; with 304 the small levels
+// gain: 141x97x203 BF16 4745 -> 4659 us, 32^3 1061 -> 1050).  The order and the results of the work
+// are those of plain launches; pdl_wait does nothing in a kernel launched without the
+// attribute.  SAAMG_PDL=0 in the environment turns the attribute off.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+constexpr unsigned kPdlEarlyBlocks = 304;
+__device__ __forceinline__ void pdl_wait() {
+  if (gridDim.x * gridDim.y <= kPdlEarlyBlocks)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 bool pdl_enabled();
 
 template <typename... KArgs, typename... Args>
