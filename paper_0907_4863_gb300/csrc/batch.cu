@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(256, 5) bcopy_k(const MTask* __restrict__ task
 }
 
 // --- CG vector kernels ----------------------------------------------------------------------
-// Every (task t, block b) pair computes block b of the one-solve grid (kVecBlocks blocks of
+// Every (task t, block b) pair computes block b of the one-solve grid (kRedBlocks blocks of
 // kRedThreads) for task t, emulated by one warp (rows::*_block_warp), so each partial has the
 // one-solve bits; warps take pairs in turn.  The list holds the blocks with elements only (the
 // partials of the others stay 0, what the one-solve block sums): over all blocks of all tasks in
@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(256, 5) bzero_k(const VTask* __restrict__ task
 // --- CG scalars: a block per task -------------------------------------------------------------
 __global__ void __launch_bounds__(kRedThreads) binit_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
-  const double bb = rows::sum_fixed(k.part2, kVecBlocks);
-  const double rr = rows::sum_fixed(k.part1, kVecBlocks);
+  const double bb = rows::sum_fixed(k.part2, kRedBlocks);
+  const double rr = rows::sum_fixed(k.part1, kRedBlocks);
   if (threadIdx.x == 0) {
     k.ctl->rtol = k.rtol;
     *k.go = finish_init(k.ctl, bb, rr, k.maxit);
@@ -294,15 +294,15 @@ __global__ void __launch_bounds__(kRedThreads) binit_k(const VTask* __restrict__
 
 __global__ void __launch_bounds__(kRedThreads) bstore_true_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
-  const double rr = rows::sum_fixed(k.part0, kVecBlocks);
+  const double rr = rows::sum_fixed(k.part0, kRedBlocks);
   if (threadIdx.x == 0) k.ctl->rr_true = rr;
 }
 
 __global__ void __launch_bounds__(kRedThreads) bbeta_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
-  const double rz = rows::sum_fixed(k.part0, kVecBlocks);
-  const double zq = k.rule == 1 ? rows::sum_fixed(k.part2, kVecBlocks) : 0.0;
+  const double rz = rows::sum_fixed(k.part0, kRedBlocks);
+  const double zq = k.rule == 1 ? rows::sum_fixed(k.part2, kRedBlocks) : 0.0;
   if (threadIdx.x == 0) finish_beta(k.ctl, rz, zq, k.rule);
 }
 
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kRedThreads) balpha_k(const VTask* __restrict_
 __global__ void __launch_bounds__(kRedThreads) bcheck_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
-  const double rr = rows::sum_fixed(k.part1, kVecBlocks);
+  const double rr = rows::sum_fixed(k.part1, kRedBlocks);
   if (threadIdx.x == 0) *k.go = finish_check(k.ctl, rr, k.maxit);
 }
 
@@ -829,7 +829,7 @@ void alloc_work(SolveWork& w, cudaStream_t s) {
   } else {
     w.z.alloc(n, s);
   }
-  w.part.alloc(3 * kVecBlocks + kRedBlocks, s);
+  w.part.alloc(3 * kRedBlocks + kRedBlocks, s);
   SAAMG_CUDA(cudaMemsetAsync(w.part.p, 0, w.part.bytes(), s));
   const int nl = (int)h->lev.size();
   if (mx) {
@@ -969,9 +969,9 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
     t.z = mx ? (const void*)w.z32.p : (const void*)w.z.p;
     t.r32 = mx ? w.r32.p : nullptr;
     t.part0 = w.part.p;
-    t.part1 = w.part.p + kVecBlocks;
-    t.part2 = w.part.p + 2 * kVecBlocks;
-    t.partq = w.part.p + 3 * kVecBlocks;
+    t.part1 = w.part.p + kRedBlocks;
+    t.part2 = w.part.p + 2 * kRedBlocks;
+    t.partq = w.part.p + 3 * kRedBlocks;
     t.rule = h->prm.beta_rule;
     t.maxit = h->prm.maxit;
     t.rtol = rtol;
@@ -1009,7 +1009,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
                                cudaMemcpyHostToDevice, s));
   {
     std::vector<int2> pr;
-    auto blocks = [](int n) { return std::min(kVecBlocks, (n + kRedThreads - 1) / kRedThreads); };
+    auto blocks = [](int n) { return std::min(kRedBlocks, (n + kRedThreads - 1) / kRedThreads); };
     auto add = [&](int task, int nb) {
       for (int b = 0; b < nb; ++b) pr.push_back(make_int2(task, b));
     };
@@ -1048,7 +1048,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       t.go = L.go.p + i;
       t.x = w.p.p;
       t.y = w.q.p;
-      t.part = w.part.p + 3 * kVecBlocks;
+      t.part = w.part.p + 3 * kRedBlocks;
       dt[i] = t;
     }
     L.dot_tasks.alloc(m, s);

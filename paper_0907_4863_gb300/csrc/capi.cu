@@ -338,9 +338,9 @@ static void alloc_pcg_vectors(saamg_hierarchy* h, int n, cudaStream_t s) {
     h->z32.alloc(n, s);
     h->r32.alloc(n, s);
   }
-  h->part0.alloc(kVecBlocks, s);
-  h->part1.alloc(kVecBlocks, s);
-  h->part2.alloc(kVecBlocks, s);
+  h->part0.alloc(kRedBlocks, s);
+  h->part1.alloc(kRedBlocks, s);
+  h->part2.alloc(kRedBlocks, s);
   h->ctl.alloc(1, s);
 }
 

@@ -252,9 +252,6 @@ struct DevCsr {
 // the summation tree, which must not change with the part the library runs on.
 constexpr int kRedBlocks = 608;
 constexpr int kRedThreads = 256;
-// The dot products and the x / r update of the CG loop wait for memory and take six blocks per
-// SM, as many as the update's registers allow at once.  A p with p'q keeps 608: 1216 were slower.
-constexpr int kVecBlocks = 912;
 
 // ---------------------------------------------------------------------------
 // Host launchers (implemented in the .cu files; each file owns its kernels)

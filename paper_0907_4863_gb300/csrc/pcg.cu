@@ -16,13 +16,13 @@ using rows::sum_fixed;
 // Blocks of the vector reductions of n elements: those of the fixed grid that hold any (the
 // partials of the others are 0; a short vector has few, and each costs a fence and an atomic).
 inline int red_blocks(int n) {
-  return std::max(1, std::min(kVecBlocks, (n + kRedThreads - 1) / kRedThreads));
+  return std::max(1, std::min(kRedBlocks, (n + kRedThreads - 1) / kRedThreads));
 }
 
 // Loads of four grid strides are issued before their (in-order) multiply-adds: the sum is
 // the same sequence of operations as the plain strided loop, with more bytes in flight.
 template <class TA, class TB>
-__global__ void __launch_bounds__(kRedThreads, 6) dot_k(int n, const TA* __restrict__ a,
+__global__ void __launch_bounds__(kRedThreads) dot_k(int n, const TA* __restrict__ a,
                                                         const TB* __restrict__ b,
                                                         double* __restrict__ part) {
   pdl_wait();
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kRedThreads, 6) dot_k(int n, const TA* __restr
 
 // r'z (and z'q in the same sweep) and, in the last block, beta
 template <class TZ, bool PR>
-__global__ void __launch_bounds__(kRedThreads, 6) beta_k(int n, const double* __restrict__ r,
+__global__ void __launch_bounds__(kRedThreads) beta_k(int n, const double* __restrict__ r,
                                                          const TZ* __restrict__ z,
                                                          const double* __restrict__ q,
                                                          double* part_rz, double* part_zq,
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kRedThreads, 6) beta_k(int n, const double* __
 }
 
 // r32 (mixed precision): the FP32 copy of the new residual, the next V-cycle's input
-__global__ void __launch_bounds__(kRedThreads, 6) update_k(int n, double* __restrict__ x,
+__global__ void __launch_bounds__(kRedThreads) update_k(int n, double* __restrict__ x,
                                                            double* __restrict__ r,
                                                            const double* __restrict__ p,
                                                            const double* __restrict__ q,

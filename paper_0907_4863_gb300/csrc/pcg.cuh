@@ -89,7 +89,7 @@ __device__ __forceinline__ bool last_block(unsigned* tick) {
   return last != 0;
 }
 
-// partials[blockIdx] of sum a_i b_i (fixed grid kVecBlocks, of which the blocks with elements run)
+// partials[blockIdx] of sum a_i b_i (fixed grid kRedBlocks, of which the blocks with elements run)
 template <class TA, class TB>
 void dot_partials(int n, const TA* a, const TB* b, double* partials, cudaStream_t s);
 

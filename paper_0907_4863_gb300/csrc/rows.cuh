@@ -319,13 +319,13 @@ __device__ __forceinline__ double sum_fixed(const double* part, int count) {
   return r;
 }
 
-// Block `blk` of a fixed grid of kVecBlocks x kRedThreads: its partial of sum a_i b_i (loads
+// Block `blk` of a fixed grid of kRedBlocks x kRedThreads: its partial of sum a_i b_i (loads
 // of four grid strides in flight, the multiply-adds in index order).  Valid in thread 0.
 template <class TA, class TB>
 __device__ __forceinline__ double dot_block(int blk, int n, const TA* __restrict__ a,
                                             const TB* __restrict__ b) {
   double acc = 0.0;
-  const int st = kVecBlocks * kRedThreads;
+  const int st = kRedBlocks * kRedThreads;
   int i = blk * kRedThreads + threadIdx.x;
   for (; i + 3 * st < n; i += 4 * st) {
     const double a0 = (double)a[i], a1 = (double)a[i + st], a2 = (double)a[i + 2 * st],
@@ -349,7 +349,7 @@ __device__ __forceinline__ void dot2_block(int blk, int n, const double* __restr
                                            const double* __restrict__ q, double& t1,
                                            double& t2) {
   double a1 = 0.0, a2 = 0.0;
-  const int st = kVecBlocks * kRedThreads;
+  const int st = kRedBlocks * kRedThreads;
   int i = blk * kRedThreads + threadIdx.x;
   // loads of four grid strides in flight (the fixed grid holds half the warps an SM can)
   for (; i + 3 * st < n; i += 4 * st) {
@@ -383,10 +383,26 @@ __device__ __forceinline__ double update_block(int blk, int n, double a, double*
                                                const double* __restrict__ q,
                                                float* __restrict__ r32) {
   double acc = 0.0;
-  for (int i = blk * kRedThreads + threadIdx.x; i < n; i += kVecBlocks * kRedThreads) {
-    const double xi = x[i], pi = p[i], rv = r[i], qi = q[i];
-    x[i] = xi + a * pi;
-    const double ri = rv - a * qi;
+  const int st = kRedBlocks * kRedThreads;
+  int i = blk * kRedThreads + threadIdx.x;
+  // two grid strides per step, every load before the stores
+  for (; i + st < n; i += 2 * st) {
+    const double x0 = x[i], x1 = x[i + st], p0 = p[i], p1 = p[i + st];
+    const double rv0 = r[i], rv1 = r[i + st], q0 = q[i], q1 = q[i + st];
+    x[i] = x0 + a * p0;
+    const double ri0 = rv0 - a * q0;
+    r[i] = ri0;
+    if (r32) r32[i] = (float)ri0;
+    acc += ri0 * ri0;
+    x[i + st] = x1 + a * p1;
+    const double ri1 = rv1 - a * q1;
+    r[i + st] = ri1;
+    if (r32) r32[i + st] = (float)ri1;
+    acc += ri1 * ri1;
+  }
+  for (; i < n; i += st) {
+    x[i] = x[i] + a * p[i];
+    double ri = r[i] - a * q[i];
     r[i] = ri;
     if (r32) r32[i] = (float)ri;
     acc += ri * ri;
@@ -428,7 +444,7 @@ __device__ __forceinline__ double warp_tree8(const double v[kVirtWarps], int lan
 // f(i, w) for every element i of the block's threads 32 w + lane, in each thread's order
 template <class F>
 __device__ __forceinline__ void virt_block(int blk, int n, int lane, F&& f) {
-  for (int base = blk * kRedThreads; base < n; base += kVecBlocks * kRedThreads) {
+  for (int base = blk * kRedThreads; base < n; base += kRedBlocks * kRedThreads) {
 #pragma unroll
     for (int w = 0; w < kVirtWarps; ++w) {
       if (base + 32 * w >= n) break;  // uniform
