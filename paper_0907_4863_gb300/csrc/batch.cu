@@ -1064,6 +1064,7 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       const OperatorData& od = w.h->op->d;
       BoxTask& t = box[i];
       t.g = od.g;
+      t.s0 = make_divc(od.s0);
       t.lines = od.lines.p;
       t.chunks = od.chunks.p;
       t.scale = od.scale.p;

@@ -252,6 +252,10 @@ struct DevCsr {
 // the summation tree, which must not change with the part the library runs on.
 constexpr int kRedBlocks = 608;
 constexpr int kRedThreads = 256;
+// D^-1 A x with its norm on the sparse levels (power iteration): at most as many blocks as the
+// smoother takes, because its gathers wait for memory (256^3, level 1 SELL in FP64: 113 us with
+// 608 blocks, 71 with these; 183x160x171, level 1 CSR: 52 -> 44).
+constexpr int kPowerBlocks = 2432;
 
 // ---------------------------------------------------------------------------
 // Host launchers (implemented in the .cu files; each file owns its kernels)

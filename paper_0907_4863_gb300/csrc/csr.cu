@@ -61,13 +61,9 @@ template <class TV, class TM, int G>
 void launch_g(int mode, int n, const int* rowptr, const int* col, const TM* val, const TV* x,
               TV* y, const TV* b, TV* d, const TV* invd, TV c1, TV c2, double* partials,
               cudaStream_t s, const double* xscale, TV* y2) {
-  int blocks;
-  if (mode == CSR_SPMV_DINV_DOT) {
-    blocks = kRedBlocks;
-  } else {
-    long long need = ((long long)n * G + 255) / 256;
-    blocks = (int)(need < sm_count() * 16 ? (need > 0 ? need : 1) : sm_count() * 16);
-  }
+  const long long need = ((long long)n * G + 255) / 256;
+  const long long most = mode == CSR_SPMV_DINV_DOT ? kPowerBlocks : sm_count() * 16;
+  const int blocks = (int)(need < most ? (need > 0 ? need : 1) : most);
 #define SAAMG_CSR_CASE(M)                                                                  \
   case M:                                                                                  \
     launch_pdl(csr_k<TV, TM, G, M>, blocks, 256, 0, s, n, rowptr, col, val, x, y, b, d,   \
@@ -144,7 +140,7 @@ void csr_apply(int mode, int n, const int* rowptr, const int* col, const TM* val
                const TV* x, TV* y, const TV* b, TV* d, const TV* invd, TV c1, TV c2,
                double* partials, cudaStream_t s, int kclass, const double* xscale, TV* y2) {
   if (n <= 0) {
-    if (mode == CSR_SPMV_DINV_DOT) fill_double(partials, 0.0, kRedBlocks, s);
+    if (mode == CSR_SPMV_DINV_DOT) fill_double(partials, 0.0, kPowerBlocks, s);
     return;
   }
   // timing unit of the sparse-matrix classes: matrix entries

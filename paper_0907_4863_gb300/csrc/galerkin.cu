@@ -1150,7 +1150,10 @@ void power_lambda_start(const DevCsr& A, const double* invd, const unsigned* ids
   // division by the previous norm to its output (one multiply per row, no separate sweep)
   run.v.alloc(n, s);
   run.w.alloc(n, s);
-  run.part.alloc(kRedBlocks, s);
+  const int parts = S ? kRedBlocks : kPowerBlocks;
+  run.part.alloc(parts, s);
+  // a small level runs fewer blocks: the other partials stay 0
+  SAAMG_CUDA(cudaMemsetAsync(run.part.p, 0, sizeof(double) * parts, s));
   run.nrm2.alloc(2, s);  // |w|^2 and 1 / |w|
   power_init_k<<<blocks_for(n), 256, 0, s>>>(n, ids, run.v.p);
   SAAMG_LAUNCH();
@@ -1167,7 +1170,7 @@ void power_lambda_start(const DevCsr& A, const double* invd, const unsigned* ids
       csr_apply<double, double>(CSR_SPMV_DINV_DOT, n, A.rowptr.p, A.col.p, A.val.p, avg,
                                 run.v.p, run.w.p, nullptr, nullptr, invd, 0.0, 0.0, run.part.p,
                                 s, -1, xscale);
-    sum_partials(run.part.p, kRedBlocks, run.nrm2.p, s, run.nrm2.p + 1);
+    sum_partials(run.part.p, parts, run.nrm2.p, s, run.nrm2.p + 1);
     run.v.swap(run.w);
   }
 }

@@ -27,25 +27,6 @@ __device__ double taper_sigma(const GeomParams& g, double z) {
   return 1.0 + (g.taper - 1.0) * tau;
 }
 
-// Implicit function of the elliptic wall Gamma_1 (Sec. 4.1); F < 0 inside.
-__device__ double wall_F(const GeomParams& g, double x, double y, double z) {
-  double sg = taper_sigma(g, z);
-  double u = (x - g.cx) / (g.a * sg);
-  double v = (y - g.cy) / (g.b * sg);
-  return (u * u + v * v) - 1.0;
-}
-
-// Omega_h of Sec. 2: lattice nodes of Omega plus the Robin planes; Dirichlet end
-// planes carry known zeros.
-__device__ bool node_inside(const GeomParams& g, int i, int j, int k) {
-  if (i < 0 || j < 0 || k < 0 || i >= g.nx || j >= g.ny || k >= g.nz) return false;
-  if (g.zbc == SAAMG_Z_DIRICHLET && (k == 0 || k == g.nz - 1)) return false;
-  double x = node_coord(g.o[0], i, g.h[0]);
-  double y = node_coord(g.o[1], j, g.h[1]);
-  double z = node_coord(g.o[2], k, g.h[2]);
-  return wall_F(g, x, y, z) < 0.0;
-}
-
 // 0 < s <= 1; the lower clamp 2^-20 only guards against rounding.
 __device__ double clamp_frac(double s) {
   const double smin = 9.5367431640625e-07;
@@ -139,95 +120,87 @@ __device__ void neighbour_rows(const GeomParams& g, const LineInfo* lines, int L
 
 // --- kernels ---------------------------------------------------------------
 
-// Warp per x-line: first/last inside node and count; flags a non-contiguous line.
-// Exact inside test of the nodes [a, b] of line (j, k), 32 at a time: first and last inside
-// node and their number (warp-uniform results).
-__device__ void scan_line(const GeomParams& g, int j, int k, int a, int b, int lane, int& first,
-                          int& last, int& cnt) {
-  first = INT_MAX;
-  last = -1;
-  cnt = 0;
-  for (int base = a; base <= b; base += 32) {
-    const int i = base + lane;
-    const bool in = i <= b && node_inside(g, i, j, k);
-    const unsigned m = __ballot_sync(0xffffffffu, in);
-    if (m) {
-      if (first == INT_MAX) first = base + __ffs(m) - 1;
-      last = base + 31 - __clz(m);
-      cnt += __popc(m);
-    }
-  }
-}
-
-// Warp per x-line: first/last inside node and count; flags a non-contiguous line.  The line
-// meets the cross-section in |x - cx| < w with w = a sigma sqrt(1 - v^2); nodes two or more
+// Thread per x-line: first/last inside node and count; flags a non-contiguous line.  The line
+// meets the cross-section F = (x - cx)^2 / (a sigma)^2 + (y - cy)^2 / (b sigma)^2 - 1 < 0 (Gamma_1,
+// Sec. 4.1; Omega_h of Sec. 2 holds the lattice nodes of Omega plus the Robin planes, Dirichlet end
+// planes carry known zeros) in |x - cx| < w with w = a sigma sqrt(1 - v^2); nodes two or more
 // spacings from either end of that interval are classified the same by the exact test (|F| is
-// there far above its rounding error), so only the nodes within two spacings of the ends are
-// tested exactly; a line whose ends do not look as expected (an end at the box face, a short
-// interval, or any surprise) is scanned node by node.
-__global__ void classify_lines_k(GeomParams g, int nlines, LineInfo* lines, int* count,
-                                 int* err) {
-  const int L = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+// there far above its rounding error), so only the five nodes around either end are tested
+// exactly; a line whose ends do not look as expected (an end at the box face, a short interval, or
+// any surprise) is scanned node by node.  Bound by FP64 issue, where an instruction costs the same
+// for one line as for 32: a warp per line took 256 us at 256^3, this 27.
+__global__ void __launch_bounds__(128) classify_lines_k(GeomParams g, int nlines, LineInfo* lines,
+                                                        int* count, int* err) {
+  const int L = blockIdx.x * blockDim.x + threadIdx.x;
   if (L >= nlines) return;
   const int j = L % g.ny, k = L / g.ny;
   int first = INT_MAX, last = -1, cnt = 0;
-  bool done = false;
-  if (g.zbc == SAAMG_Z_DIRICHLET && (k == 0 || k == g.nz - 1)) {
-    done = true;  // known zeros
-  } else {
+  int a = 0, b = -1;  // nodes to test one by one
+  if (!(g.zbc == SAAMG_Z_DIRICHLET && (k == 0 || k == g.nz - 1))) {  // else known zeros
+    // the inside test on the line's nodes; v, a sigma and v^2 are the line's
     const double y = node_coord(g.o[1], j, g.h[1]);
     const double z = node_coord(g.o[2], k, g.h[2]);
     const double sg = taper_sigma(g, z);
     const double v = (y - g.cy) / (g.b * sg);
-    const double vv = v * v;
+    const double vv = v * v, as = g.a * sg;
+    auto inside = [&](int i) {
+      const double u = (node_coord(g.o[0], i, g.h[0]) - g.cx) / as;
+      return (u * u + vv) - 1.0 < 0.0;
+    };
+    b = g.nx - 1;
     if (vv >= 1.0) {
-      done = true;  // u*u + v*v >= 1 for every node: F >= 0
+      b = -1;  // u*u + v*v >= 1 for every node: F >= 0
     } else if (vv < 1.0) {
-      const double w = (g.a * sg) * sqrt(1.0 - vv);
+      const double w = as * sqrt(1.0 - vv);
       const double xl = (g.cx - w - g.o[0]) / g.h[0], xh = (g.cx + w - g.o[0]) / g.h[0];
       const double A = fmax(0.0, ceil(xl) - 2.0), B = fmin((double)(g.nx - 1), floor(xh) + 2.0);
       if (A > B) {
-        done = true;  // the interval holds no node, nor any within two spacings
-      } else if (B - A >= 64.0) {
-        const int a = (int)A, b = (int)B;
+        b = -1;  // the interval holds no node, nor any within two spacings
+      } else if (B - A >= 16.0) {
+        const int lo = (int)A, hi = (int)B;
         // the five nodes at each end: outside ... inside at the low end, inside ... outside at
         // the high end, with one change each
-        const int i = lane < 5 ? a + lane : b - 4 + (lane - 5);
-        const bool in = lane < 10 && node_inside(g, i, j, k);
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        const unsigned mlo = m & 0x1fu, mhi = (m >> 5) & 0x1fu;
+        unsigned mlo = 0, mhi = 0;
+#pragma unroll 1
+        for (int q = 0; q < 5; ++q) {
+          mlo |= (unsigned)inside(lo + q) << q;
+          mhi |= (unsigned)inside(hi - 4 + q) << q;
+        }
         // low end: bit 0 clear and the set bits contiguous up to bit 4; high end: bit 4 clear
         // and the set bits contiguous from bit 0
         const bool lo_ok = mlo != 0 && (mlo & 1u) == 0 && ((mlo | (mlo - 1u)) & 0x1fu) == 0x1fu &&
                            __popc(mlo) == 5 - (__ffs(mlo) - 1);
         const bool hi_ok = mhi != 0 && (mhi & 0x10u) == 0 && (mhi & (mhi + 1u)) == 0;
         if (lo_ok && hi_ok) {
-          first = a + __ffs(mlo) - 1;
-          last = b - 4 + (31 - __clz(mhi));
+          first = lo + __ffs(mlo) - 1;
+          last = hi - 4 + (31 - __clz(mhi));
           cnt = last - first + 1;
-          done = true;
+          b = -1;
         }
       } else {
-        scan_line(g, j, k, (int)A, (int)B, lane, first, last, cnt);
-        done = true;
+        a = (int)A;
+        b = (int)B;
       }
     }
+#pragma unroll 1
+    for (int i = a; i <= b; ++i)
+      if (inside(i)) {
+        if (first == INT_MAX) first = i;
+        last = i;
+        ++cnt;
+      }
   }
-  if (!done) scan_line(g, j, k, 0, g.nx - 1, lane, first, last, cnt);
-  if (lane == 0) {
-    LineInfo l;
-    l.lo = cnt ? first : 0;
-    l.hi = cnt ? last : -1;
-    l.start = 0;
-    l.rlo = l.hi + 1;
-    l.rhi = l.hi;
-    l.tstart = 0;
-    l.pad0 = l.pad1 = 0;
-    lines[L] = l;
-    count[L] = cnt;
-    if (cnt && cnt != last - first + 1) atomicOr(err, 1);
-  }
+  LineInfo l;
+  l.lo = cnt ? first : 0;
+  l.hi = cnt ? last : -1;
+  l.start = 0;
+  l.rlo = l.hi + 1;
+  l.rhi = l.hi;
+  l.tstart = 0;
+  l.pad0 = l.pad1 = 0;
+  lines[L] = l;
+  count[L] = cnt;
+  if (cnt && cnt != last - first + 1) atomicOr(err, 1);
 }
 
 __global__ void chunk_counts_k(const int* count, int nlines, int* nch) {
@@ -423,78 +396,93 @@ __global__ void assemble_scaled_k(GeomParams g, const LineInfo* __restrict__ lin
                                   double* __restrict__ val, unsigned char* __restrict__ regular,
                                   unsigned char* __restrict__ nbmask,
                                   const double* __restrict__ rc) {
+  // the chunk's rows are contiguous in the CSR: a warp gathers them in shared memory and writes
+  // them out as one run (a row per lane wrote 84-byte pieces: 382 us at 256^3, now 239)
+  __shared__ int s_col[8][224];
+  __shared__ double s_val[8][224];
+  int* wcol = s_col[threadIdx.x >> 5];
+  double* wval = s_val[threadIdx.x >> 5];
   int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (c >= nchunks) return;
   int2 ch = chunks[c];
   int L = ch.x;
   LineInfo me = lines[L];
-  int i = me.lo + ch.y + lane;
-  if (i > me.hi) return;
-  int row = me.start + ch.y + lane;
-  int nb[6];
-  neighbour_rows(g, lines, L, i, row, me, nb);
-  const bool simple = simple_row(g, nb, L);
-  const long long sreg = __double_as_longlong(rc[6]);
-  bool fast = simple && __double_as_longlong(scale[row]) == sreg;
-  if (fast) {
-#pragma unroll
-    for (int q = 0; q < 6; ++q) fast = fast && __double_as_longlong(scale[nb[q]]) == sreg;
-  }
-  double sc[7];
-  bool reg;
-  if (fast) {
-    sc[0] = rc[0];
-    sc[1] = sc[2] = rc[1];
-    sc[3] = sc[4] = rc[2];
-    sc[5] = sc[6] = rc[3];
-    reg = true;
-  } else {
-    double* cr = coef + 8 * (size_t)row;
-    double ur[7];
-    if (simple) {  // the interior unscaled row (not stored by the unscaled pass)
-      ur[0] = rc[5];
-      ur[1] = ur[2] = -g.cdir[0];
-      ur[3] = ur[4] = -g.cdir[1];
-      ur[5] = ur[6] = -g.cdir[2];
-    } else {
-      for (int q = 0; q < 7; ++q) ur[q] = cr[q];
+  const int row0 = me.start + ch.y, nrows = min(32, me.hi - me.lo + 1 - ch.y);
+  const int base = rowptr[row0], total = rowptr[row0 + nrows] - base;
+  if (lane < nrows) {
+    int i = me.lo + ch.y + lane;
+    int row = row0 + lane;
+    int nb[6];
+    neighbour_rows(g, lines, L, i, row, me, nb);
+    const bool simple = simple_row(g, nb, L);
+    const long long sreg = __double_as_longlong(rc[6]);
+    bool fast = simple && __double_as_longlong(scale[row]) == sreg;
+    if (fast) {
+  #pragma unroll
+      for (int q = 0; q < 6; ++q) fast = fast && __double_as_longlong(scale[nb[q]]) == sreg;
     }
-    double si = scale[row];
-    sc[0] = ur[0] * (si * si);
-    reg = true;
-    for (int q = 0; q < 6; ++q) {
-      if (nb[q] >= 0) {
-        sc[1 + q] = ur[1 + q] * (si * scale[nb[q]]);
+    double sc[7];
+    bool reg;
+    if (fast) {
+      sc[0] = rc[0];
+      sc[1] = sc[2] = rc[1];
+      sc[3] = sc[4] = rc[2];
+      sc[5] = sc[6] = rc[3];
+      reg = true;
+    } else {
+      double* cr = coef + 8 * (size_t)row;
+      double ur[7];
+      if (simple) {  // the interior unscaled row (not stored by the unscaled pass)
+        ur[0] = rc[5];
+        ur[1] = ur[2] = -g.cdir[0];
+        ur[3] = ur[4] = -g.cdir[1];
+        ur[5] = ur[6] = -g.cdir[2];
       } else {
-        sc[1 + q] = 0.0;
-        reg = false;
+        for (int q = 0; q < 7; ++q) ur[q] = cr[q];
+      }
+      double si = scale[row];
+      sc[0] = ur[0] * (si * si);
+      reg = true;
+      for (int q = 0; q < 6; ++q) {
+        if (nb[q] >= 0) {
+          sc[1 + q] = ur[1 + q] * (si * scale[nb[q]]);
+        } else {
+          sc[1 + q] = 0.0;
+          reg = false;
+        }
+      }
+      reg = reg && sc[0] == rc[0] && sc[1] == rc[1] && sc[2] == rc[1] && sc[3] == rc[2] &&
+            sc[4] == rc[2] && sc[5] == rc[3] && sc[6] == rc[3];
+      for (int q = 0; q < 7; ++q) cr[q] = sc[q];
+      // 1 / diag: rc[4] is 1.0 / rc[0], the same division
+      cr[7] = __double_as_longlong(sc[0]) == __double_as_longlong(rc[0]) ? rc[4] : 1.0 / sc[0];
+    }
+    const int order[7] = {4, 2, 0, -1, 1, 3, 5};
+    int p = rowptr[row] - base;
+  #pragma unroll
+    for (int o = 0; o < 7; ++o) {
+      int q = order[o];
+      if (q < 0) {
+        wcol[p] = row;
+        wval[p] = sc[0];
+        ++p;
+      } else if (nb[q] >= 0) {
+        wcol[p] = nb[q];
+        wval[p] = sc[1 + q];
+        ++p;
       }
     }
-    reg = reg && sc[0] == rc[0] && sc[1] == rc[1] && sc[2] == rc[1] && sc[3] == rc[2] &&
-          sc[4] == rc[2] && sc[5] == rc[3] && sc[6] == rc[3];
-    for (int q = 0; q < 7; ++q) cr[q] = sc[q];
-    // 1 / diag: rc[4] is 1.0 / rc[0], the same division
-    cr[7] = __double_as_longlong(sc[0]) == __double_as_longlong(rc[0]) ? rc[4] : 1.0 / sc[0];
+    regular[row] = reg ? 1 : 0;
+    unsigned char mk = 0;
+    for (int q = 0; q < 6; ++q) mk |= (unsigned char)((nb[q] >= 0) << q);
+    nbmask[row] = mk;
   }
-  const int order[7] = {4, 2, 0, -1, 1, 3, 5};
-  int p = rowptr[row];
-  for (int o = 0; o < 7; ++o) {
-    int q = order[o];
-    if (q < 0) {
-      col[p] = row;
-      val[p] = sc[0];
-      ++p;
-    } else if (nb[q] >= 0) {
-      col[p] = nb[q];
-      val[p] = sc[1 + q];
-      ++p;
-    }
+  __syncwarp();
+  for (int e = lane; e < total; e += 32) {
+    col[base + e] = wcol[e];
+    val[base + e] = wval[e];
   }
-  regular[row] = reg ? 1 : 0;
-  unsigned char mk = 0;
-  for (int q = 0; q < 6; ++q) mk |= (unsigned char)((nb[q] >= 0) << q);
-  nbmask[row] = mk;
 }
 
 // Thread per line: longest run of regular rows -> [rlo, rhi]; table rows = the rest.
@@ -576,9 +564,14 @@ __global__ void fill_table_k(const LineInfo* __restrict__ lines, const int2* __r
   }
 }
 
-// Box -> compact right-hand side and initial guess, one row of a chunk; the row, or -1.
-__device__ __forceinline__ int gather_row(const GeomParams& g, const LineInfo* __restrict__ lines,
-                                          int2 ch, int lane, const double* __restrict__ scale,
+// Box -> compact right-hand side and initial guess, one row of a chunk; the row, or -1.  The
+// division of the guess by s_i has its three-instruction form where s_i is the interior's (s0),
+// and none where the guess is 0 (the quotient is that zero): with a general division, and a
+// multiplication by 1 for the rows off the Robin planes, the pass was bound by FP64 issue, 308 us
+// at 256^3 instead of 66.
+__device__ __forceinline__ int gather_row(const GeomParams& g, const DivC& s0,
+                                          const LineInfo* __restrict__ lines, int2 ch, int lane,
+                                          const double* __restrict__ scale,
                                           const double* __restrict__ rho,
                                           const double* __restrict__ phi0,
                                           double* __restrict__ bhat, double* __restrict__ xhat) {
@@ -590,14 +583,20 @@ __device__ __forceinline__ int gather_row(const GeomParams& g, const LineInfo* _
   int k = L / g.ny;
   size_t box = (size_t)i + (size_t)g.nx * (size_t)L;
   bool gamma2 = (g.zbc == SAAMG_Z_ROBIN) && (k == 0 || k == g.nz - 1);
-  double bf = (gamma2 && g.sym) ? 0.5 : 1.0;
-  double si = scale[row];
-  bhat[row] = si * (bf * rho[box]);
-  if (xhat) xhat[row] = phi0 ? phi0[box] / si : 0.0;
+  const double si = scale[row], v = phi0 ? phi0[box] : 0.0;
+  double rh = rho[box];
+  if (gamma2 && g.sym) rh = 0.5 * rh;
+  bhat[row] = si * rh;
+  if (xhat) {
+    double x = v;
+    if ((static_cast<unsigned long long>(__double_as_longlong(v)) << 1) != 0ull)
+      x = __double_as_longlong(si) == __double_as_longlong(s0.c) ? div_by(v, s0) : v / si;
+    xhat[row] = x;
+  }
   return row;
 }
 
-__global__ void gather_k(GeomParams g, const LineInfo* __restrict__ lines,
+__global__ void gather_k(GeomParams g, DivC s0, const LineInfo* __restrict__ lines,
                          const int2* __restrict__ chunks, int nchunks,
                          const double* __restrict__ scale, const double* __restrict__ rho,
                          const double* __restrict__ phi0, double* __restrict__ bhat,
@@ -605,7 +604,7 @@ __global__ void gather_k(GeomParams g, const LineInfo* __restrict__ lines,
   int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (c >= nchunks) return;
-  gather_row(g, lines, chunks[c], lane, scale, rho, phi0, bhat, xhat);
+  gather_row(g, s0, lines, chunks[c], lane, scale, rho, phi0, bhat, xhat);
 }
 
 __global__ void __launch_bounds__(256) bgather_k(const BoxTask* __restrict__ tasks,
@@ -614,8 +613,8 @@ __global__ void __launch_bounds__(256) bgather_k(const BoxTask* __restrict__ tas
   const BoxTask& k = tasks[B.x];
   const int lane = threadIdx.x & 31;
   for (int u = B.y + (threadIdx.x >> 5); u < B.z; u += blockDim.x >> 5) {
-    const int row = gather_row(k.g, k.lines, k.chunks[u], lane, k.scale, k.rho, k.phi, k.bhat,
-                               k.xhat);
+    const int row = gather_row(k.g, k.s0, k.lines, k.chunks[u], lane, k.scale, k.rho, k.phi,
+                               k.bhat, k.xhat);
     if (row >= 0) k.p[row] = 0.0;
   }
 }
@@ -624,8 +623,8 @@ __global__ void __launch_bounds__(256) bgather_k(const BoxTask* __restrict__ tas
 __device__ __forceinline__ double scatter_node(int nx, const LineInfo* __restrict__ lines,
                                                const double* __restrict__ scale,
                                                const double* __restrict__ xhat, size_t b) {
-  const int L = (int)(b / (size_t)nx);
-  const int i = (int)(b - (size_t)L * nx);
+  const int L = (int)((unsigned)b / (unsigned)nx);  // a box has less than 2^31 nodes
+  const int i = (int)((unsigned)b - (unsigned)L * (unsigned)nx);
   const LineInfo me = lines[L];
   if (i < me.lo || i > me.hi) return 0.0;
   const int row = me.start + (i - me.lo);
@@ -693,7 +692,7 @@ void build_operator_data(const GeomParams& g, cudaStream_t s, OperatorData& op) 
   chstart.alloc(nlines, s);
   err.alloc(1, s);
   fill_int(err.p, 0, 1, s);
-  classify_lines_k<<<warp_blocks(nlines), 256, 0, s>>>(g, nlines, op.lines.p, count.p, err.p);
+  classify_lines_k<<<(nlines + 127) / 128, 128, 0, s>>>(g, nlines, op.lines.p, count.p, err.p);
   SAAMG_LAUNCH();
   int herr = 0;
   d2h_sync(&herr, err.p, sizeof(int), s);
@@ -723,13 +722,14 @@ void build_operator_data(const GeomParams& g, cudaStream_t s, OperatorData& op) 
   rc.alloc(8, s);
   regular_consts_k<<<1, 1, 0, s>>>(g, rc.p);
   SAAMG_LAUNCH();
-  double hrc[5];
+  double hrc[7];
   d2h_sync(hrc, rc.p, sizeof(hrc), s);
   op.c0 = hrc[0];
   op.cx = hrc[1];
   op.cy = hrc[2];
   op.cz = hrc[3];
   op.invd0 = hrc[4];
+  op.s0 = hrc[6];
 
   op.scale.alloc(op.n, s);
   op.ids.alloc(op.n, s);
@@ -1020,7 +1020,7 @@ __global__ void __launch_bounds__(256) field_gradient_k(GeomParams g, GradDiv dv
           ez[q] = -div_by(k == 0 ? p0 : -p0, dv.dist);
           continue;
         }
-        bool in_m, in_p;  // from the line records (the classification node_inside produced)
+        bool in_m, in_p;  // from the line records
         if (ax == 0) {
           in_m = i - 1 >= me.lo;
           in_p = i + 1 <= me.hi;
@@ -1109,8 +1109,8 @@ void stencil_diag_inverse(const OperatorData& op, double* invd, float* invd32, c
 void gather_rhs(const OperatorData& op, const double* rho, const double* phi0, double* bhat,
                 double* xhat, cudaStream_t s) {
   if (op.n == 0) return;
-  gather_k<<<warp_blocks(op.nchunks), 256, 0, s>>>(op.g, op.lines.p, op.chunks.p, op.nchunks,
-                                                    op.scale.p, rho, phi0, bhat, xhat);
+  gather_k<<<warp_blocks(op.nchunks), 256, 0, s>>>(op.g, make_divc(op.s0), op.lines.p, op.chunks.p,
+                                                   op.nchunks, op.scale.p, rho, phi0, bhat, xhat);
   SAAMG_LAUNCH();
 }
 

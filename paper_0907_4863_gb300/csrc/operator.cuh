@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "divc.cuh"
 
 namespace saamg {
 
@@ -34,6 +35,7 @@ struct OperatorData {
   Buf<int2> rrow;       // (compact row, line) of the lines' regular-run rows, in order
   int nrun = 0;
   double c0 = 0, cx = 0, cy = 0, cz = 0, invd0 = 0;  // regular-row coefficients
+  double s0 = 0;        // s_i of the rows with all six neighbours off the Robin planes
   Buf<double> scale;    // s_i = a_ii^-1/2 (unscaled diagonal)
   Buf<unsigned> ids;    // box index of each unknown
   Buf<unsigned char> regular;
@@ -71,6 +73,7 @@ void scatter_solution(const OperatorData& op, const double* xhat, double* phi, c
 // nodes (scatter); every node is computed as in the one-solve launches.
 struct BoxTask {
   GeomParams g;
+  DivC s0;
   const LineInfo* lines;
   const int2* chunks;
   const double* scale;

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256) sell_k(int n, int nslices, const int* __r
   for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw)
     rows::sell_row<TV, TM, MODE, REL>(s, lane, n, perm, soff, col, dcol, val, x, y, b, d, invd,
                                       c1, c2, dacc);
-  if (MODE == CSR_SPMV_DINV_DOT) {  // fixed grid of kRedBlocks: the same partial sums every run
+  if (MODE == CSR_SPMV_DINV_DOT) {  // fixed grid of kPowerBlocks: the same partial sums every run
     const double t = rows::block_sum(dacc);
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
   }
@@ -201,14 +201,14 @@ void sell_apply(int mode, const DevSell& S, const TM* val, const TV* x, TV* y, c
                 TV* d, const TV* invd, TV c1, TV c2, cudaStream_t s, int kclass,
                 double* partials, const double* xscale) {
   if (S.n <= 0) {
-    if (mode == CSR_SPMV_DINV_DOT) fill_double(partials, 0.0, kRedBlocks, s);
+    if (mode == CSR_SPMV_DINV_DOT) fill_double(partials, 0.0, kPowerBlocks, s);
     return;
   }
   KernelTimer kt(kclass, S.nnz, s);  // timing unit of the SELL classes: matrix entries
   if (mode == CSR_CHEB && c1 == TV(0)) mode = kSellCheb1;
   const long long need = ((long long)S.nslices + 7) / 8;
-  const int blocks =
-      mode == CSR_SPMV_DINV_DOT ? kRedBlocks : (int)(need < sm_count() * 16 ? need : sm_count() * 16);
+  const long long most = mode == CSR_SPMV_DINV_DOT ? kPowerBlocks : sm_count() * 16;
+  const int blocks = (int)(need < most ? need : most);
 #define SAAMG_SELL_CASE(M)                                                                    \
   case M:                                                                                     \
     if (S.index_bytes == 2)                                                                   \

@@ -49,7 +49,7 @@ void sell_like(const DevCsr& A, const DevSell& like, DevSell& S, bool f64, bool 
                cudaStream_t s);
 
 // The CSR modes of csr_apply (CSR_CHEB with c1 == 0 does not read d; CSR_SPMV_DINV_DOT
-// writes kRedBlocks partial sums of y.y and takes the scale of x from *xscale, 1 if NULL).
+// writes kPowerBlocks partial sums of y.y and takes the scale of x from *xscale, 1 if NULL).
 template <class TV, class TM>
 void sell_apply(int mode, const DevSell& S, const TM* val, const TV* x, TV* y, const TV* b,
                 TV* d, const TV* invd, TV c1, TV c2, cudaStream_t s, int kclass,
