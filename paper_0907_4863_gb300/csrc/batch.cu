@@ -303,14 +303,14 @@ __global__ void __launch_bounds__(kRedThreads) bbeta_k(const VTask* __restrict__
   if (!*k.go) return;
   const double rz = rows::sum_fixed(k.part0, kRedBlocks);
   const double zq = k.rule == 1 ? rows::sum_fixed(k.part2, kRedBlocks) : 0.0;
-  if (threadIdx.x == 0) finish_beta(k.ctl, rz, zq, k.rule);
+  if (threadIdx.x == 0) finish_beta(k.ctl, rz, zq, k.rule, BetaIn(k.ctl));
 }
 
 __global__ void __launch_bounds__(kRedThreads) balpha_k(const VTask* __restrict__ tasks) {
   const VTask& k = tasks[blockIdx.x];
   if (!*k.go) return;
   const double pq = rows::sum_fixed(k.partq, kRedBlocks);
-  if (threadIdx.x == 0) finish_alpha(k.ctl, pq);
+  if (threadIdx.x == 0) finish_alpha(k.ctl, pq, k.ctl->rz);
 }
 
 __global__ void __launch_bounds__(kRedThreads) bcheck_k(const VTask* __restrict__ tasks) {

@@ -61,12 +61,16 @@ template <class TV, class TM, int G>
 void launch_g(int mode, int n, const int* rowptr, const int* col, const TM* val, const TV* x,
               TV* y, const TV* b, TV* d, const TV* invd, TV c1, TV c2, double* partials,
               cudaStream_t s, const double* xscale, TV* y2) {
-  const long long need = ((long long)n * G + 255) / 256;
+  // a small level spreads over the SMs in blocks of 64 threads (an SM takes FP64 instructions of
+  // one warp per quarter at a time)
+  const int block =
+      mode != CSR_SPMV_DINV_DOT && (long long)n * G < sm_count() * 256LL ? 64 : 256;
+  const long long need = ((long long)n * G + block - 1) / block;
   const long long most = mode == CSR_SPMV_DINV_DOT ? kPowerBlocks : sm_count() * 16;
   const int blocks = (int)(need < most ? (need > 0 ? need : 1) : most);
 #define SAAMG_CSR_CASE(M)                                                                  \
   case M:                                                                                  \
-    launch_pdl(csr_k<TV, TM, G, M>, blocks, 256, 0, s, n, rowptr, col, val, x, y, b, d,   \
+    launch_pdl(csr_k<TV, TM, G, M>, blocks, block, 0, s, n, rowptr, col, val, x, y, b, d,   \
                invd, c1, c2, partials, xscale, y2);                                        \
     break;
   switch (mode) {

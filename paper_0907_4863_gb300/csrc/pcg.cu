@@ -46,9 +46,10 @@ __global__ void __launch_bounds__(kRedThreads) beta_k(int n, const double* __res
     if (PR) part_zq[blockIdx.x] = t2;
   }
   if (!last_block(&ctl->tick[0])) return;
+  const BetaIn in(ctl);
   const double rz = sum_fixed(part_rz, gridDim.x);
   const double zq = PR ? sum_fixed(part_zq, gridDim.x) : 0.0;
-  if (threadIdx.x == 0) finish_beta(ctl, rz, zq, PR ? 1 : 0);
+  if (threadIdx.x == 0) finish_beta(ctl, rz, zq, PR ? 1 : 0, in);
 }
 
 // r32 (mixed precision): the FP32 copy of the new residual, the next V-cycle's input

@@ -25,10 +25,10 @@ struct PcgCtl {
 };
 
 // --- CG scalars, on the device -------------------------------------------------------------
-// alpha = rz / pq (breakdown flag on 0/NaN)
-__device__ __forceinline__ void finish_alpha(PcgCtl* ctl, double pq) {
+// alpha = rz / pq (breakdown flag on 0/NaN); rz: ctl->rz
+__device__ __forceinline__ void finish_alpha(PcgCtl* ctl, double pq, double rz) {
   ctl->pq = pq;
-  double a = ctl->rz / pq;
+  double a = rz / pq;
   if (!(pq != 0.0) || !isfinite(a)) {
     ctl->breakdown = 1;
     a = 0.0;
@@ -36,9 +36,16 @@ __device__ __forceinline__ void finish_alpha(PcgCtl* ctl, double pq) {
   ctl->alpha = a;
 }
 // beta: 0 on the first pass (p = z), else rz_new / rz (rule 0) or -alpha zq / rz (rule 1)
-__device__ __forceinline__ void finish_beta(PcgCtl* ctl, double rz, double zq, int rule) {
+struct BetaIn {  // read before the sums
+  int iters;
+  double alpha, rz;
+  __device__ __forceinline__ explicit BetaIn(const PcgCtl* c)
+      : iters(c->iters), alpha(c->alpha), rz(c->rz) {}
+};
+__device__ __forceinline__ void finish_beta(PcgCtl* ctl, double rz, double zq, int rule,
+                                            const BetaIn& in) {
   double b = 0.0;
-  if (ctl->iters > 0) b = (rule == 1) ? (-ctl->alpha * zq) / ctl->rz : rz / ctl->rz;
+  if (in.iters > 0) b = (rule == 1) ? (-in.alpha * zq) / in.rz : rz / in.rz;
   if (!isfinite(b) || !isfinite(rz)) {
     ctl->breakdown = 1;
     b = 0.0;

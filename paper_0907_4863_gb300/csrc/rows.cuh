@@ -290,33 +290,33 @@ __device__ __forceinline__ void gemv_row(int i, int n, int lane, const double* _
 }
 
 // --- reductions -----------------------------------------------------------------------------
-// Sum over the block, valid in thread 0 (warp shuffles, then the warps in order).
+// The tail of a reduction is a chain of dependent FP64 additions (66 clocks each) and barriers (40):
+// shuffles inside the warps, one barrier, shuffles over the warps' sums.
+__device__ __forceinline__ double warp_tree(double v, int width) {
+  for (int o = width / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sum over the block (a power of two of warps), valid in the threads of warp 0.
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sh[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int nw = (int)(blockDim.x >> 5);
+  v = warp_tree(v, 32);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
   double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
+  if (threadIdx.x < 32) t = warp_tree((int)threadIdx.x < nw ? sh[threadIdx.x] : 0.0, nw);
   return t;
 }
 
-// Ordered sum of `count` partials by one block of kRedThreads threads, valid in all threads.  The
-// partials are read through L2: blocks of the same launch may have written them.
+// Ordered sum of `count` partials by one block, valid in the threads of warp 0.  The partials are
+// read through L2: blocks of the same launch may have written them.
 __device__ __forceinline__ double sum_fixed(const double* part, int count) {
-  __shared__ double sh[kRedThreads];
   double acc = 0.0;
+#pragma unroll 4
   for (int i = threadIdx.x; i < count; i += blockDim.x) acc += __ldcg(part + i);
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  double r = sh[0];
-  __syncthreads();
-  return r;
+  __syncthreads();  // block_sum's shared array may still be read from an earlier sum
+  return block_sum(acc);
 }
 
 // Block `blk` of a fixed grid of kRedBlocks x kRedThreads: its partial of sum a_i b_i (loads
@@ -413,15 +413,16 @@ __device__ __forceinline__ double update_block(int blk, int n, double a, double*
 // --- the same blocks emulated by one warp ---------------------------------------------------
 // A warp can stand in for a block of kRedThreads = 8 x 32 threads: lane l holds the accumulators
 // of the block's threads 32 w + l (w = 0..7, the block's warps), every accumulator is reduced by
-// the warp's xor tree (the block's per-warp reduction), and the eight sums are added in warp
-// order (the block's final loop).  The result has the bits of the block's partial, in every
+// the warp's xor tree (the block's per-warp reduction), and the eight sums by the block's tree
+// over its warps.  The result has the bits of the block's partial, in every
 // lane, without shared memory or barriers, and eight of these run side by side in a block.
 constexpr int kVirtWarps = kRedThreads / 32;
 
 // The eight xor trees (16, 8, 4, 2, 1) at once: at the first three levels a lane keeps half of its
 // accumulators and passes the other half on, so a tree level is 4, 2, 1, 1, 1 additions for all
 // eight instead of 8 each (an FP64 instruction holds a quarter of the SM for 64 clocks, whatever
-// its lanes do); each sum adds the same two numbers as the plain tree.
+// its lanes do); each sum adds the same two numbers as the plain tree.  Lane bits 4, 3 and 2 then
+// hold the warp's number, and three more levels are the block's sum over its warps.
 __device__ __forceinline__ double warp_tree8(const double v[kVirtWarps], int lane) {
   double u[4], w[2];
   const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
@@ -432,13 +433,9 @@ __device__ __forceinline__ double warp_tree8(const double v[kVirtWarps], int lan
   for (int q = 0; q < 2; ++q)
     w[q] = (h8 ? u[q + 2] : u[q]) + __shfl_xor_sync(0xffffffffu, h8 ? u[q] : u[q + 2], 8);
   double s = (h4 ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, h4 ? w[0] : w[1], 4);
-  s += __shfl_xor_sync(0xffffffffu, s, 2);
-  s += __shfl_xor_sync(0xffffffffu, s, 1);
-  double t = 0.0;
 #pragma unroll
-  for (int a = 0; a < kVirtWarps; ++a)
-    t += __shfl_sync(0xffffffffu, s, ((a >> 2) & 1) * 16 + ((a >> 1) & 1) * 8 + (a & 1) * 4);
-  return t;
+  for (int o : {2, 1, 16, 8, 4}) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 
 // f(i, w) for every element i of the block's threads 32 w + lane, in each thread's order

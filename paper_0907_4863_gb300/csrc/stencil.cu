@@ -271,20 +271,13 @@ __global__ void __launch_bounds__(256) stencil_k(StencilDev<T> S, const T* __res
     }
   }
   if (MODE == ST_SPMV_DOT || MODE == ST_DINV_DOT) {
-    __shared__ double sh[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dacc += __shfl_xor_sync(0xffffffffu, dacc, o);
-    if (lane == 0) sh[threadIdx.x >> 5] = dacc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < wpb; ++w) t += sh[w];
-      partials[blockIdx.x] = t;
-    }
+    const double t = rows::block_sum(dacc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = t;
     if (MODE == ST_SPMV_DOT && ctl) {  // CG: the last block adds the partials and forms alpha
       if (!last_block(&ctl->tick[1])) return;
+      const double rz = ctl->rz;
       const double pq = rows::sum_fixed(partials, gridDim.x);
-      if (threadIdx.x == 0) finish_alpha(ctl, pq);
+      if (threadIdx.x == 0) finish_alpha(ctl, pq, rz);
     }
   }
 }
@@ -450,12 +443,16 @@ template <class T, int MODE>
 void launch_shaped(const StencilCfg& cfg, long long units, int blocks_cap, const StencilDev<T>& S,
                    const T* x, T* y, const T* b, T* d, T c1, T c2, T c2i0, double* partials,
                    const double* xscale, const int* agg, cudaStream_t s) {
-  const int wpb = cfg.block / 32;
+  // a small level spreads over the SMs in smaller blocks (an SM takes FP64 instructions of one
+  // warp per quarter at a time)
+  int block = cfg.block;
+  while (block > 64 && units * 32 < (long long)sm_count() * block) block >>= 1;
+  const int wpb = block / 32;
   const long long need = (units + (long long)wpb * cfg.k - 1) / ((long long)wpb * cfg.k);
   const int blocks = (int)std::max<long long>(1, std::min<long long>(need, blocks_cap));
 #define SAAMG_SHAPE(KK, PP)                                                                  \
   if (cfg.k == KK && (cfg.packed != 0) == PP) {                                              \
-    launch_pdl(stencil_k<T, MODE, KK, PP>, blocks, cfg.block, 0, s, S, x, y, b, d, c1, c2,   \
+    launch_pdl(stencil_k<T, MODE, KK, PP>, blocks, block, 0, s, S, x, y, b, d, c1, c2,       \
                c2i0, partials, xscale, agg, (PcgCtl*)nullptr);                               \
     return;                                                                                  \
   }
