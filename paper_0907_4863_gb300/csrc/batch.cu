@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256, 5) bdirection_k(const VTask* __restrict__
     const TZ* z = (const TZ*)k.z;
     for (int u = B.y; u < B.z; ++u) {
       const int i = u * 256 + threadIdx.x;
-      if (i < k.n) k.p[i] = (double)z[i] + beta * k.p[i];
+      if (i < k.n) k.p[i] = rows::widen(z[i]) + beta * k.p[i];
     }
   }
 }

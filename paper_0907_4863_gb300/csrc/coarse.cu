@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kGjThreads)
                int* __restrict__ step, int* __restrict__ prow, int* __restrict__ err) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
+  asm volatile("griddepcontrol.wait;" ::: "memory");               // the update before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the update beside this panel
   constexpr int B = kGjB;
   struct Cand {
@@ -562,7 +563,8 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
   const int rpt = (n + rt - 1) / rt;
   const dim3 ugrid((n + cpb - 1) / cpb, rt);
   // panel q reads the matrix before update q - 1 and the panel q - 1; update q the same matrix as
-  // panel q + 1, and the panel q.  A panel is launched plainly: everything before it has finished.
+  // panel q + 1, and the panel q.  Panel q waits at its entry for the launch before it, update
+  // q - 2, which ends after panel q - 1 beside it: everything before has finished.
   const int panels = (n + B - 1) / B;
   auto panel = [&](int q) {
     const int pq = (q & 1) ^ 1;
@@ -571,12 +573,14 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
     cfg.blockDim = kGjThreads;
     cfg.dynamicSmemBytes = kGjPanelSmem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kGjCluster;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     SAAMG_CUDA(cudaLaunchKernelEx(&cfg, gj_panel_k, n, q * B, rpb, (const double*)w.p,
                                   q > 0 ? B : 0, (const GjPanel*)pn[pq].p, (const double*)c[pq].p,
                                   pn[q & 1].p, c[q & 1].p, (const int*)step[pq].p, step[q & 1].p,

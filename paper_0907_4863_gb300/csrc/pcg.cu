@@ -78,7 +78,7 @@ __global__ void direction_k(int n, const TZ* __restrict__ z, double* __restrict_
   pdl_wait();
   const double b = ctl->beta;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = (double)z[i] + b * p[i];
+    p[i] = rows::widen(z[i]) + b * p[i];
 }
 
 __global__ void init_k(const double* __restrict__ part_bb, const double* __restrict__ part_rr,
