@@ -41,6 +41,7 @@ constexpr int kLaneSolves = 32;   // solves per lane (about)
 // --- tasks ----------------------------------------------------------------------------------
 struct MTask {  // a sparse-matrix, coarse-solve or copy operation of one solve
   const int* go;
+  int g;        // CSR: lanes per row
   int n;        // rows (CSR, SELL, coarse inverse) or elements (copy)
   int nslices;  // SELL
   const int* rowptr;
@@ -85,38 +86,38 @@ struct VTask {  // the CG recursion of one solve
   if (!*k.go) continue;
 
 // --- sparse-matrix kernels --------------------------------------------------------------------
-template <class TV, class TM, int G, int MODE>
-__global__ void __launch_bounds__(256, 4) bcsr_k(const MTask* __restrict__ tasks,
+// Tasks of one mode, each with its own lanes per row G: one launch for solves of every size.
+template <class TV, class TM, int MODE>
+__global__ void __launch_bounds__(256, sizeof(TV) == 8 ? 3 : 4) bcsr_k(const MTask* __restrict__ tasks,
                                               const int4* __restrict__ wbs, int nwb) {
-  const int lane = threadIdx.x & 31, gl = lane % G, warp = threadIdx.x >> 5;
-  constexpr int kRows = 32 / G;
-  double dacc = 0.0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int wb = blockIdx.x; wb < nwb; wb += gridDim.x) {
     SAAMG_WORK_BLOCK(MTask)
-    if (MODE == CSR_CHEB0) {
+    const int G = k.g, rpw = 32 / G, gl = lane & (G - 1);
+    if (MODE == CSR_CHEB0) {  // a lane per row would do; the units are those of the level's G
       for (int u = B.y + warp; u < B.z; u += kWarps) {
-        const int row = u * kRows + lane / G;
-        rows::csr_group_row<TV, TM, G, MODE>(row, row < k.n, gl, k.rowptr, k.col,
-                                             (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
-                                             (const TV*)k.b, (TV*)k.d, (const TV*)k.invd, (TV)k.c1,
-                                             (TV)k.c2, dacc);
-      }
-    } else {
-      // four row groups a warp step, their loads in flight together
-      constexpr int NR = G < 4 ? G : 4;
-      for (int u = B.y + warp; u < B.z; u += NR * kWarps) {
-        int row[NR];
-        bool active[NR];
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          row[q] = (u + q * kWarps) * kRows + lane / G;
-          active[q] = u + q * kWarps < B.z && row[q] < k.n;
+        const int row = u * rpw + lane / G;
+        if (row < k.n && gl == 0) {
+          const TV w = (TV)k.c2 * (((const TV*)k.invd)[row] * ((const TV*)k.b)[row]);
+          ((TV*)k.d)[row] = w;
+          ((TV*)k.y)[row] = w;
         }
-        rows::csr_group_rows<TV, TM, G, MODE, NR>(row, active, gl, k.rowptr, k.col,
-                                                  (const TM*)k.val, (const TV*)k.x, (TV*)k.y,
-                                                  (const TV*)k.b, (TV*)k.d, (const TV*)k.invd,
-                                                  (TV)k.c1, (TV)k.c2, (TV*)k.y2);
       }
+      continue;
+    }
+    // four row groups a warp step (two with G = 2), their loads in flight together
+    const int nr = G < 4 ? 2 : 4;
+    for (int u = B.y + warp; u < B.z; u += nr * kWarps) {
+      int row[4];
+      bool active[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        row[q] = (u + q * kWarps) * rpw + lane / G;
+        active[q] = q < nr && u + q * kWarps < B.z && row[q] < k.n;
+      }
+      rows::csr_group_rows<TV, TM, MODE>(row, active, gl, G, k.rowptr, k.col, (const TM*)k.val,
+                                         (const TV*)k.x, (TV*)k.y, (const TV*)k.b, (TV*)k.d,
+                                         (const TV*)k.invd, (TV)k.c1, (TV)k.c2, (TV*)k.y2);
     }
   }
 }
@@ -336,9 +337,9 @@ __global__ void bany_k(const int* __restrict__ go, int count, cudaGraphCondition
 enum Family { F_ST32, F_ST64, F_CSR, F_SHORT, F_SELL, F_GEMV, F_COPY };
 // value types: TV 0 double / 1 float; TM 0 double / 1 float / 2 bf16
 struct Key {
-  int fam = 0, tv = 0, tm = 0, g = 0, mode = 0, rel = 0;
+  int fam = 0, tv = 0, tm = 0, mode = 0, rel = 0;
   bool operator<(const Key& o) const {
-    return std::tie(fam, tv, tm, g, mode, rel) < std::tie(o.fam, o.tv, o.tm, o.g, o.mode, o.rel);
+    return std::tie(fam, tv, tm, mode, rel) < std::tie(o.fam, o.tv, o.tm, o.mode, o.rel);
   }
   bool operator==(const Key& o) const {
     return !(*this < o) && !(o < *this);
@@ -368,29 +369,18 @@ inline int grid_wb(int nwb, const void* kernel) {
 #define SAAMG_WB_LAUNCH(KERNEL)                                                        \
   KERNEL<<<grid_wb(nwb, reinterpret_cast<const void*>(KERNEL)), 256, 0, s>>>(t, wbs, nwb)
 
-template <class TV, class TM, int G>
-void launch_csr_g(int mode, const MTask* t, const int4* wbs, int nwb, cudaStream_t s) {
+template <class TV, class TM>
+void launch_csr(int mode, const MTask* t, const int4* wbs, int nwb, cudaStream_t s) {
   switch (mode) {
-    case CSR_SPMV: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_SPMV>)); break;
-    case CSR_SPMV_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_SPMV_CHEB0>)); break;
-    case CSR_RESID: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_RESID>)); break;
-    case CSR_CHEB: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_CHEB>)); break;
-    case CSR_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_CHEB0>)); break;
-    case CSR_ADD: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, G, CSR_ADD>)); break;
+    case CSR_SPMV: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_SPMV>)); break;
+    case CSR_SPMV_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_SPMV_CHEB0>)); break;
+    case CSR_RESID: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_RESID>)); break;
+    case CSR_CHEB: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_CHEB>)); break;
+    case CSR_CHEB0: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_CHEB0>)); break;
+    case CSR_ADD: SAAMG_WB_LAUNCH((bcsr_k<TV, TM, CSR_ADD>)); break;
     default: fail(SAAMG_EINVAL, "batched CSR mode");
   }
   SAAMG_LAUNCH();
-}
-
-template <class TV, class TM>
-void launch_csr(int g, int mode, const MTask* t, const int4* wbs, int nwb, cudaStream_t s) {
-  switch (g) {
-    case 2: launch_csr_g<TV, TM, 2>(mode, t, wbs, nwb, s); break;
-    case 4: launch_csr_g<TV, TM, 4>(mode, t, wbs, nwb, s); break;
-    case 8: launch_csr_g<TV, TM, 8>(mode, t, wbs, nwb, s); break;
-    case 16: launch_csr_g<TV, TM, 16>(mode, t, wbs, nwb, s); break;
-    default: launch_csr_g<TV, TM, 32>(mode, t, wbs, nwb, s); break;
-  }
 }
 
 template <class TV, class TM, bool REL>
@@ -430,9 +420,9 @@ void launch_group(const Key& k, const void* tasks, const int4* wbs, int nwb, cud
       batched_stencil<double>(k.mode, static_cast<const StTask<double>*>(tasks), wbs, nwb, s);
       return;
     case F_CSR:
-      if (k.tv == 0) launch_csr<double, double>(k.g, k.mode, mt, wbs, nwb, s);
-      else if (k.tm == 1) launch_csr<float, float>(k.g, k.mode, mt, wbs, nwb, s);
-      else launch_csr<float, __nv_bfloat16>(k.g, k.mode, mt, wbs, nwb, s);
+      if (k.tv == 0) launch_csr<double, double>(k.mode, mt, wbs, nwb, s);
+      else if (k.tm == 1) launch_csr<float, float>(k.mode, mt, wbs, nwb, s);
+      else launch_csr<float, __nv_bfloat16>(k.mode, mt, wbs, nwb, s);
       return;
     case F_SHORT:
       if (k.tv == 0) launch_short<double, double>(k.mode, mt, wbs, nwb, s);
@@ -609,7 +599,7 @@ struct Planner {
       const int g = csr_plan(mode0, L.n, L.avg, dbl);
       o.key.fam = F_CSR;
       o.key.mode = mode0;
-      o.key.g = g;
+      o.m.g = g;
       o.m.n = L.n;
       o.m.rowptr = L.A.rowptr.p;
       o.m.col = L.A.col.p;
@@ -677,7 +667,7 @@ struct Planner {
       o.units = (M.n + 31) / 32;
     } else {
       o.key.fam = F_CSR;
-      o.key.g = g;
+      o.m.g = g;
       o.units = (M.n + 32 / g - 1) / (32 / g);
     }
     add(o);

@@ -117,13 +117,13 @@ __device__ __forceinline__ void csr_group_row(int row, bool active, int gl,
   }
 }
 
-// NR <= G rows of a group at a time, as csr_group_row computes each: the rows' bounds, the first
-// two entries of every lane, their x and the update's operands are loaded for all rows before the
-// first is summed, and lane q of the group applies MODE to row q (the butterfly leaves the same
-// sum in every lane).  A warp that takes many short rows of many matrices waits for one chain of
-// loads instead of NR (each row is a lane's entry or two, then the shuffles).
-template <class TV, class TM, int G, int MODE, int NR>
-__device__ __forceinline__ void csr_group_rows(const int row[NR], const bool active[NR], int gl,
+// Up to four rows of a group at a time, as csr_group_row computes each, G (2 .. 32) known at run time:
+// the rows' bounds, two entries of every lane and row, their x and the update's operands are loaded
+// for all rows before the first is summed, and lane q of the group applies MODE to row q (the
+// butterfly leaves the same sum in every lane; with G = 2 the caller passes two rows).  A warp
+// that takes many short rows of many matrices waits for one chain of loads instead of four.
+template <class TV, class TM, int MODE>
+__device__ __forceinline__ void csr_group_rows(const int row[4], const bool active[4], int gl, int G,
                                                const int* __restrict__ rowptr,
                                                const int* __restrict__ col,
                                                const TM* __restrict__ val,
@@ -131,7 +131,7 @@ __device__ __forceinline__ void csr_group_rows(const int row[NR], const bool act
                                                const TV* __restrict__ b, TV* __restrict__ d,
                                                const TV* __restrict__ invd, TV c1, TV c2,
                                                TV* __restrict__ y2) {
-  static_assert(NR <= G, "a lane per row");
+  constexpr int NR = 4, E = 2;
   int p[NR], p1[NR], er = -1;
 #pragma unroll
   for (int q = 0; q < NR; ++q) {
@@ -150,33 +150,38 @@ __device__ __forceinline__ void csr_group_rows(const int row[NR], const bool act
     if (MODE == CSR_ADD) xv = y[er];
     if (MODE == CSR_SPMV_CHEB0) iv = invd[er];
   }
-  int k[NR][2];
-  TV a[NR][2], acc[NR];
+  TV acc[NR];
 #pragma unroll
-  for (int q = 0; q < NR; ++q)
+  for (int q = 0; q < NR; ++q) acc[q] = TV(0);
+  for (bool more = true; more;) {
+    int k[NR][E];
+    TV a[NR][E];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const bool on = p[q] + e * G < p1[q];
-      k[q][e] = on ? col[p[q] + e * G] : -1;
-      a[q][e] = on ? (TV)ldv(val, p[q] + e * G) : TV(0);
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int pe = p[q] + e * G;
+        const bool on = pe < p1[q];
+        k[q][e] = on ? col[pe] : -1;
+        a[q][e] = on ? (TV)ldv(val, pe) : TV(0);
+      }
+    more = false;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      TV xe[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) xe[e] = k[q][e] >= 0 ? x[k[q][e]] : TV(0);
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (k[q][e] >= 0) acc[q] += a[q][e] * xe[e];
+      p[q] += E * G;
+      more |= p[q] < p1[q];
     }
-#pragma unroll
-  for (int q = 0; q < NR; ++q) {
-    TV xe[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) xe[e] = k[q][e] >= 0 ? x[k[q][e]] : TV(0);
-    acc[q] = TV(0);
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-      if (k[q][e] >= 0) acc[q] += a[q][e] * xe[e];
   }
+  __syncwarp();
+  for (int o = G >> 1; o > 0; o >>= 1)
 #pragma unroll
-  for (int q = 0; q < NR; ++q)
-    for (int e = p[q] + 2 * G; e < p1[q]; e += G) acc[q] += (TV)ldv(val, e) * x[col[e]];
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1)
-#pragma unroll
-    for (int q = 0; q < NR; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o, G);
+    for (int q = 0; q < NR; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
   TV s = acc[0];
 #pragma unroll
   for (int q = 1; q < NR; ++q)
