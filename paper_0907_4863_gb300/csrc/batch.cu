@@ -930,7 +930,8 @@ void build_lane(Lane& L, std::vector<std::unique_ptr<SolveWork>>& work,
       units.push_back(o.units);
     }
     std::vector<int4> wb;
-    work_blocks(units, kWarps * kWarpUnits, wb);
+    // a coarse solve's rows are few and long: one per warp and work block
+    work_blocks(units, first.key.fam == F_GEMV ? kWarps : kWarps * kWarpUnits, wb);
     g.nwb = (int)wb.size();
     align(16);
     g.wb_off = host.size();

@@ -224,12 +224,14 @@ __device__ __forceinline__ void csr_short_row(int row, const int* __restrict__ r
     k[q] = on ? col[p0 + q] : 0;
     a[q] = on ? (TV)ldv(val, p0 + q) : TV(0);
   }
-  TV acc = TV(0);
+  // the sum starts from y: the six predicated steps and an addition would be seven FP64
+  // instructions a row, and FP64 issue binds the level-0 prolongation
+  TV acc = y0;
 #pragma unroll
   for (int q = 0; q < kShortWin; ++q)
     if (p0 + q < p1) acc += a[q] * x[k[q]];
   for (int p = p0 + kShortWin; p < p1; ++p) acc += (TV)ldv(val, p) * x[col[p]];
-  y[row] = MODE == CSR_ADD ? y0 + acc : acc;
+  y[row] = acc;
 }
 
 // --- SELL-32, a thread per row of slice s ---------------------------------------------------
@@ -316,6 +318,7 @@ __device__ __forceinline__ void gemv_row(int i, int n, int lane, const double* _
                                          const TV* __restrict__ b, TV* __restrict__ x) {
   const double* row = inv + (size_t)i * n;
   double acc = 0.0;
+#pragma unroll 8  // that many loads in flight, added in order
   for (int c = lane; c < n; c += 32) acc += row[c] * widen(b[c]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
