@@ -72,6 +72,10 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
                                             T c2, T c2invd0, double& dacc,
                                             const int* __restrict__ agg) {
     constexpr bool kPair = MODE == ST_PAIR0 || MODE == ST_PAIR || MODE == ST_PAIR_D;
+    // a table row's part in the pair passes: in FP32 its coefficients are scaled, so that all lanes
+    // of a chunk run the same arithmetic; in FP64, where table rows have warps of their own, A x is
+    // formed and scaled (9 FP64 operations instead of 14)
+    constexpr bool kPairRow = kPair && sizeof(T) == 4;
     int row;
     int ra = 0, rb = 0, tl = 0;  // chunk path: lanes of the regular run, table row of lane 0
     int4 nb;
@@ -113,7 +117,7 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       ayp = tb[4];
       azm = tb[5];
       azp = tb[6];
-      if (kPair) {  // the row of k0 I - k1 A (c2 = k0, c1 = k1)
+      if (kPairRow) {  // the row of k0 I - k1 A (c2 = k0, c1 = k1)
         a0 = fma(-c1, a0, c2);
         axm *= -c1;
         axp *= -c1;
@@ -121,7 +125,7 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
         ayp *= -c1;
         azm *= -c1;
         azp *= -c1;
-      } else {
+      } else if (!kPair) {
         c2i = c2 * tb[7];
       }
       oxm = nonzero(axm) ? oxm : 0;
@@ -185,13 +189,15 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       acc = fma(-azm, vzm, acc);
       acc = fma(-azp, vzp, acc);
     } else {
-      acc = MODE == ST_PAIR ? fma(a0, xc, y[row]) : a0 * xc;
+      const bool own = kPair && !kPairRow && t >= 0;
+      acc = MODE == ST_PAIR && !own ? fma(a0, xc, y[row]) : a0 * xc;
       acc = fma(axm, vxm, acc);
       acc = fma(axp, vxp, acc);
       acc = fma(aym, vym, acc);
       acc = fma(ayp, vyp, acc);
       acc = fma(azm, vzm, acc);
       acc = fma(azp, vzp, acc);
+      if (own) acc = fma(-c1, acc, MODE == ST_PAIR ? fma(c2, xc, y[row]) : c2 * xc);
     }
     if (MODE == ST_DINV_DOT) {  // c2 carries the scale of x: w = c2 D^-1 A x
       const T w = c2i * acc;
