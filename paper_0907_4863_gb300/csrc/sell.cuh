@@ -20,8 +20,10 @@ namespace saamg {
 
 constexpr int kSellWindow = 512;
 // smallest level stored as SELL: below it one thread per row leaves most of the GPU idle and
-// the CSR kernel with wide row groups is faster
-constexpr int kSellMinRows = 100000;
+// the CSR kernel with wide row groups is faster.  Whole FP64 solves, CSR / SELL on level 1: 34 k rows
+// (96^3 pipe) 2.41 / 2.58 ms, 81 k rows (128^3) 4.75 / 4.43 (FP32 V-cycle 3.04 / 2.96): a row group's
+// shuffle additions cost as much FP64 time as a thread's whole row saves it.
+constexpr int kSellMinRows = 60000;
 
 struct DevSell {
   int n = 0, m = 0, nslices = 0;

@@ -453,11 +453,14 @@ void launch_shaped(const StencilCfg& cfg, long long units, int blocks_cap, const
   // warp per quarter at a time)
   int block = cfg.block;
   while (block > 64 && units * 32 < (long long)sm_count() * block) block >>= 1;
+  // several chunks per step only where a resident warp (64 per SM) has eight or more: fewer, longer
+  // steps leave SMs idle below that (32^3 solve 986 us with one chunk per step, 1063 with two)
+  const int k = units < 8LL * 64 * sm_count() ? 1 : cfg.k;
   const int wpb = block / 32;
-  const long long need = (units + (long long)wpb * cfg.k - 1) / ((long long)wpb * cfg.k);
+  const long long need = (units + (long long)wpb * k - 1) / ((long long)wpb * k);
   const int blocks = (int)std::max<long long>(1, std::min<long long>(need, blocks_cap));
 #define SAAMG_SHAPE(KK, PP)                                                                  \
-  if (cfg.k == KK && (cfg.packed != 0) == PP) {                                              \
+  if (k == KK && (cfg.packed != 0) == PP) {                                                  \
     launch_pdl(stencil_k<T, MODE, KK, PP>, blocks, block, 0, s, S, x, y, b, d, c1, c2,       \
                c2i0, partials, xscale, agg, (PcgCtl*)nullptr);                               \
     return;                                                                                  \
