@@ -698,7 +698,7 @@ struct Planner {
     const SmoothPair<T> sp = pr ? SmoothPair<T>(L.cheb.c2[0], L.cheb.c1[1], L.cheb.c2[1])
                                 : SmoothPair<T>(0.0, 0.0, 0.0);
     int cur = pr ? 1 : 0;
-    if (pr) pair<T>(P_PRE, 0, ST_PAIR0, b, bufs[cur], nu > 2 ? d : nullptr, sp);
+    if (pr) pair<T>(P_PRE, 0, nu > 2 ? ST_PAIR0_D : ST_PAIR0, b, bufs[cur], d, sp);
     else if (l == 0 || !restriction_smooths(h, l - 1, sizeof(T) == 8))
       smooth<T>(P_PRE, l, 0, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0]);
     for (int k = pr ? 2 : 1; k < nu; ++k) {

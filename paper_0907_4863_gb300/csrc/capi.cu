@@ -850,8 +850,8 @@ static void vcycle_level(saamg_hierarchy* h, int l, const T* b, T* out, cudaStre
   int cur = pair ? 1 : 0;
   // presmoothing from x = 0
   if (pair)
-    stencil_apply<T>(h->op->d.template view<T>(), ST_PAIR0, b, bufs[cur], nullptr,
-                     nu > 2 ? d : nullptr, sp.k1, sp.k0, nullptr, s, nullptr, sp.g);
+    stencil_apply<T>(h->op->d.template view<T>(), nu > 2 ? ST_PAIR0_D : ST_PAIR0, b, bufs[cur],
+                     nullptr, d, sp.k1, sp.k0, nullptr, s, nullptr, sp.g);
   else if (!first_done)
     smooth_step<T>(h, l, CSR_CHEB0, nullptr, bufs[cur], b, d, T(0), (T)L.cheb.c2[0], s);
   for (int k = pair ? 2 : 1; k < nu; ++k) {

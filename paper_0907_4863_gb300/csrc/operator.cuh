@@ -104,9 +104,10 @@ enum StencilMode {
   ST_CHEB1 = 6,     // ST_CHEB with c1 = 0 (first step from a nonzero x): d is not read
   ST_PROLONG = 7,   // y += P v with P = (I - omega D^-1 A) T, T from the aggregates
   // the first two Chebyshev steps as one pass (see SmoothPair): x is b or the residual
-  ST_PAIR0 = 8,     // y = k0 x - k1 A x; d = y - g x (if d is not null)
+  ST_PAIR0 = 8,     // y = k0 x - k1 A x
   ST_PAIR = 9,      // y += k0 x - k1 A x
-  ST_PAIR_D = 10    // e = k0 x - k1 A x; y += e; d = e - g x
+  ST_PAIR_D = 10,   // e = k0 x - k1 A x; y += e; d = e - g x
+  ST_PAIR0_D = 11   // y = k0 x - k1 A x; d = y - g x
 };
 
 // Two Chebyshev steps on level 0 from x with residual r = b - A x (x = 0: r = b).  The scaled

@@ -71,7 +71,8 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
                                             const T* __restrict__ b, T* __restrict__ d, T c1,
                                             T c2, T c2invd0, double& dacc,
                                             const int* __restrict__ agg) {
-    constexpr bool kPair = MODE == ST_PAIR0 || MODE == ST_PAIR || MODE == ST_PAIR_D;
+    constexpr bool kPair =
+        MODE == ST_PAIR0 || MODE == ST_PAIR0_D || MODE == ST_PAIR || MODE == ST_PAIR_D;
     // a table row's part in the pair passes: in FP32 its coefficients are scaled, so that all lanes
     // of a chunk run the same arithmetic; in FP64, where table rows have warps of their own, A x is
     // formed and scaled (9 FP64 operations instead of 14)
@@ -208,11 +209,13 @@ __device__ __forceinline__ void stencil_row(const StencilDev<T>& S, int c, int l
       if (MODE == ST_SPMV_DOT) dacc = fma(to_d(xc), to_d(acc), dacc);
     } else if (MODE == ST_RESID) {
       y[row] = acc;
-    } else if (MODE == ST_PAIR) {
+    } else if (MODE == ST_PAIR || MODE == ST_PAIR0) {
       y[row] = acc;
-    } else if (MODE == ST_PAIR0) {  // the c2invd0 argument holds g
+    } else if (MODE == ST_PAIR0_D) {  // the c2invd0 argument holds g
+      // a mode of its own: under a test of d, the multiply-add holds the FP64 pipe also where it
+      // is predicated off (one V-cycle at 193 x 131 x 160: 282 -> 279 us)
       y[row] = acc;
-      if (d) d[row] = fma(-c2invd0, xc, acc);
+      d[row] = fma(-c2invd0, xc, acc);
     } else if (MODE == ST_PAIR_D) {
       y[row] = y[row] + acc;
       d[row] = fma(-c2invd0, xc, acc);
@@ -414,6 +417,9 @@ void batched_stencil(int mode, const StTask<T>* tasks, const int4* wbs, int nwb,
     case ST_PAIR0:
       SAAMG_BST(ST_PAIR0);
       break;
+    case ST_PAIR0_D:
+      SAAMG_BST(ST_PAIR0_D);
+      break;
     case ST_PAIR:
       SAAMG_BST(ST_PAIR);
       break;
@@ -485,7 +491,7 @@ template <class T>
 void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T* b, T* d, T c1,
                    T c2, double* partials, cudaStream_t s, const double* xscale, T g,
                    PcgCtl* ctl) {
-  const bool pair = mode == ST_PAIR0 || mode == ST_PAIR || mode == ST_PAIR_D;
+  const bool pair = mode == ST_PAIR0 || mode == ST_PAIR0_D || mode == ST_PAIR || mode == ST_PAIR_D;
   const StencilDev<T> S = pair ? pair_stencil(S0, c2, c1) : S0;
   if (S.nchunks == 0) {
     if (mode == ST_SPMV_DOT || mode == ST_DINV_DOT) fill_double(partials, 0.0, kRedBlocks, s);
@@ -549,6 +555,10 @@ void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T*
     case ST_PAIR0:
       launch_shaped<T, ST_PAIR0>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
+      break;
+    case ST_PAIR0_D:
+      launch_shaped<T, ST_PAIR0_D>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+                                   nullptr, s);
       break;
     case ST_PAIR:
       launch_shaped<T, ST_PAIR>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
