@@ -39,6 +39,11 @@ __global__ void densify_k(int n, const int* __restrict__ rowptr, const int* __re
 // update start once its blocks are resident (programmatic dependent launch); their shared-memory
 // requests keep the two off the same SM, where the update's warps would queue before every FP64
 // instruction of the panel's serial chain (n = 1250: 70 instead of 52 us a panel).
+// What the update reads was written by the launches before the panel beside it, and a programmatic
+// dependent has no order with those but through griddepcontrol.wait, which would have it wait for
+// the panel as well.  The panel has waited for them: it says so by a release store before it lets
+// the update start, and the update's blocks read that with an acquire load (or wait, if they do not
+// see it).
 constexpr int kGjB = 16;           // steps of a panel
 constexpr int kGjCluster = 16;     // blocks of the panel kernel (an opt-in size)
 constexpr int kGjThreads = 256;    // panel kernel: two of the panel's columns per warp
@@ -101,11 +106,16 @@ __global__ void __launch_bounds__(kGjThreads)
     gj_panel_k(int n, int k0, int rpb, const double* __restrict__ a, int pend,
                const GjPanel* __restrict__ ppn, const double* __restrict__ pc,
                GjPanel* __restrict__ opn, double* __restrict__ oc, const int* __restrict__ pstep,
-               int* __restrict__ step, int* __restrict__ prow, int* __restrict__ err) {
+               int* __restrict__ step, int* __restrict__ prow, int* __restrict__ err, int seq,
+               int* ready) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  asm volatile("griddepcontrol.wait;" ::: "memory");               // the update before
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the update beside this panel
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the update before
+  if (threadIdx.x == 0) {                             // the update beside this panel
+    if (blockIdx.x == 0)
+      asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(ready), "r"(seq) : "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   constexpr int B = kGjB;
   struct Cand {
     double v[B];
@@ -260,12 +270,13 @@ __global__ void __launch_bounds__(kGjThreads)
 }
 
 // dst = src after the steps of the panel at k0: a tile of cpb columns and rpt rows per block.
+// seq > 0: launched beside the panel that stores seq to *ready (the inputs are not __restrict__:
+// they must not be read through the non-coherent path or ahead of that).
 __global__ void __launch_bounds__(kGjUpdThreads) gj_update_k(int n, int k0, int cpb, int rpt,
-                                                             const GjPanel* __restrict__ gpn,
-                                                             const double* __restrict__ cc,
-                                                             const int* __restrict__ step,
-                                                             const double* __restrict__ src,
-                                                             double* __restrict__ dst) {
+                                                             const GjPanel* gpn, const double* cc,
+                                                             const int* step, const double* src,
+                                                             double* __restrict__ dst, int seq,
+                                                             const int* ready) {
   constexpr int B = kGjB;
   __shared__ GjPanel pn;
   __shared__ double rr[kGjUpdCols][B];
@@ -273,6 +284,14 @@ __global__ void __launch_bounds__(kGjUpdThreads) gj_update_k(int n, int k0, int 
   const int bw = min(B, n - k0);
   const int c0 = blockIdx.x * cpb, nc = min(cpb, n - c0);
   const int r0 = blockIdx.y * rpt, r1 = min(n, r0 + rpt);
+  if (seq > 0) {
+    if (tid == 0) {
+      int seen;
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(ready) : "memory");
+      if (seen != seq) asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    __syncthreads();
+  }
   {
     const double* g = reinterpret_cast<const double*>(gpn);
     double* d = reinterpret_cast<double*>(&pn);
@@ -531,14 +550,14 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
   Buf<double> w2, c[2];
   Buf<GjPanel> pn[2];
   prow.alloc(n, s);
-  err.alloc(1, s);
+  err.alloc(2, s);  // zero pivot, last panel that has begun
   w2.alloc((size_t)n * n, s);
   for (int q = 0; q < 2; ++q) {
     step[q].alloc(n, s);
     c[q].alloc((size_t)B * n, s);
     pn[q].alloc(1, s);
   }
-  fill_int(err.p, 0, 1, s);
+  fill_int(err.p, 0, 2, s);
   fill_int(step[1].p, -1, n, s);  // read by panel 0: no row is pivoted
   const int rpb = (n + kGjCluster - 1) / kGjCluster;
   SAAMG_CUDA(cudaFuncSetAttribute(gj_panel_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -564,7 +583,9 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
   const dim3 ugrid((n + cpb - 1) / cpb, rt);
   // panel q reads the matrix before update q - 1 and the panel q - 1; update q the same matrix as
   // panel q + 1, and the panel q.  Panel q waits at its entry for the launch before it, update
-  // q - 2, which ends after panel q - 1 beside it: everything before has finished.
+  // q - 2, which ends after panel q - 1 beside it: everything before has finished.  Update q starts
+  // once panel q + 1 has passed that wait, so update q - 1 and panel q have finished, and takes their
+  // writes from panel q + 1 through err[1].
   const int panels = (n + B - 1) / B;
   auto panel = [&](int q) {
     const int pq = (q & 1) ^ 1;
@@ -584,7 +605,7 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
     SAAMG_CUDA(cudaLaunchKernelEx(&cfg, gj_panel_k, n, q * B, rpb, (const double*)w.p,
                                   q > 0 ? B : 0, (const GjPanel*)pn[pq].p, (const double*)c[pq].p,
                                   pn[q & 1].p, c[q & 1].p, (const int*)step[pq].p, step[q & 1].p,
-                                  prow.p, err.p));
+                                  prow.p, err.p, q, err.p + 1));
     SAAMG_LAUNCH();
   };
   panel(0);
@@ -593,7 +614,8 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
     if (beside) panel(q + 1);
     auto args = [&](auto&& launch) {
       launch(n, q * B, cpb, rpt, (const GjPanel*)pn[q & 1].p, (const double*)c[q & 1].p,
-             (const int*)step[q & 1].p, (const double*)w.p, w2.p);
+             (const int*)step[q & 1].p, (const double*)w.p, w2.p, beside ? q + 1 : 0,
+             (const int*)(err.p + 1));
     };
     args([&](auto... a) {
       if (beside) launch_pdl(gj_update_k, ugrid, kGjUpdThreads, kGjUpdSmem, s, a...);

@@ -1,5 +1,10 @@
 """The blocked elimination of the dense inverse at the edges of its panels (16 steps), of the rows
 that a block of the panel's cluster holds, and of the update's tiles."""
+import hashlib
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -43,3 +48,33 @@ def test_inverse_at_panel_edges(S, n, kind):
     for c in range(2):
         x = O.dense_lu_solve(m, b[:, c])
         assert np.linalg.norm(inv @ b[:, c] - x) <= 1e-12 * np.linalg.norm(x)
+
+
+SIZES = [17, 48, 545, 1250, 2050]
+
+
+def _digests(S):
+    import torch
+    out = []
+    for n in SIZES:
+        rng = np.random.default_rng(n)
+        m = rng.uniform(-1.0, 1.0, (n, n)) / n
+        m[np.arange(n), np.arange(n)] = 2.0 + rng.uniform(0.0, 1.0, n)
+        a = torch.from_numpy(m[rng.permutation(n)]).cuda()
+        inv = torch.empty_like(a)
+        for _ in range(3):  # the buffers of one call are the next call's
+            S.dense_inverse(a, inv)
+            out.append(hashlib.sha256(inv.cpu().numpy().tobytes()).hexdigest())
+    return out
+
+
+def test_panels_beside_updates_give_the_bits_of_launches_in_turn(S):
+    """The update of a panel runs beside the factorisation of the next one; without dependent
+    launches every kernel starts after the one before it has ended."""
+    code = ("from tests.test_gpu_dense_inverse_panels import _digests\n"
+            "from paper_0907_4863_gb300 import saamg\nprint(' '.join(_digests(saamg)))")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True,
+                       timeout=300, env=dict(os.environ, SAAMG_PDL="0"))
+    assert p.returncode == 0, p.stderr
+    assert p.stdout.split() == _digests(S)
