@@ -974,6 +974,13 @@ static int pcg_impl(saamg_hierarchy* h, double rtol, cudaStream_t s, saamg_solve
   SAAMG_LAUNCH();
   pcg_prologue(h, nullptr, s);
   d2h_sync(hc, ctl, sizeof(PcgCtl), s);
+  // thrown before the caller scatters: phi keeps its values
+  if (!std::isfinite(hc->bb)) fail(SAAMG_NUMERICAL, "right-hand side holds NaN or Inf");
+  if (hc->bb == 0.0) {  // x is zeroed, whatever the initial guess was
+    info->converged = 1;
+    return SAAMG_OK;
+  }
+  if (!std::isfinite(hc->rr)) fail(SAAMG_NUMERICAL, "initial residual holds NaN or Inf");
   while (!hc->converged && !hc->breakdown && hc->iters < h->prm.maxit) {
     pcg_pass(h, nullptr, s);
     d2h_sync(hc, ctl, sizeof(PcgCtl), s);

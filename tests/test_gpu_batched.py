@@ -83,6 +83,45 @@ def test_device_loop_edge_cases(S):
     assert S.solve_wait(h)["iters"] == 0
 
 
+@pytest.mark.parametrize("where", ["device", "host"])
+def test_host_loop_edge_cases(S, where):
+    """The host-driven loop names what is not finite and leaves phi alone then; a zero right-hand
+    side has the solution 0 whatever the initial guess holds."""
+    import torch
+    w = I.pipe_workload(24, I.LINEAR)
+    h = _setup(S, w, max_coarse=100, device_loop=0)
+    m = w.grid.n[0] // 2
+    inside = m + w.grid.n[0] * (m + w.grid.n[1] * m)
+
+    def solve(rho, phi):
+        if where == "device":
+            d = torch.from_numpy(phi).cuda()
+            try:
+                return S.solve(h, torch.from_numpy(rho).cuda(), d)
+            finally:
+                phi[:] = d.cpu().numpy()
+        return S.solve_host(h, rho, phi)
+
+    rho = I.gaussian_bunch(w.grid, w.centre, w.sigma, 0)
+    for bad in (np.nan, np.inf):
+        b = rho.copy()
+        b[inside] = bad
+        phi = np.full(w.grid.nbox, 2.0)
+        with pytest.raises(S.SaamgError, match="right-hand side holds NaN or Inf") as e:
+            solve(b, phi)
+        assert e.value.status == S.NUMERICAL and np.all(phi == 2.0)
+        phi[inside] = bad
+        kept = phi.copy()
+        with pytest.raises(S.SaamgError, match="initial residual holds NaN or Inf") as e:
+            solve(rho, phi)
+        assert e.value.status == S.NUMERICAL and np.array_equal(phi, kept, equal_nan=True)
+        info = solve(np.zeros_like(rho), phi)
+        assert info["status"] == 0 and info["converged"] == 1 and info["iters"] == 0
+        assert info["relres"] == 0.0 and info["relres_true"] == 0.0 and np.all(phi == 0.0)
+    phi = np.zeros_like(rho)  # nothing of the failed solves stays in the handle
+    assert solve(rho, phi)["converged"] == 1 and np.all(np.isfinite(phi))
+
+
 def test_batched_results_equal_solo_results(S):
     """Uneven instances (sizes, geometries, modes, precisions) and several rhs per instance:
     every result in the batch equals the same solve run alone, bit for bit."""
