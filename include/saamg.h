@@ -314,12 +314,16 @@ typedef struct saamg_stencil_config {
 /* The shape op uses for precision 0 (FP64 passes) or 1 (FP32 passes, also the BF16 mode's). */
 saamg_status saamg_stencil_config_get(const saamg_operator *op, int precision,
                                       saamg_stencil_config *cfg);
-/* Sets it (cfg NULL: the default); EINVAL for a shape outside the sets above.  Hierarchies
- * set up later, and solve graphs captured later, use it; graphs captured before keep theirs. */
+/* Sets it (cfg NULL, or the shape that get returns on a new operator: the default); EINVAL for a
+ * shape outside the sets above.  Hierarchies set up later, and solve graphs captured later, use it;
+ * graphs captured before keep theirs.  The default is fitted to the operator: one chunk per step on
+ * a small one, as get returns it, and blocks of down to 64 threads where 256 would leave SMs without
+ * one.  Any other shape runs as it is set. */
 saamg_status saamg_stencil_config_set(saamg_operator *op, int precision,
                                       const saamg_stencil_config *cfg);
 /* Autotuner of the launch shape: times the level-0 smoothing pass of precision 0 or 1 under
- * all 36 shapes on scratch vectors of op's size (allocated and freed here), sets the fastest
+ * all 36 shapes and the default on scratch vectors of op's size (allocated and freed here), sets the
+ * fastest
  * on op and returns it with its time in microseconds (median of three launches). */
 saamg_status saamg_autotune_stencil(saamg_operator *op, int precision, void *stream,
                                     saamg_stencil_config *best, double *best_us);

@@ -1804,7 +1804,7 @@ saamg_status saamg_stencil_config_get(const saamg_operator* op, int precision,
   return guard("saamg_stencil_config_get", [&] {
     if (!op || op->magic != kOpMagic || !cfg) fail(SAAMG_EINVAL, "NULL or invalid argument");
     if (precision != 0 && precision != 1) fail(SAAMG_EINVAL, "precision must be 0 or 1");
-    const StencilCfg& c = op->d.cfg[precision];
+    const StencilCfg c = op->d.launched(op->d.cfg[precision]);
     *cfg = saamg_stencil_config{c.k, c.packed, c.block, c.per_sm};
   });
 }
@@ -1814,13 +1814,15 @@ saamg_status saamg_stencil_config_set(saamg_operator* op, int precision,
   return guard("saamg_stencil_config_set", [&] {
     if (!op || op->magic != kOpMagic) fail(SAAMG_EINVAL, "NULL or invalid argument");
     if (precision != 0 && precision != 1) fail(SAAMG_EINVAL, "precision must be 0 or 1");
+    const StencilCfg def = OperatorData::kDefaultCfg[precision];
     if (!cfg) {
-      op->d.cfg[precision] = OperatorData{}.cfg[precision];
+      op->d.cfg[precision] = def;
       return;
     }
     check_stencil_cfg(*cfg);
-    op->d.cfg[precision] = StencilCfg{cfg->chunks_per_step, cfg->packed, cfg->block,
-                                      cfg->blocks_per_sm};
+    const StencilCfg c{cfg->chunks_per_step, cfg->packed, cfg->block, cfg->blocks_per_sm};
+    // the default as saamg_stencil_config_get returns it is the default again
+    op->d.cfg[precision] = c.same_shape(op->d.launched(def)) ? def : c;
   });
 }
 
@@ -1831,9 +1833,10 @@ saamg_status saamg_autotune_stencil(saamg_operator* op, int precision, void* str
     if (precision != 0 && precision != 1) fail(SAAMG_EINVAL, "precision must be 0 or 1");
     cudaStream_t s = (cudaStream_t)stream;
     double us = 0;
-    const StencilCfg c = precision == 0 ? stencil_autotune<double>(op->d.view<double>(), s, &us)
-                                        : stencil_autotune<float>(op->d.view<float>(), s, &us);
+    StencilCfg c = precision == 0 ? stencil_autotune<double>(op->d.view<double>(), s, &us)
+                                  : stencil_autotune<float>(op->d.view<float>(), s, &us);
     op->d.cfg[precision] = c;
+    c = op->d.launched(c);
     if (best) *best = saamg_stencil_config{c.k, c.packed, c.block, c.per_sm};
     if (best_us) *best_us = us;
   });

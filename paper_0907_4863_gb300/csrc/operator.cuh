@@ -45,7 +45,16 @@ struct OperatorData {
   // packed rows; FP32 is latency-bound and takes line chunks on as many blocks as are resident.
   // Solves at 256^3 against one chunk per step and 16 blocks per SM (FP64), 16 blocks per SM (FP32):
   // 24.82 -> 24.41 and 14.93 -> 14.71 ms
-  StencilCfg cfg[2] = {{2, 1, 256, 32}, {2, 0, 256, 8}};
+  static constexpr StencilCfg kDefaultCfg[2] = {{2, 1, 256, 32, true}, {2, 0, 256, 8, true}};
+  StencilCfg cfg[2] = {kDefaultCfg[0], kDefaultCfg[1]};
+  // shape c as the passes of this operator launch it (all of one precision have as many chunks); the
+  // default's blocks may still be smaller
+  StencilCfg launched(StencilCfg c) const {
+    const long long units =
+        c.packed ? ((long long)nrun + 31) / 32 + (ntable + 31) / 32 : (long long)nchunks;
+    c.k = stencil_chunks(c, units, sm_count());
+    return c;
+  }
   size_t bytes() const {
     return lines.bytes() + nbr.bytes() + chunks.bytes() + crec.bytes() + rline.bytes() + table.bytes() +
            table32.bytes() + trow.bytes() + rrow.bytes() + scale.bytes() +
@@ -147,7 +156,7 @@ template <class T>
 void stencil_prolong(const StencilDev<T>& S, const int* agg, T omega, const T* v, T* y,
                      cudaStream_t s);
 // Times the level-0 smoothing pass under every launch shape (K 1/2/4, packed or line chunks,
-// 128/256 threads, 8/16/32 blocks per SM) on scratch vectors and returns the fastest; its
+// 128/256 threads, 8/16/32 blocks per SM; the default) on scratch vectors and returns the fastest; its
 // time (median of three launches) in *best_us.
 template <class T>
 StencilCfg stencil_autotune(const StencilDev<T>& S, cudaStream_t s, double* best_us);

@@ -452,22 +452,13 @@ void batched_stencil_dot(const StTask<double>* tasks, const int2* pairs, int npa
 
 // Launches MODE with the shape of cfg (K and packed from the instantiated set).
 template <class T, int MODE>
-void launch_shaped(const StencilCfg& cfg, long long units, int blocks_cap, const StencilDev<T>& S,
-                   const T* x, T* y, const T* b, T* d, T c1, T c2, T c2i0, double* partials,
-                   const double* xscale, const int* agg, cudaStream_t s) {
-  // a small level spreads over the SMs in smaller blocks (an SM takes FP64 instructions of one
-  // warp per quarter at a time)
-  int block = cfg.block;
-  while (block > 64 && units * 32 < (long long)sm_count() * block) block >>= 1;
-  // several chunks per step only where a resident warp (64 per SM) has eight or more: fewer, longer
-  // steps leave SMs idle below that (32^3 solve 986 us with one chunk per step, 1063 with two)
-  const int k = units < 8LL * 64 * sm_count() ? 1 : cfg.k;
-  const int wpb = block / 32;
-  const long long need = (units + (long long)wpb * k - 1) / ((long long)wpb * k);
-  const int blocks = (int)std::max<long long>(1, std::min<long long>(need, blocks_cap));
+void launch_shaped(const StencilCfg& cfg, long long units, const StencilDev<T>& S, const T* x, T* y,
+                   const T* b, T* d, T c1, T c2, T c2i0, double* partials, const double* xscale,
+                   const int* agg, cudaStream_t s) {
+  const StencilLaunch l = stencil_launch(cfg, units, sm_count());
 #define SAAMG_SHAPE(KK, PP)                                                                  \
-  if (k == KK && (cfg.packed != 0) == PP) {                                                  \
-    launch_pdl(stencil_k<T, MODE, KK, PP>, blocks, block, 0, s, S, x, y, b, d, c1, c2,       \
+  if (l.k == KK && (cfg.packed != 0) == PP) {                                                \
+    launch_pdl(stencil_k<T, MODE, KK, PP>, l.blocks, l.block, 0, s, S, x, y, b, d, c1, c2,   \
                c2i0, partials, xscale, agg, (PcgCtl*)nullptr);                               \
     return;                                                                                  \
   }
@@ -530,42 +521,41 @@ void stencil_apply(const StencilDev<T>& S0, int mode, const T* x, T* y, const T*
   }
   const StencilCfg& cfg = S.cfg;
   const long long units = shaped_units(S, cfg.packed != 0);
-  const int cap = sm_count() * cfg.per_sm;
   switch (mode) {
     case ST_SPMV:
-      launch_shaped<T, ST_SPMV>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_SPMV>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                 nullptr, s);
       break;
     case ST_RESID:
-      launch_shaped<T, ST_RESID>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_RESID>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
       break;
     case ST_CHEB:
-      launch_shaped<T, ST_CHEB>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_CHEB>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                 nullptr, s);
       break;
     case ST_CHEB0:
-      launch_shaped<T, ST_CHEB0>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_CHEB0>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
       break;
     case ST_CHEB1:
-      launch_shaped<T, ST_CHEB1>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_CHEB1>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
       break;
     case ST_PAIR0:
-      launch_shaped<T, ST_PAIR0>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_PAIR0>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                  nullptr, s);
       break;
     case ST_PAIR0_D:
-      launch_shaped<T, ST_PAIR0_D>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_PAIR0_D>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                    nullptr, s);
       break;
     case ST_PAIR:
-      launch_shaped<T, ST_PAIR>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_PAIR>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                 nullptr, s);
       break;
     case ST_PAIR_D:
-      launch_shaped<T, ST_PAIR_D>(cfg, units, cap, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
+      launch_shaped<T, ST_PAIR_D>(cfg, units, S, x, y, b, d, c1, c2, c2i0, partials, xscale,
                                   nullptr, s);
       break;
     default:
@@ -580,14 +570,13 @@ void stencil_prolong(const StencilDev<T>& S, const int* agg, T omega, const T* v
   if (S.nchunks == 0) return;
   KernelTimer kt(SAAMG_KT_PROLONG0, S.n, s);
   const StencilCfg& cfg = S.cfg;
-  launch_shaped<T, ST_PROLONG>(cfg, shaped_units(S, cfg.packed != 0), sm_count() * cfg.per_sm, S,
-                               v, y, nullptr, nullptr, T(0), omega, T(omega * S.invd0), nullptr,
-                               nullptr, agg, s);
+  launch_shaped<T, ST_PROLONG>(cfg, shaped_units(S, cfg.packed != 0), S, v, y, nullptr, nullptr,
+                               T(0), omega, T(omega * S.invd0), nullptr, nullptr, agg, s);
   SAAMG_LAUNCH();
 }
 
-// Times the smoothing pass of every launch shape on scratch vectors and returns the fastest
-// (median of three launches after one untimed).
+// Times the smoothing pass of every launch shape, and of the default as it is fitted to the operator,
+// on scratch vectors and returns the fastest (median of three launches after one untimed).
 template <class T>
 StencilCfg stencil_autotune(const StencilDev<T>& S0, cudaStream_t s, double* best_us) {
   StencilDev<T> S = S0;
@@ -602,29 +591,32 @@ StencilCfg stencil_autotune(const StencilDev<T>& S0, cudaStream_t s, double* bes
   SAAMG_CUDA(cudaMemsetAsync(d.p, 0, n * sizeof(T), s));
   cudaEvent_t e[4];
   for (auto& ev : e) SAAMG_CUDA(cudaEventCreate(&ev));
-  StencilCfg best = S0.cfg;
+  const StencilCfg fitted = OperatorData::kDefaultCfg[sizeof(T) == 4 ? 1 : 0];
+  StencilCfg best = fitted;
   float best_ms = -1.f;
+  auto time = [&](const StencilCfg& c) {
+    S.cfg = c;
+    stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
+    float t[3];
+    for (int r = 0; r < 3; ++r) {
+      SAAMG_CUDA(cudaEventRecord(e[0], s));
+      stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
+      SAAMG_CUDA(cudaEventRecord(e[1], s));
+      SAAMG_CUDA(cudaEventSynchronize(e[1]));
+      SAAMG_CUDA(cudaEventElapsedTime(&t[r], e[0], e[1]));
+    }
+    std::sort(t, t + 3);
+    if (best_ms < 0.f || t[1] < best_ms) {
+      best_ms = t[1];
+      best = c;
+    }
+  };
   try {
+    time(fitted);
     for (int k : {1, 2, 4})
       for (int packed : {0, 1})
         for (int block : {128, 256})
-          for (int per_sm : {8, 16, 32}) {
-            S.cfg = StencilCfg{k, packed, block, per_sm};
-            stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
-            float t[3];
-            for (int r = 0; r < 3; ++r) {
-              SAAMG_CUDA(cudaEventRecord(e[0], s));
-              stencil_apply<T>(S, ST_PAIR, x.p, y.p, b.p, d.p, T(0.5), T(0.25), nullptr, s);
-              SAAMG_CUDA(cudaEventRecord(e[1], s));
-              SAAMG_CUDA(cudaEventSynchronize(e[1]));
-              SAAMG_CUDA(cudaEventElapsedTime(&t[r], e[0], e[1]));
-            }
-            std::sort(t, t + 3);
-            if (best_ms < 0.f || t[1] < best_ms) {
-              best_ms = t[1];
-              best = S.cfg;
-            }
-          }
+          for (int per_sm : {8, 16, 32}) time(StencilCfg{k, packed, block, per_sm});
   } catch (...) {
     for (auto& ev : e) cudaEventDestroy(ev);
     throw;

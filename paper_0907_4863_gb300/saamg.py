@@ -519,7 +519,7 @@ def set_stencil_config(op: Operator, precision: int, cfg=None):
 
 @_entry
 def autotune_stencil(op: Operator, precision: int, stream=None):
-    """Times the 36 launch shapes of the level-0 smoothing pass, sets the fastest on op and
+    """Times the launch shapes of the level-0 smoothing pass, sets the fastest on op and
     returns (shape, microseconds)."""
     c = StencilConfig()
     us = C.c_double(0)

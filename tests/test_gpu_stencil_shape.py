@@ -94,3 +94,22 @@ def test_grid_too_long_in_x_is_rejected(S):
     with pytest.raises(S.SaamgError) as e:
         S.build_operator(S.make_domain(w.domain), S.make_grid(g), w.mode)
     assert e.value.status == S.EINVAL
+
+
+def test_the_default_is_restored_by_its_own_shape(S):
+    """What stencil_config returns on a new operator, set again, is the default; it reports the one
+    chunk per step that a small operator launches."""
+    w = I.cylinder_workload(24, I.LINEAR)
+    op = S.build_operator(S.make_domain(w.domain), S.make_grid(w.grid), w.mode)
+    for prec in (0, 1):
+        default = S.stencil_config(op, prec)
+        assert default["chunks_per_step"] == 1
+        shape = dict(chunks_per_step=4, packed=1, block=128, blocks_per_sm=8)
+        S.set_stencil_config(op, prec, shape)
+        assert S.stencil_config(op, prec) == shape
+        S.set_stencil_config(op, prec, default)
+        assert S.stencil_config(op, prec) == default
+        S.set_stencil_config(op, prec, shape)
+        S.set_stencil_config(op, prec, None)
+        assert S.stencil_config(op, prec) == default
+    op.free()
