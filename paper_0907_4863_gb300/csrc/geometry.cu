@@ -882,6 +882,7 @@ __device__ __forceinline__ bool line_has(const LineInfo& l, int i) { return i >=
 //   plus side outside:  (-(s s) pm + (s s - 1) p0) / ((h s) (1 + s))
 //   minus side outside: ((t t) pp - (t t - 1) p0) / ((h t) (1 + t)), the first with -1 before it
 //   both:               p0 (s - t) / ((h s) t)
+// A side's sign goes to the two products, so that a zero has the reference's sign too.
 // pn: the value on the side that is inside.
 __device__ __forceinline__ double wall_derivative(const GeomParams& g, const GradDiv& dv, int ax,
                                                   bool in_m, bool in_p, int i, int j, int k,
@@ -904,8 +905,8 @@ __device__ __forceinline__ double wall_derivative(const GeomParams& g, const Gra
     f = boundary_fraction(g, i, j, k, in_m ? 5 : 4);
   }
   const double ff = f * f;
-  const double num = -ff * pn + (ff - 1.0) * p0;
-  return (in_m ? num : -num) / (g.h[ax] * f * (1.0 + f));
+  const double b = (ff - 1.0) * p0;
+  return ((in_m ? -ff : ff) * pn + (in_m ? b : -b)) / (g.h[ax] * f * (1.0 + f));
 }
 
 constexpr int kGradLines = 16;  // lattice lines per block, two per warp

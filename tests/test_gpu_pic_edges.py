@@ -59,6 +59,23 @@ def test_gradient_bitwise(S, w, values):
         assert np.array_equal(a.cpu().numpy(), b, equal_nan=True)
 
 
+@pytest.mark.parametrize("w", WORKLOADS, ids=lambda w: w.name)
+def test_gradient_signs_of_zeros(S, w):
+    """Potentials of zeros of either sign and few other values: differences that vanish, beside the
+    wall too, keep the reference's sign."""
+    import torch
+    o = oracle_operator(w)
+    rng = np.random.default_rng(12)
+    op = S.build_operator(S.make_domain(w.domain), S.make_grid(w.grid), w.mode)
+    for values in ([0.0], [-0.0], [0.0, -0.0, 1.0, -1.0]):
+        phi = rng.choice(values, w.grid.nbox)
+        ref = O.field_gradient(o, phi)
+        e = [torch.empty(w.grid.nbox, dtype=torch.float64, device="cuda") for _ in range(3)]
+        S.field_gradient(op, dev(phi), *e)
+        for a, b in zip(e, ref):
+            assert np.array_equal(a.cpu().numpy().view(np.int64), b.view(np.int64))
+
+
 def edge_particles(g, rng):
     """Positions on nodes, on cell edges' neighbours, on and beyond the faces, far outside."""
     lo, h, n = np.array(g.origin), np.array(g.h), np.array(g.n)
