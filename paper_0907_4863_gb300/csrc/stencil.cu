@@ -587,6 +587,7 @@ StencilCfg stencil_autotune(const StencilDev<T>& S0, cudaStream_t s, double* bes
   b.alloc(n, s);
   d.alloc(n, s);
   SAAMG_CUDA(cudaMemsetAsync(x.p, 0, n * sizeof(T), s));
+  SAAMG_CUDA(cudaMemsetAsync(y.p, 0, n * sizeof(T), s));  // the pass adds to it
   SAAMG_CUDA(cudaMemsetAsync(b.p, 0, n * sizeof(T), s));
   SAAMG_CUDA(cudaMemsetAsync(d.p, 0, n * sizeof(T), s));
   cudaEvent_t e[4];

@@ -113,3 +113,36 @@ def test_the_default_is_restored_by_its_own_shape(S):
         S.set_stencil_config(op, prec, None)
         assert S.stencil_config(op, prec) == default
     op.free()
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "fp32"])
+def test_autotuner_reads_only_what_it_has_set(S, prec):
+    """Device memory that arrives full of NaN: the vectors of the timed pass hold none at the end."""
+    import numpy as np
+    import torch
+    w = I.pipe_workload(40, I.LINEAR)
+    op = S.build_operator(S.make_domain(w.domain), S.make_grid(w.grid), w.mode)
+    n = S.operator_size(op)[0]
+    live, nans = {}, []
+
+    def alloc(nbytes, stream, ctx):
+        t = torch.full((int(nbytes),), 0xFF, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        live[t.data_ptr()] = t
+        return t.data_ptr()
+
+    def free(ptr, stream, ctx):
+        torch.cuda.synchronize()
+        v = live.pop(ptr).cpu().numpy().view(np.float32 if prec else np.float64)
+        nans.append(int(np.isnan(v[:n]).sum()))
+
+    hooks = (S.ALLOC_FN(alloc), S.FREE_FN(free))
+    S._all_hooks.append(hooks)
+    S._hooks = None
+    assert S.lib().saamg_set_allocator(hooks[0], hooks[1], None) == S.OK
+    try:
+        S.autotune_stencil(op, prec)
+    finally:
+        S.use_torch_allocator()
+    assert not live and nans == [0, 0, 0, 0]
+    op.free()
