@@ -113,6 +113,28 @@ def test_gather_bitwise(S, g):
         assert not np.any(np.signbit(a) & (a == 0.0))  # a sum from +0 never ends at -0
 
 
+@pytest.mark.parametrize("special", [-0.0, 5e-324, -1e-310, 2.2250738585072014e-308, 1e-305, 1e300,
+                                     -1.7976931348623157e308, np.inf, np.nan], ids=str)
+@pytest.mark.parametrize("g", GRIDS[:2], ids=lambda g: "x".join(map(str, g.n)))
+def test_gather_special_fields(S, g, special):
+    """Field values whose products with the weights the integer multiplication hands back, or rounds
+    at an end of the exponent range, in every component."""
+    import torch
+    rng = np.random.default_rng(9)
+    e = [rng.standard_normal(g.nbox) for _ in range(3)]
+    for c in e:
+        c[rng.integers(0, 6, g.nbox) == 0] = special
+    lo, h, n = np.array(g.origin), np.array(g.h), np.array(g.n)
+    inner = rng.uniform(lo, lo + (n - 1) * h, size=(4096, 3)).T
+    x, y, z = (np.concatenate(p) for p in zip(inner, edge_particles(g, rng)))
+    with np.errstate(all="ignore"):
+        ref = O.gather_cic(g, e, x, y, z)
+    out = [torch.empty(len(x), dtype=torch.float64, device="cuda") for _ in range(3)]
+    S.gather_cic(S.make_grid(g), *[dev(c) for c in e], dev(x), dev(y), dev(z), *out)
+    for a, b in zip(out, ref):
+        assert np.array_equal(a.cpu().numpy(), b, equal_nan=True)
+
+
 @pytest.mark.parametrize("scale", [1.0, 1e-280, 1e-320, 1e250])
 @pytest.mark.parametrize("g", GRIDS, ids=lambda g: "x".join(map(str, g.n)))
 def test_deposit_edges(S, g, scale):
