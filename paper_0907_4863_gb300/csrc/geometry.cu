@@ -120,7 +120,7 @@ __device__ void neighbour_rows(const GeomParams& g, const LineInfo* lines, int L
 
 // --- kernels ---------------------------------------------------------------
 
-// Thread per x-line: first/last inside node and count; flags a non-contiguous line.  The line
+// G lanes per x-line (a power of two, uniform): first/last inside node and count; flags a non-contiguous line.  The line
 // meets the cross-section F = (x - cx)^2 / (a sigma)^2 + (y - cy)^2 / (b sigma)^2 - 1 < 0 (Gamma_1,
 // Sec. 4.1; Omega_h of Sec. 2 holds the lattice nodes of Omega plus the Robin planes, Dirichlet end
 // planes carry known zeros) in |x - cx| < w with w = a sigma sqrt(1 - v^2); nodes two or more
@@ -128,25 +128,31 @@ __device__ void neighbour_rows(const GeomParams& g, const LineInfo* lines, int L
 // there far above its rounding error), so only the five nodes around either end are tested
 // exactly; a line whose ends do not look as expected (an end at the box face, a short interval, or
 // any surprise) is scanned node by node.  Bound by FP64 issue, where an instruction costs the same
-// for one line as for 32: a warp per line took 256 us at 256^3, this 27.
-__global__ void __launch_bounds__(128) classify_lines_k(GeomParams g, int nlines, LineInfo* lines,
-                                                        int* count, int* err) {
-  const int L = blockIdx.x * blockDim.x + threadIdx.x;
-  if (L >= nlines) return;
+// for one line as for 32: a warp per line took 256 us at 256^3, a lane per line 27.  Few lines are
+// bound by the chain of tests instead, and share it (900 x 24 x 24 nodes, the wall outside the box:
+// the whole build took 958 us with a lane per line and takes 418).
+__global__ void __launch_bounds__(128) classify_lines_k(GeomParams g, int nlines, int G,
+                                                        LineInfo* lines, int* count, int* err) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int L = t / G, gl = t & (G - 1);
+  const bool on = L < nlines;  // whole groups; the warp's other lanes take part in the shuffles
   const int j = L % g.ny, k = L / g.ny;
   int first = INT_MAX, last = -1, cnt = 0;
-  int a = 0, b = -1;  // nodes to test one by one
-  if (!(g.zbc == SAAMG_Z_DIRICHLET && (k == 0 || k == g.nz - 1))) {  // else known zeros
-    // the inside test on the line's nodes; v, a sigma and v^2 are the line's
+  int a = 0, b = -1;         // nodes to test one by one
+  int lo = 0, hi = -1;       // ends to test (hi >= lo)
+  double vv = 0.0, as = 1.0;
+  auto inside = [&](int i) {
+    const double u = (node_coord(g.o[0], i, g.h[0]) - g.cx) / as;
+    return (u * u + vv) - 1.0 < 0.0;
+  };
+  if (on && !(g.zbc == SAAMG_Z_DIRICHLET && (k == 0 || k == g.nz - 1))) {  // else known zeros
+    // v, a sigma and v^2 are the line's
     const double y = node_coord(g.o[1], j, g.h[1]);
     const double z = node_coord(g.o[2], k, g.h[2]);
     const double sg = taper_sigma(g, z);
     const double v = (y - g.cy) / (g.b * sg);
-    const double vv = v * v, as = g.a * sg;
-    auto inside = [&](int i) {
-      const double u = (node_coord(g.o[0], i, g.h[0]) - g.cx) / as;
-      return (u * u + vv) - 1.0 < 0.0;
-    };
+    vv = v * v;
+    as = g.a * sg;
     b = g.nx - 1;
     if (vv >= 1.0) {
       b = -1;  // u*u + v*v >= 1 for every node: F >= 0
@@ -157,39 +163,48 @@ __global__ void __launch_bounds__(128) classify_lines_k(GeomParams g, int nlines
       if (A > B) {
         b = -1;  // the interval holds no node, nor any within two spacings
       } else if (B - A >= 16.0) {
-        const int lo = (int)A, hi = (int)B;
-        // the five nodes at each end: outside ... inside at the low end, inside ... outside at
-        // the high end, with one change each
-        unsigned mlo = 0, mhi = 0;
-#pragma unroll 1
-        for (int q = 0; q < 5; ++q) {
-          mlo |= (unsigned)inside(lo + q) << q;
-          mhi |= (unsigned)inside(hi - 4 + q) << q;
-        }
-        // low end: bit 0 clear and the set bits contiguous up to bit 4; high end: bit 4 clear
-        // and the set bits contiguous from bit 0
-        const bool lo_ok = mlo != 0 && (mlo & 1u) == 0 && ((mlo | (mlo - 1u)) & 0x1fu) == 0x1fu &&
-                           __popc(mlo) == 5 - (__ffs(mlo) - 1);
-        const bool hi_ok = mhi != 0 && (mhi & 0x10u) == 0 && (mhi & (mhi + 1u)) == 0;
-        if (lo_ok && hi_ok) {
-          first = lo + __ffs(mlo) - 1;
-          last = hi - 4 + (31 - __clz(mhi));
-          cnt = last - first + 1;
-          b = -1;
-        }
+        lo = (int)A;
+        hi = (int)B;
       } else {
         a = (int)A;
         b = (int)B;
       }
     }
+  }
+  // the five nodes at each end, bits 0-4 and 5-9: outside ... inside at the low end, inside ...
+  // outside at the high end, with one change each
+  unsigned m = 0;
+  if (hi >= lo)
 #pragma unroll 1
-    for (int i = a; i <= b; ++i)
+    for (int q = gl; q < 10; q += G) m |= (unsigned)inside(q < 5 ? lo + q : hi - 9 + q) << q;
+  for (int o = G >> 1; o > 0; o >>= 1) m |= __shfl_xor_sync(0xffffffffu, m, o);
+  const unsigned mlo = m & 0x1fu, mhi = m >> 5;
+  // low end: bit 0 clear and the set bits contiguous up to bit 4; high end: bit 4 clear
+  // and the set bits contiguous from bit 0
+  const bool lo_ok = mlo != 0 && (mlo & 1u) == 0 && ((mlo | (mlo - 1u)) & 0x1fu) == 0x1fu &&
+                     __popc(mlo) == 5 - (__ffs(mlo) - 1);
+  const bool hi_ok = mhi != 0 && (mhi & 0x10u) == 0 && (mhi & (mhi + 1u)) == 0;
+  if (lo_ok && hi_ok) {
+    first = lo + __ffs(mlo) - 1;
+    last = hi - 4 + (31 - __clz(mhi));
+    cnt = last - first + 1;
+  } else {
+#pragma unroll 1
+    for (int i = a + gl; i <= b; i += G)
       if (inside(i)) {
         if (first == INT_MAX) first = i;
         last = i;
         ++cnt;
       }
   }
+  const bool ends = lo_ok && hi_ok;  // the same in the group's lanes
+  for (int o = G >> 1; o > 0; o >>= 1) {
+    first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
+    last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+    const int c = __shfl_xor_sync(0xffffffffu, cnt, o);
+    cnt += ends ? 0 : c;
+  }
+  if (!on || gl != 0) return;
   LineInfo l;
   l.lo = cnt ? first : 0;
   l.hi = cnt ? last : -1;
@@ -692,7 +707,10 @@ void build_operator_data(const GeomParams& g, cudaStream_t s, OperatorData& op) 
   chstart.alloc(nlines, s);
   err.alloc(1, s);
   fill_int(err.p, 0, 1, s);
-  classify_lines_k<<<(nlines + 127) / 128, 128, 0, s>>>(g, nlines, op.lines.p, count.p, err.p);
+  // lanes per line: as many as keep the launch below the threads that a lane per line has at 256^3
+  int G = 1;
+  while (G < 32 && 2LL * G * nlines <= 65536) G <<= 1;
+  classify_lines_k<<<(nlines * G + 127) / 128, 128, 0, s>>>(g, nlines, G, op.lines.p, count.p, err.p);
   SAAMG_LAUNCH();
   int herr = 0;
   d2h_sync(&herr, err.p, sizeof(int), s);

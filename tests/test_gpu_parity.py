@@ -321,3 +321,23 @@ def test_mis2_aggregate_large_graph(S, deg, loops):
     assert nagg == nagg_ref
     assert np.array_equal(root.cpu().numpy(), root_ref)
     assert np.array_equal(agg.cpu().numpy(), agg_ref)
+
+
+# lines of the box: 32, 16, 8, 4, 2 lanes and one lane per line; short and long lines
+LINE_GRIDS = [(300, 24, 24), (5, 3, 7), (70, 64, 50), (45, 100, 60), (40, 128, 100), (33, 200, 130),
+              (24, 260, 256)]
+LINE_WALLS = {"pipe": I.Domain(0.45, 0.30), "clipped": I.Domain(0.9, 0.45, cx=0.2),
+              "whole_box": I.Domain(5.0, 5.0), "taper": I.Domain(0.5, 0.45, taper=0.4),
+              "on_nodes": I.Domain(0.5 - 0.5 / 40, 0.5, zbc=I.Z_DIRICHLET)}
+
+
+@pytest.mark.parametrize("wall", LINE_WALLS)
+@pytest.mark.parametrize("n", LINE_GRIDS, ids=lambda n: "x".join(map(str, n)))
+def test_unknowns_of_lines(S, n, wall):
+    """The inside test by every number of lanes per line, the wall across, at and beyond the box."""
+    w = I.Workload(wall, I.cell_centred_grid(*n), LINE_WALLS[wall], I.LINEAR)
+    o = oracle_operator(w)
+    g = gpu_op(S, w)
+    assert g.size() == (o.n, o.nnz)
+    assert np.array_equal(S.operator_copy(g)["node_of_row"], o.node_of_row)
+    g.free()
