@@ -117,6 +117,14 @@ __device__ __forceinline__ unsigned long long wmul(unsigned long long a, unsigne
   return __umul64hi(a, w);
 }
 
+// The warp's sum modulo 2^64: pieces of 27 bits, of which 32 add up below 2^32.
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x7ffffffu);
+  const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 27) & 0x7ffffffu);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 54));
+  return lo + ((unsigned long long)mid << 27) + ((unsigned long long)hi << 54);
+}
+
 // A particle adds round(2^S (q / V) wx wy wz) to each of its eight nodes.  The weights are
 // 64-bit fixed-point fractions and the products integer multiplications: |q / V| 2^S < 2^61, so
 // a product's three truncations are off by less than 3/8 of the fixed-point unit, where the
@@ -169,6 +177,30 @@ __global__ void __launch_bounds__(256) cic_deposit_k(Lattice g, int np,
   const bool inner = ci >= 0 && cj >= 0 && ck >= 0 && ci + 1 < g.nx && cj + 1 < g.ny &&
                      ck + 1 < g.nz;
   const long long v0 = ci + (long long)g.nx * (cj + (long long)g.ny * ck);
+  auto weight = [&](int a, int b, int c) {  // what node (a, b, c) of the cell takes
+    const unsigned long long r = wmul(wmul(mx[a], wy[b]), wz[c]);
+    const unsigned long long w = sh < 64 ? (r >> sh) + ((r & half) != 0) : (r >> 63);
+    return neg ? 0ull - w : w;
+  };
+  // 32 particles of one cell: their sum per node, one atomic each (an inner cell's index is below
+  // 4.0e9, the most nodes a grid may have).  Additions to the same address are served one after the
+  // other: 10^6 particles in one cell took 926 us without this (841 with the FP64 weights), now 90
+  if (__activemask() == 0xffffffffu) {
+    const unsigned lane = threadIdx.x & 31;
+    int same;
+    __match_all_sync(0xffffffffu, inner ? (unsigned)v0 : ~lane, &same);
+    if (same) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned long long w = weight(k & 1, (k >> 1) & 1, k >> 2);
+        const unsigned long long sum = warp_sum64(w);
+        if (lane == k && sum)
+          atomicAdd(&acc[v0 + (k & 1) + (long long)g.nx * (((k >> 1) & 1) + (long long)g.ny * (k >> 2))],
+                    sum);
+      }
+      return;
+    }
+  }
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
@@ -178,9 +210,8 @@ __global__ void __launch_bounds__(256) cic_deposit_k(Lattice g, int np,
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
         if (!inner && !(line && ci + a >= 0 && ci + a < g.nx)) continue;
-        const unsigned long long r = wmul(wmul(mx[a], wy[b]), wz[c]);
-        const unsigned long long w = sh < 64 ? (r >> sh) + ((r & half) != 0) : (r >> 63);
-        if (w) atomicAdd(&acc[v + a], neg ? 0ull - w : w);
+        const unsigned long long w = weight(a, b, c);
+        if (w) atomicAdd(&acc[v + a], w);
       }
     }
 }

@@ -157,6 +157,33 @@ def test_deposit_edges(S, g, scale):
     assert np.all(np.abs(got - ref) <= tol)
 
 
+@pytest.mark.parametrize("count", [32, 33, 96, 1000])
+@pytest.mark.parametrize("scale", [1.0, 1e-300, 1e200])
+def test_deposit_of_one_cell(S, scale, count):
+    """Particles that share a cell, warp by warp, and the same ones in turn with those of other
+    cells (a corner cell of the box, one across its face): the sums are of integers, so the bits
+    do not depend on the order."""
+    import torch
+    g = I.Grid((40, 9, 11), (0.3, 0.125, 1e-3), (-3.0, 2.0, 100.0))
+    rng = np.random.default_rng(count)
+    lo, h = np.array(g.origin), np.array(g.h)
+    cells = np.array([[17, 4, 6], [38, 7, 9], [0, 0, 0], [39, 3, 3]])
+    pts = lo + (cells[:, None, :] + rng.uniform(0, 1, (4, count, 3))) * h   # cell by cell
+    q = rng.uniform(-1.0, 1.0, (4, count)) * scale
+    sums = []
+    for order in (lambda a: a, lambda a: np.swapaxes(a, 0, 1)):
+        p, c = order(pts).reshape(-1, 3), order(q).reshape(-1)
+        rho = torch.full((g.nbox,), 7.0, dtype=torch.float64, device="cuda")
+        S.deposit_cic(S.make_grid(g), *[dev(p[:, d]) for d in range(3)], dev(c), rho)
+        sums.append(rho.cpu().numpy())
+    assert np.array_equal(sums[0].view(np.int64), sums[1].view(np.int64))
+    x, y, z = (np.ascontiguousarray(pts.reshape(-1, 3)[:, d]) for d in range(3))
+    ref = O.deposit_cic(g, x, y, z, q.reshape(-1))
+    bound = O.deposit_cic(g, x, y, z, np.abs(q.reshape(-1)))
+    total = np.sum(np.abs(q) / ((g.h[0] * g.h[1]) * g.h[2]))
+    assert np.all(np.abs(sums[0] - ref) <= q.size * 2.0 ** -60 * total + 2.0 ** -50 * bound)
+
+
 def test_deposit_single_charges_to_the_unit(S):
     """One particle: every node within one fixed-point unit (2^-60 of the density) of the exact
     product, which integers of any size give."""
