@@ -98,7 +98,7 @@ __device__ __forceinline__ double gj_forward(double x, int t, const GjPanel& pn,
 }
 
 // Factors the panel of columns k0 .. k0 + bw - 1 after applying the pending panel (pend = 0: none)
-// to them.  A step's chain -- the next column's update and pivot search, the exchange of the
+// to them (pstep: the rows' steps before it, NULL for none).  A step's chain -- the next column's update and pivot search, the exchange of the
 // blocks' candidates through distributed shared memory, one division -- is what bounds the kernel:
 // the candidate's own row is brought up to date by one instruction per panel column, and the rest
 // of the panel is updated while the cluster barrier is on its way.
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kGjThreads)
   const int G = kGjThreads / rp, gi = tid & (rp - 1), gg = tid / rp;
   // the pivot step of every own row so far sits behind the panel
   int* own = reinterpret_cast<int*>(pan + (size_t)B * rpb);
-  for (int i = tid; i < rows; i += kGjThreads) own[i] = pstep[i0 + i];
+  for (int i = tid; i < rows; i += kGjThreads) own[i] = pstep ? pstep[i0 + i] : -1;
   if (pend > 0) {
     const double* src = reinterpret_cast<const double*>(ppn);
     double* dst = reinterpret_cast<double*>(&pn);
@@ -544,21 +544,23 @@ void coarse_gs_setup(const DevCsr& A, const double* invd, const unsigned* ids, i
 
 // A^-1 by Gauss-Jordan elimination of the column-major n x n work array w (overwritten),
 // written by rows to inv; synchronises to read the zero-pivot flag
-static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_t s) {
+static void gauss_jordan_inverse(int n, const Buf<double>& w, double* inv, cudaStream_t s) {
   constexpr int B = kGjB;
-  Buf<int> prow, step[2], err;
-  Buf<double> w2, c[2];
-  Buf<GjPanel> pn[2];
-  prow.alloc(n, s);
-  err.alloc(2, s);  // zero pivot, last panel that has begun
-  w2.alloc((size_t)n * n, s);
-  for (int q = 0; q < 2; ++q) {
-    step[q].alloc(n, s);
-    c[q].alloc((size_t)B * n, s);
-    pn[q].alloc(1, s);
-  }
-  fill_int(err.p, 0, 2, s);
-  fill_int(step[1].p, -1, n, s);  // read by panel 0: no row is pivoted
+  // one array for everything: panels, multipliers, the second matrix, then the integers (an array
+  // for each took a call at n <= 3 from 49 to 55 us)
+  constexpr size_t kPanel = sizeof(GjPanel) / sizeof(double);
+  static_assert(sizeof(GjPanel) == kPanel * sizeof(double), "panels lie among doubles");
+  const size_t nn = (size_t)n * n, nb = (size_t)B * n;
+  Buf<double> work;
+  work.alloc(2 * (kPanel + nb) + nn + (3 * (size_t)n + 3) / 2, s);
+  GjPanel* const pn[2] = {reinterpret_cast<GjPanel*>(work.p),
+                          reinterpret_cast<GjPanel*>(work.p + kPanel)};
+  double* const c[2] = {work.p + 2 * kPanel, work.p + 2 * kPanel + nb};
+  double *src = w.p, *dst = work.p + 2 * (kPanel + nb);
+  int* const err = reinterpret_cast<int*>(dst + nn);  // zero pivot, last panel that has begun
+  int* const prow = err + 2;
+  int* const step[2] = {prow + n, prow + 2 * (size_t)n};
+  SAAMG_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), s));
   const int rpb = (n + kGjCluster - 1) / kGjCluster;
   SAAMG_CUDA(cudaFuncSetAttribute(gj_panel_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kGjPanelSmem));
@@ -602,10 +604,10 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
     attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    SAAMG_CUDA(cudaLaunchKernelEx(&cfg, gj_panel_k, n, q * B, rpb, (const double*)w.p,
-                                  q > 0 ? B : 0, (const GjPanel*)pn[pq].p, (const double*)c[pq].p,
-                                  pn[q & 1].p, c[q & 1].p, (const int*)step[pq].p, step[q & 1].p,
-                                  prow.p, err.p, q, err.p + 1));
+    SAAMG_CUDA(cudaLaunchKernelEx(&cfg, gj_panel_k, n, q * B, rpb, (const double*)src,
+                                  q > 0 ? B : 0, (const GjPanel*)pn[pq], (const double*)c[pq],
+                                  pn[q & 1], c[q & 1], (const int*)(q > 0 ? step[pq] : nullptr),
+                                  step[q & 1], prow, err, q, err + 1));
     SAAMG_LAUNCH();
   };
   panel(0);
@@ -613,22 +615,22 @@ static void gauss_jordan_inverse(int n, Buf<double>& w, double* inv, cudaStream_
     const bool beside = q + 1 < panels;
     if (beside) panel(q + 1);
     auto args = [&](auto&& launch) {
-      launch(n, q * B, cpb, rpt, (const GjPanel*)pn[q & 1].p, (const double*)c[q & 1].p,
-             (const int*)step[q & 1].p, (const double*)w.p, w2.p, beside ? q + 1 : 0,
-             (const int*)(err.p + 1));
+      launch(n, q * B, cpb, rpt, (const GjPanel*)pn[q & 1], (const double*)c[q & 1],
+             (const int*)step[q & 1], (const double*)src, dst, beside ? q + 1 : 0,
+             (const int*)(err + 1));
     };
     args([&](auto... a) {
       if (beside) launch_pdl(gj_update_k, ugrid, kGjUpdThreads, kGjUpdSmem, s, a...);
       else gj_update_k<<<ugrid, kGjUpdThreads, kGjUpdSmem, s>>>(a...);
     });
     SAAMG_LAUNCH();
-    w.swap(w2);
+    std::swap(src, dst);
   }
   const dim3 tiles((n + 31) / 32, (n + 31) / 32);
-  gj_gather_k<<<tiles, 256, 0, s>>>(n, w.p, step[(panels - 1) & 1].p, prow.p, inv);
+  gj_gather_k<<<tiles, 256, 0, s>>>(n, src, step[(panels - 1) & 1], prow, inv);
   SAAMG_LAUNCH();
   int herr = 0;
-  d2h_sync(&herr, err.p, sizeof(int), s);
+  d2h_sync(&herr, err, sizeof(int), s);
   if (herr) fail(SAAMG_NUMERICAL, "zero pivot in the coarse factorisation");
 }
 
