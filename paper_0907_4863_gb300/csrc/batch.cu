@@ -1332,18 +1332,6 @@ long long batch_engine_kernels(const BatchEngine* e) {
   return k;
 }
 
-long long batch_engine_bytes(const BatchEngine* e) {
-  long long b = 0;
-  for (const auto& L : e->lanes) b += L->tasks.bytes();
-  for (const auto& w : e->work) {
-    b += w->bhat.bytes() + w->xhat.bytes() + w->r.bytes() + w->z.bytes() + w->p.bytes() +
-         w->q.bytes() + w->z32.bytes() + w->r32.bytes();
-    for (auto& v : w->fx0) b += v.bytes() * 5;
-    for (auto& v : w->dx0) b += v.bytes() * 5;
-  }
-  return b;
-}
-
 void batch_engine_free(BatchEngine* e) { delete e; }
 
 }  // namespace saamg

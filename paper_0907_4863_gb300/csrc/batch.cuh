@@ -56,7 +56,6 @@ void batch_engine_launch(BatchEngine* e, cudaStream_t s);
 const PcgCtl* batch_engine_results(const BatchEngine* e);
 // Kernels the last run executed.
 long long batch_engine_kernels(const BatchEngine* e);
-long long batch_engine_bytes(const BatchEngine* e);
 void batch_engine_free(BatchEngine* e);
 
 }  // namespace saamg

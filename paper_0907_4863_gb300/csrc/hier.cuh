@@ -68,7 +68,6 @@ struct saamg_hierarchy {
   saamg::Buf<double> part0, part1, part2;
   saamg::Buf<saamg::PcgCtl> ctl;
   saamg::HostScratch host;
-  saamg::Buf<double> scratch;
   long long bytes = 0;
   // identity for cached batch graphs: a new value at creation and whenever the V-cycle
   // changes (a cached graph never outlives the kernels and pointers it was captured with)
