@@ -343,7 +343,8 @@ def run_ours(args):
     if rank == 0:
         if not args.no_cpu_baseline:
             out["cpu_baseline"] = cpu_baseline(args.n)
-        print(json.dumps(out), flush=True)
+        print(json.dumps(out), file=sys.stderr, flush=True)  # every leg in full
+        print(json.dumps(headline(out)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
@@ -935,6 +936,35 @@ def solo_solve_ms(S, torch, geoms, params):
         h.free()
         op.free()
     return out
+
+
+# Longest entry of the result line, in characters: whoever keeps the last few kilobytes of the output
+# keeps the whole line (with every leg in it, it is 22 kB).
+LINE_ENTRY = 700
+
+
+def shortened(v, limit):
+    """v, or of a longer dict its plain members, its short dicts and the rates and latencies of the
+    others."""
+    if len(json.dumps(v)) <= limit or not isinstance(v, dict):
+        return v
+    keep = {}
+    for k, x in v.items():
+        if isinstance(x, dict) and len(json.dumps(x)) > limit // 4:
+            x = {q: x[q] for q in ("solves_per_s", "p50_ms", "p99_ms") if q in x}
+        if not isinstance(x, list) and x != {}:
+            keep[k] = x
+    return keep
+
+
+def headline(out):
+    """The result line: the entries of `out`, the long ones shortened and named (they are on stderr, in
+    the full report)."""
+    line = {k: shortened(v, LINE_ENTRY) for k, v in out.items()}
+    long = [k for k, v in out.items() if line[k] != v]
+    if long:
+        line["in_full_on_stderr"] = long
+    return line
 
 
 # ---------------------------------------------------------------------------

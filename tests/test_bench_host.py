@@ -125,3 +125,27 @@ def test_captured_traffic_is_attached_to_the_256_cube_classes(bench):
             assert bench.roofline(name, rec, prec, n=256)["traffic"] is None
     assert bench.roofline("stencil_resid", rec, 0, n=256)["traffic"] is None
     assert bench.roofline("stencil_smooth", rec, 1, n=512)["traffic"] is None
+
+
+def test_the_result_line_is_short_and_holds_the_contract(bench):
+    """Legs of a few kilobytes each: the line keeps what identifies the run and its numbers, below
+    the 8 kB that a log's tail holds at least, and names what it leaves to the full report."""
+    import json
+    contract = {k: 1.0 for k in (
+        "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+        "scaling", "vs_baseline", "dtype", "data", "iters", "gpu_launches")}
+    contract["config"] = {"workload": "x" * 300, "grid": [256, 256, 256]}
+    contract["roofline"] = {"kernel": "k" * 20, **{f"f{i}": 1.0 / 3.0 for i in range(12)}}
+    contract["clocks"] = {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []}
+    contract["e2e"] = {"value": 1.0, "unit": "solves/s", "h2d_bytes_per_step": 1,
+                       "d2h_bytes_per_step": 1}
+    table = {f"number{j}": j / 7.0 for j in range(60)}
+    legs = {f"leg{i}": {"ms": 1.0, "classes": table, "list": list(range(300)), "hbm": {"frac": 0.5},
+                        "served": {**table, "p99_ms": 3.0}} for i in range(12)}
+    out = {**contract, **legs, "small_leg": {"ms": 1.0}}
+    line = bench.headline(out)
+    assert {k: line[k] for k in contract} == contract and line["small_leg"] == {"ms": 1.0}
+    assert sorted(line["in_full_on_stderr"]) == sorted(legs)
+    assert line["leg3"] == {"ms": 1.0, "hbm": {"frac": 0.5}, "served": {"p99_ms": 3.0}}
+    assert len(json.dumps(line)) < 8000 < len(json.dumps(out))
+    assert bench.headline(contract) == contract
