@@ -28,12 +28,12 @@ RTOL = 1e-8
 METRIC = "solves/s to rel-residual 1e-8 at 256^3 (mixed/batched vs FP64 GPU); HBM GB/s; p99"
 UNIT = "solves/s"
 PREC = {"fp64": 0, "fp32": 1, "bf16": 2}
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the FP64 level-0 Chebyshev step
-# on the 256^3 elliptic pipe, from its ncu capture; None for other kernels or sizes, and to be
-# reset whenever that kernel changes
-# (class, precision, n) -> DRAM bytes per launch (ncu, dram__bytes_read + dram__bytes_write); the
-# BF16 mode's level-0 passes are the FP32 kernels
+# (class, precision, n) -> DRAM bytes per launch of a level-0 pass on the elliptic pipe (ncu,
+# dram__bytes_read + dram__bytes_write; stencil_pair: the mean of its two passes); the BF16 mode's
+# level-0 passes are the FP32 kernels.  To be captured again whenever the kernel changes.
 TRAFFIC_BYTES = {("stencil_smooth", 0, 256): 364.0e6,
+                 ("stencil_pair", 0, 256): 220.9e6,
+                 ("stencil_pair", 1, 256): 64.3e6, ("stencil_pair", 2, 256): 64.3e6,
                  ("stencil_smooth", 1, 256): 125.1e6, ("stencil_smooth", 2, 256): 125.1e6,
                  ("stencil_resid", 1, 256): 82.5e6, ("stencil_resid", 2, 256): 82.5e6,
                  ("prolong0", 1, 256): 81.3e6, ("prolong0", 2, 256): 81.3e6}

@@ -156,7 +156,8 @@ void csr_apply(int mode, int n, const int* rowptr, const int* col, const TM* val
   // Lanes per row: FP64 shuffle-adds cost as much as the row's multiply-adds on this part, so
   // double vectors use few lanes (FP32 can afford wider groups for better coalescing) -- but
   // a small level (few rows, long rows: the deep levels of the hierarchy) needs wider groups
-  // to fill the GPU at all: enough lanes for ~150 k threads, never more than the row length.
+  // to fill the GPU at all: enough lanes for 150 k (FP32: 40 k) threads, never more than the row
+  // length.
   const int g = csr_plan(mode, n, avg_nnz, sizeof(TV) == 8);
   if (g == 0) {
     const long long need = ((long long)n + 255) / 256;

@@ -124,9 +124,9 @@ enum StencilMode {
 //   x1 = x + g r, r1 = r - g A r, x2 = x1 + c1 g r + c2 r1 = x + k0 r - k1 A r,
 //   k0 = g + c1 g + c2, k1 = c2 g;   d = x2 - x1.
 // From x = 0 that is one pass over b instead of two (7 FP64 operations a row instead of 11, 16 bytes
-// instead of 64), after the prolongation the residual and one pass (15 instead of 19 operations, 48
+// instead of 64), after the prolongation the residual and one pass (14 instead of 19 operations, 48
 // bytes instead of 72).  Measured at 256^3 in FP64: 43 + 148 us from zero and 134 + 148 after the
-// prolongation became 117 (the mean of the pair passes) and 107 + 117.
+// prolongation became 110 (the mean of the pair passes) and 107 + 110.
 template <class T>
 struct SmoothPair {
   T k0, k1, g;
