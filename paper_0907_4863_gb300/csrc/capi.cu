@@ -438,7 +438,7 @@ static void setup_levels(const saamg_operator* op, const saamg_params& prm, cuda
     if (coarsen) {
       // a smoothed level >= 1 large enough for SELL gets its SELL copy now (it is not the
       // coarsest), so that in the FP64 V-cycle the power iteration runs on it too
-      if (l >= 1 && L.n >= kSellMinRows && L.As.n == 0)
+      if (l >= 1 && L.n >= sell_min_rows(!mixed(h)) && L.As.n == 0)
         build_level_sell(h, L, s, prev ? prev->lev[l].get() : nullptr);
       const StencilDev<double> S0 = od.view<double>();
       cudaEvent_t fork;
@@ -580,7 +580,7 @@ static void setup_levels(const saamg_operator* op, const saamg_params& prm, cuda
     const bool bf16 = prm.precision == SAAMG_PREC_FP32_BF16;
     // SELL for the large smoothed levels (built before their spectral bound); a small level
     // runs on CSR with wide row groups
-    if (q >= 1 && q < nl - 1 && L.n >= kSellMinRows) {
+    if (q >= 1 && q < nl - 1 && L.n >= sell_min_rows(!mixed(h))) {
       if (L.As.n == 0)
         build_level_sell(h, L, s,
                          prev && q < (int)prev->lev.size() ? prev->lev[q].get() : nullptr);

@@ -67,3 +67,27 @@ def test_reuse_rejects_a_different_pattern(S):
     with pytest.raises(S.SaamgError) as e:
         S.setup_reuse(_op(S, w2), h)
     assert e.value.status == S.EINVAL
+
+
+def test_reuse_across_precisions_where_one_stores_sell(S):
+    """A level of 63,182 rows: SELL in FP64, CSR in the mixed modes, where the smoother's shuffles cost
+    nothing; a hierarchy rebuilt on the other's aggregates gives the bits of a fresh one."""
+    import torch
+    w = I.pipe_workload(118, I.LINEAR)
+    op = S.build_operator(S.make_domain(w.domain), S.make_grid(w.grid), w.mode)
+    rho = I.gaussian_bunch_torch(w.grid, w.centre, w.sigma, 5)
+    prm = [S.params_default(max_coarse=1000, precision=p) for p in (0, 1, 2)]
+    fresh = [S.setup(op, p) for p in prm]
+    ref = []
+    for h, sell in zip(fresh, (2, 0, 0)):
+        info = h.info()
+        assert info["n"][1] == 63182 and info["sell_index_bytes"][1] == sell
+        ref.append(torch.zeros_like(rho))
+        S.solve(h, rho, ref[-1])
+    for p, prev in ((0, 1), (1, 0), (2, 0), (1, 2)):
+        h = S.setup_reuse(op, fresh[prev], prm[p])
+        assert h.info()["sell_index_bytes"][1] == (2 if p == 0 else 0)
+        phi = torch.zeros_like(rho)
+        assert S.solve(h, rho, phi)["converged"] == 1
+        assert torch.equal(phi, ref[p])
+        h.free()
