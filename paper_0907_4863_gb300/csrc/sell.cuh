@@ -22,12 +22,13 @@ constexpr int kSellWindow = 512;
 // Smallest level stored as SELL: below it one thread per row leaves most of the GPU idle and
 // the CSR kernel with wide row groups is faster.  In FP64 SELL gains from fewer rows on, because a row
 // group's shuffle additions cost FP64 time.  Whole solves, time with CSR over time with SELL on
-// level 1, pipes and cylinders of 96^3 to 136^3 and 80-160 a side:
-//   rows  34 k   44 k   51 k   54 k   63 k   65 k   74 k   81 k   94 k
-//   FP64  0.995  0.99   1.02   1.03   1.055  1.05   1.07   1.085  1.09
-//   FP32  0.95   0.955  0.97   0.975  0.98   0.98   1.01   1.01   1.02
-//   BF16  0.94   0.96   0.965  0.98   0.985  1.005  1.00   1.03   1.005
-inline int sell_min_rows(bool f64) { return f64 ? 60000 : 74000; }
+// level 1, pipes and cylinders of 80 to 160 nodes a side (mixed modes: medians over ten placements
+// of the arrays, which alone move such a solve by 2 %):
+//   rows  34 k   44 k   54 k   63 k   65 k   74 k   81 k   94 k
+//   FP64  0.995  0.99   1.03   1.055  1.05   1.07   1.085  1.09
+//   FP32  0.95   0.955  0.975  0.99   0.985  1.005  1.025  1.02
+//   BF16  0.94   0.96   0.975  0.97   0.985  1.005  1.02   1.005
+inline int sell_min_rows(bool f64) { return f64 ? 60000 : 70000; }
 
 struct DevSell {
   int n = 0, m = 0, nslices = 0;
