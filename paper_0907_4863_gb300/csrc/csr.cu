@@ -132,6 +132,10 @@ int csr_plan(int mode, int n, double avg_nnz, bool dbl) {
   if ((mode == CSR_ADD || mode == CSR_SPMV) && avg_nnz <= kShortWin && n >= 100000) return 0;
   int g = dbl ? (avg_nnz <= 10.0 ? 2 : (avg_nnz <= 48.0 ? 4 : 8))
               : (avg_nnz <= 6.0 ? 2 : (avg_nnz <= 20.0 ? 4 : (avg_nnz <= 64.0 ? 8 : 16)));
+  // lanes for that many threads.  FP32: the same lanes serve a solve alone and in a batch (the bits
+  // agree), where fewer are better: 32 solves on 32-64 nodes a side in one call take 6.04 ms with 40 k
+  // threads, 6.36 with 70 k and 6.67 with 150 k; alone, a solve on 64 a side 1.02, 1.00 and 1.01 ms,
+  // one on 56 a side 1.00, 0.96 and 0.965 (medians over ten placements of the arrays)
   int gpar = 1;
   while (gpar < 32 && (long long)n * gpar < (dbl ? 150000 : 40000)) gpar <<= 1;
   // no more lanes than the row length needs: one entry per lane in FP32; in FP64, where a
